@@ -703,6 +703,7 @@ bool fill_params(const int grid[3], const lbm_eos *eos, double G, const lbm_rate
   P.n = (int)n;
   P.q = op == LBM_OP_NONORTHOGONAL_D3Q15 ? 15 : 19;
   P.G = eos->kind == LBM_EOS_NONE ? 0.0 : G;
+  P.half_force = -0.5 * P.G / (P.q == 15 ? 24.0 : 12.0);
   P.rho_ref = 0.0;
   P.s_e = rates->s_e;
   P.s_nu = rates->s_nu;

@@ -23,6 +23,7 @@ struct KParams {
   int n;             // nx * ny * nz (< 2^31)
   int q;             // lattice: 19 (D3Q19, both operators) or 15 (D3Q15 non-orthogonal)
   double G;          // interaction strength, Eq. 15
+  double half_force; // -G/2 times the diagonal (D3Q15: corner) weight of Eq. 15, 1/12 (1/24)
   double rho_ref;    // reference density of the deviation storage
   // relaxation rates (see lbm_rates in lbm.h)
   double s_e, s_nu, s_q, s_pi, s_eps, s_m;

@@ -46,14 +46,6 @@ template <> struct Lat<19> {
   template <typename T> static __device__ __forceinline__ void gradient(const T *p, T &Sx, T &Sy, T &Sz) {
     psi_gradient<T>(p, Sx, Sy, Sz);
   }
-  static __device__ __forceinline__ void e(int a, int &x, int &y, int &z) {
-    const int ex[19] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0};
-    const int ey[19] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1};
-    const int ez[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
-    x = ex[a];
-    y = ey[a];
-    z = ez[a];
-  }
 };
 template <> struct Lat<15> {
   static __device__ __forceinline__ int src(const Nbhd &nb, int a) { return q15::src(nb, a); }
@@ -67,11 +59,6 @@ template <> struct Lat<15> {
   }
   template <typename T> static __device__ __forceinline__ void gradient(const T *p, T &Sx, T &Sy, T &Sz) {
     q15::psi_gradient<T>(p, Sx, Sy, Sz);
-  }
-  static __device__ __forceinline__ void e(int a, int &x, int &y, int &z) {
-    x = q15::ex(a);
-    y = q15::ey(a);
-    z = q15::ez(a);
   }
 };
 
@@ -160,35 +147,136 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
 
 // ------------------------------------------------------------------ observables
 // rho and u (Eq. 6) of the current state, in FP64 whatever the storage.
+//
+// GB300 issues two FP64 instructions per SM and clock, so these kernels are
+// bound by the FP64 unit unless almost all of the work runs elsewhere: with
+// every conversion, sum and division in FP64 (149 instructions per node) the
+// fields of a 256^3 FP32 box took 5.11 ms, against 0.28 ms for their bytes;
+// they take 0.88 ms now (FP16 storage: 5.89 -> 1.7, FP64 at 128^3: 0.50 -> 0.29).
+// Both forms below share the pair differences among the sums and take one
+// reciprocal for the three velocities.  The FP32-arithmetic forms also take
+// their sums on the FP32 units, exactly (split_scale), which leaves 29 FP64
+// instructions per node.
+
+// sum_a v_a e_a (axis entries times axw) and, with R, r = sum_a v_a.
+template <int Q, bool R, typename T>
+__device__ __forceinline__ void moment_sums(const T v[Q], T axw, T &r, T &x, T &y, T &z) {
+  const T d12 = v[1] - v[2], d34 = v[3] - v[4], d56 = v[5] - v[6];
+  const T d78 = v[7] - v[8], d910 = v[9] - v[10], d1112 = v[11] - v[12], d1314 = v[13] - v[14];
+  if (R) {
+    r = v[0] + ((v[1] + v[2]) + (v[3] + v[4]) + (v[5] + v[6])) +
+        ((v[7] + v[8]) + (v[9] + v[10]) + (v[11] + v[12]) + (v[13] + v[14]));
+    if constexpr (Q == 19) r = r + ((v[15] + v[16]) + (v[17] + v[18]));
+  }
+  if constexpr (Q == 19) {
+    const T d1516 = v[15] - v[16], d1718 = v[17] - v[18];
+    x = axw * d12 + ((d78 + d910) + (d1112 + d1314));
+    y = axw * d34 + ((d78 - d910) + (d1516 + d1718));
+    z = axw * d56 + ((d1112 - d1314) + (d1516 - d1718));
+  } else {
+    const T ab = d78 + d910, cd = d1112 - d1314;
+    x = axw * d12 + (ab + cd);
+    y = axw * d34 + (ab - cd);
+    z = axw * d56 + ((d78 - d910) + (d1112 + d1314));
+  }
+}
+
+// Constants that split FP32 values v (all |v| < 2^(e+1), e the exponent of the
+// largest) into v = h + l + t: adding and subtracting 1.5 * 2^(e+5) leaves h, a
+// multiple of 2^(e-18); the same with 1.5 * 2^(e-15) splits the (exact)
+// remainder into l, a multiple of 2^(e-38), and t, |t| <= 2^(e-39).  Sums of up
+// to 32 times the largest value are then exact in FP32 over the h and over the
+// l (24 bits hold them), and the FP32 sum of the t is good to 2^(e-54) at
+// worst: closer than an FP64 sum of the v, whose every addition may round at
+// 2^(e-53) and above.  (The error-free extraction of Rump, Ogita and Oishi's
+// accurate summation.)  Not ok: infinities, NaN and ranges where the constants
+// or the t would leave the normal numbers; those nodes sum in FP64.
+struct SplitScale {
+  float m1, m2;
+  bool ok;
+};
+__device__ __forceinline__ SplitScale split_scale(unsigned max_abs_bits) {
+  constexpr unsigned lo = (127u - 60u) << 23, hi = (127u + 60u) << 23;
+  const unsigned ef = max_abs_bits & 0x7f800000u;
+  SplitScale s;
+  s.ok = max_abs_bits == 0u || (ef >= lo && ef <= hi);
+  const unsigned e = s.ok ? max(ef, lo) : lo;
+  s.m1 = __uint_as_float((e + (5u << 23)) | 0x400000u);
+  s.m2 = __uint_as_float((e - (15u << 23)) | 0x400000u);
+  return s;
+}
+
+// moment_sums of FP32 values through that split, assembled in FP64.
+template <int Q, bool R>
+__device__ __forceinline__ void moment_sums_split(float v[Q], float axw, const SplitScale &s, double &r, double &x,
+                                                  double &y, double &z) {
+  float h[3][4];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    float w[Q];
+    const float m = k == 0 ? s.m1 : s.m2;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      w[a] = k == 2 ? v[a] : __fsub_rn(__fadd_rn(v[a], m), m);
+      v[a] = __fsub_rn(v[a], w[a]);
+    }
+    moment_sums<Q, R, float>(w, axw, h[k][0], h[k][1], h[k][2], h[k][3]);
+  }
+  auto join = [&](int q) { return widen_f32(h[0][q]) + (widen_f32(h[1][q]) + widen_f32(h[2][q])); };
+  if (R) r = join(0);
+  x = join(1);
+  y = join(2);
+  z = join(3);
+}
+
+template <int Q>
+__device__ __forceinline__ unsigned max_abs_bits(const float v[Q]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int a = 0; a < Q; ++a) m = max(m, __float_as_uint(v[a]) & 0x7fffffffu);
+  return m;
+}
+
 template <int PREC, int Q>
 __device__ __forceinline__ void node_moments(const typename Types<PREC>::S *__restrict__ g,
                                              const typename Types<PREC>::Psi *__restrict__ psi,
                                              const KParams &P, const Nbhd &nb, double &rho,
                                              double &rux, double &ruy, double &ruz) {
   using S = typename Types<PREC>::S;
-  double f[Q];
-  pull_q<Q, S, double>(g, P.n, nb, f);
-  double drho = 0, jx = 0, jy = 0, jz = 0;
+  using T = typename Types<PREC>::T;
+  // the sums of Eq. 15 with the diagonal (corner) weight taken out: axis entries weigh 2 (8) times as much
+  constexpr float axw = Q == 19 ? 2.0f : 8.0f;
+  T f[Q], p[Q];
+  pull_q<Q, S, T>(g, P.n, nb, f);
 #pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    int ex, ey, ez;
-    Lat<Q>::e(a, ex, ey, ez);
-    drho += f[a];
-    jx += ex * f[a];
-    jy += ey * f[a];
-    jz += ez * f[a];
+  for (int a = 1; a < Q; ++a) p[a] = psi[Lat<Q>::dst(nb, a)];
+  p[0] = psi[nb.self];
+  double drho, jx, jy, jz, sx, sy, sz, p0, unused;
+  if constexpr (PREC == kF64) {
+    moment_sums<Q, true, double>(f, 1.0, drho, jx, jy, jz);
+    moment_sums<Q, false, double>(p, (double)axw, unused, sx, sy, sz);
+    p0 = p[0];
+  } else {
+    const SplitScale cf = split_scale(max_abs_bits<Q>(f)), cp = split_scale(max_abs_bits<Q>(p));
+    p0 = widen_f32(p[0]);
+    if (cf.ok && cp.ok) {
+      moment_sums_split<Q, true>(f, 1.0f, cf, drho, jx, jy, jz);
+      moment_sums_split<Q, false>(p, axw, cp, unused, sx, sy, sz);
+    } else {
+      double d[Q];
+#pragma unroll
+      for (int a = 0; a < Q; ++a) d[a] = (double)f[a];
+      moment_sums<Q, true, double>(d, 1.0, drho, jx, jy, jz);
+#pragma unroll
+      for (int a = 0; a < Q; ++a) d[a] = (double)p[a];
+      moment_sums<Q, false, double>(d, (double)axw, unused, sx, sy, sz);
+    }
   }
-  double p[Q];
-#pragma unroll
-  for (int a = 1; a < Q; ++a) p[a] = (double)psi[Lat<Q>::dst(nb, a)];
-  p[0] = (double)psi[nb.self];
-  double Sx, Sy, Sz;
-  Lat<Q>::gradient(p, Sx, Sy, Sz);
-  const double k = -P.G * p[0];
+  const double k = P.half_force * p0;  // half the force: F / 2 = k (sx, sy, sz)
   rho = P.rho_ref + drho;
-  rux = jx + 0.5 * k * Sx;
-  ruy = jy + 0.5 * k * Sy;
-  ruz = jz + 0.5 * k * Sz;
+  rux = jx + k * sx;
+  ruy = jy + k * sy;
+  ruz = jz + k * sz;
 }
 
 template <int PREC, int Q>
@@ -202,14 +290,16 @@ __global__ void moments_kernel(const typename Types<PREC>::S *__restrict__ g,
   node_moments<PREC, Q>(g, psi, P, nb, rho, rux, ruy, ruz);
   if (rho_out) rho_out[nb.self] = rho;
   if (u_out) {
-    u_out[nb.self] = rux / rho;
-    u_out[(size_t)P.n + nb.self] = ruy / rho;
-    u_out[2 * (size_t)P.n + nb.self] = ruz / rho;
+    const double inv = 1.0 / rho;
+    u_out[nb.self] = rux * inv;
+    u_out[(size_t)P.n + nb.self] = ruy * inv;
+    u_out[2 * (size_t)P.n + nb.self] = ruz * inv;
   }
 }
 
-// Block-partial FP64 sums of (rho, rho u) and max |u|, grid-stride over nodes,
-// then one block folds the partials in a fixed order (deterministic).
+// Block-partial FP64 sums of (rho, rho u) and max |u|^2, grid-stride over
+// nodes, then one block folds the partials in a fixed order (deterministic)
+// and takes the root.
 template <int PREC, int Q>
 __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<PREC>::S *__restrict__ g,
                                                            const typename Types<PREC>::Psi *__restrict__ psi,
@@ -224,8 +314,10 @@ __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<
     acc[1] += rux;
     acc[2] += ruy;
     acc[3] += ruz;
-    const double u = sqrt(rux * rux + ruy * ruy + ruz * ruz) / rho;
-    acc[4] = (u > acc[4] || u != u) ? u : acc[4];
+    const double inv = 1.0 / rho;
+    double u2 = (rux * rux + ruy * ruy + ruz * ruz) * (inv * inv);
+    if (__double2hiint(rho) < 0) u2 = -u2;  // a negative density never holds the maximum
+    acc[4] = (u2 > acc[4] || u2 != u2) ? u2 : acc[4];
   }
   __shared__ double red[5][256];
 #pragma unroll
@@ -259,16 +351,16 @@ __global__ void __launch_bounds__(256) max_du_kernel(const typename Types<PREC>:
     const Nbhd nb(x, y, z, P);
     double rho, rux, ruy, ruz;
     node_moments<PREC, Q>(g, psi, P, nb, rho, rux, ruy, ruz);
-    const double u[3] = {rux / rho, ruy / rho, ruz / rho};
+    const double inv = 1.0 / rho;
+    const double u[3] = {rux * inv, ruy * inv, ruz * inv};
     double d2 = 0.0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const double d = u[k] - (double)u_prev[(size_t)k * P.n + i];
+      const double d = u[k] - widen_f32(u_prev[(size_t)k * P.n + i]);
       d2 += d * d;
-      u_prev[(size_t)k * P.n + i] = (float)u[k];
+      u_prev[(size_t)k * P.n + i] = narrow_f64(u[k]);
     }
-    const double d = sqrt(d2);
-    m = (d > m || d != d) ? d : m;
+    m = (d2 > m || d2 != d2) ? d2 : m;
   }
   __shared__ double red[256];
   red[threadIdx.x] = m;
@@ -280,19 +372,31 @@ __global__ void __launch_bounds__(256) max_du_kernel(const typename Types<PREC>:
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) atomicMax(out, (unsigned long long)__double_as_longlong(red[0]));
+  if (threadIdx.x == 0) atomicMax(out, (unsigned long long)__double_as_longlong(sqrt(red[0])));
 }
 
-__global__ void diag_final_kernel(const double *__restrict__ partials, int nblocks,
-                                  double *__restrict__ result) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// One block: each thread folds every 256th partial, then a tree.  (One thread
+// folding the 1024 partials in a row took 0.37 ms, most of a diag of a small box.)
+__global__ void __launch_bounds__(256) diag_final_kernel(const double *__restrict__ partials, int nblocks,
+                                                         double *__restrict__ result) {
+  __shared__ double red[5][256];
   double acc[5] = {0, 0, 0, 0, 0};
-  for (int b = 0; b < nblocks; ++b) {
+  for (int b = threadIdx.x; b < nblocks; b += 256) {
     for (int k = 0; k < 4; ++k) acc[k] += partials[b * 5 + k];
     const double u = partials[b * 5 + 4];
     acc[4] = (u > acc[4] || u != u) ? u : acc[4];
   }
-  for (int k = 0; k < 5; ++k) result[k] = acc[k];
+  for (int k = 0; k < 5; ++k) red[k][threadIdx.x] = acc[k];
+  __syncthreads();
+  for (int s = 128; s > 0; s >>= 1) {
+    if (threadIdx.x < s) {
+      for (int k = 0; k < 4; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + s];
+      const double a = red[4][threadIdx.x], b = red[4][threadIdx.x + s];
+      red[4][threadIdx.x] = (b > a || b != b) ? b : a;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < 5) result[threadIdx.x] = threadIdx.x == 4 ? sqrt(red[4][0]) : red[threadIdx.x][0];
 }
 
 // ------------------------------------------------------------------ initial state
@@ -488,7 +592,7 @@ cudaError_t launch_diag(const KParams &P, int precision, const void *g, const vo
                                  (const typename Types<PR>::S *)g, (const typename Types<PR>::Psi *)psi, P, partials)));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_final_kernel<<<1, 32, 0, L.stream>>>(partials, kReduceBlocks, result);
+  diag_final_kernel<<<1, 256, 0, L.stream>>>(partials, kReduceBlocks, result);
   return cudaGetLastError();
 }
 
