@@ -718,6 +718,7 @@ bool fill_params(const int grid[3], const lbm_eos *eos, double G, const lbm_rate
   P.RT = eos->R * eos->T;
   P.psi0 = eos->psi0;
   P.rho0 = eos->rho0;
+  P.exp_k = -eos->rho0 * 1.4426950408889634;
   P.b4 = 0.25 * eos->b;
   P.two_over_G = P.G != 0.0 ? 2.0 / P.G : 0.0;
   {

@@ -34,6 +34,7 @@ struct KParams {
   int eos;
   double a, b, RT;   // Carnahan-Starling (Eq. 58), RT = R * T
   double psi0, rho0; // exponential pseudopotential
+  double exp_k;      // -rho0 log2(e)
   double b4;         // b / 4
   double two_over_G; // 2 / G
   // (2/G) (RT num - (a rho + 1/3) den) = q0 + q1 rho + q2 rho^2 + q3 rho^3 + q4 rho^4,

@@ -138,3 +138,30 @@ def test_max_du_is_the_largest_change_of_u():
             assert abs(d - want) <= 1e-13 * want + 1e-16
         before = now
     b.close()
+
+
+@pytest.mark.parametrize("arith", ["f64", "f32x2"])
+@pytest.mark.parametrize("psi0, rho0", [(1.0, 1.0), (4.0, 0.3)])
+def test_exponential_psi_over_its_range(psi0, rho0, arith):
+    """u at rest is F / (2 rho), so it shows psi = psi0 exp(-rho0 / rho): densities from where psi leaves FP32's
+    normal range (the FP64 functions) through vapour and liquid to beyond."""
+    from paper_1805_08643_gb300.lbm import Lattice, Rates
+
+    grid, G = (36, 10, 9), -10.0 / 3.0
+    rng = np.random.default_rng(11)
+    field = rho0 * np.exp(rng.uniform(np.log(0.006), np.log(40.0), grid[::-1]))
+    lat = Lattice(grid, operator="nonorth", precision="f32", eos="exp", psi0=psi0, rho0=rho0, G=G, rates=Rates())
+    lat.set_eos_arith(arith)
+    lat.init_field(field, rho_ref=0.0)
+    rho, u = lat.moments()
+    assert lat.check() == 0
+    lat.close()
+    p = L.Params(grid=grid, eos="exp", psi0=psi0, rho0=rho0, G=G)
+    psi = L.pseudopotential(rho, p)
+    want = L.interaction_force(psi, G) / (2 * rho)
+    # psi sees rho after an FP32 sum (8 roundings) and is rounded itself: a relative error of 8 rho0 / rho + 1
+    # roundings, at the node and at its neighbours; below FP32's normal range the spacing is absolute
+    e = psi * (8 * rho0 / rho + 2) * 2.0 ** -24 + psi0 * 2.0 ** -140
+    near = sum(wf * L.shifted(psi, d) for wf, d in zip(L.W_FORCE, L.E))
+    tol = abs(G) * (e * near + psi * sum(wf * L.shifted(e, d) for wf, d in zip(L.W_FORCE, L.E))) / (2 * rho)
+    assert np.all(np.abs(u - want) <= tol + 1e-14 * np.abs(want))
