@@ -176,6 +176,18 @@ __device__ __forceinline__ float narrow_f64(double v) {
   return __uint_as_float(r);
 }
 
+// 1 / x in FP64: an FP32 reciprocal (error 2^-23) and one cubic Newton step,
+// r (1 + e + e^2) with e = 1 - x r, three FP64 instructions, wrong by 2^-69
+// before its last rounding; exponents FP32 cannot hold take the division.
+__device__ __forceinline__ double recip(double x) {
+  const unsigned e11 = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (e11 < 1023u - 120u || e11 > 1023u + 120u) return 1.0 / x;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(narrow_f64(x)));
+  const double r0 = widen_f32(r), e = fma(-x, r0, 1.0);
+  return fma(r0, fma(e, e, e), r0);
+}
+
 // psi0 exp(-rho0 / rho) rounded to FP32.  With CUDA's FP64 division and exp()
 // it took about 85 FP64 instructions a node (70 us per 80^3 work-list step, 45
 // with this one); this one takes 11, and everything that FP32 can carry without

@@ -129,6 +129,98 @@ inline void refresh_float_params(KParams &P) {
   }
 }
 
+// Coefficients of the collision (Eq. 4, 11, 13, 14, 16), one set per operator.
+// The relaxed moments enter the inverse transform with constant factors (1/4,
+// 1/6, 1/12, ...); with those multiplied into the rates on the host, a moment is
+// relaxed and scaled by the same instructions.  s is a rate, a = 1 - s, c = 1 - s/2.
+enum Coeff {
+  // shear rate: a/12, a/4, s/8, c/4, a/36 (D3Q15: s/16, c/8 and a/8 for the last three)
+  kN5 = 0, kN7, kNb1, kNb2, kON,
+  // odd moments
+  kQs,        // s_q                    (non-orthogonal and D3Q15)
+  kQa,        // a_q / 2; orthogonal: a_q / 40
+  kQb1, kQb2, // s_q / 12, c_q / 12; orthogonal over 60, D3Q15 over 24
+  // energy; non-orthogonal: moment 4 over 6; orthogonal: e over 2394
+  kE1, kE2, kE3, kE4, kE5,
+  // fourth-order moments over 4 (D3Q15: over 8); orthogonal: pi_xx over 72
+  kP1, kP2, kP3, kP4, kP5,
+  // orthogonal only: eps over 252, (1 - s_m) / 8
+  kO1, kO2, kO3, kO4, kO5, kO6, kOm,
+  kForce,  // F_i = force psi(x) S_i
+  kCoeffs
+};
+
+struct Coeffs64 {
+  double k[kCoeffs];
+};
+
+// force and sig: -G and the Eq. 16 coefficient (KParams::sigma_coef) for the
+// sums of Eq. 15 in units of the diagonal (corner) weight, 1/12 (1/24).
+inline Coeffs64 coeffs64(const KParams &P, int op) {
+  Coeffs64 c64;
+  double *k = c64.k;
+  const double se = P.s_e, sn = P.s_nu, sq = P.s_q, sp = P.s_pi, sx = P.s_eps, sm = P.s_m;
+  const double units = P.q == 15 ? 24.0 : 12.0, sig = P.sigma_coef / (units * units);
+  const double ce = 1 - 0.5 * se, cn = 1 - 0.5 * sn, cq = 1 - 0.5 * sq, cp = 1 - 0.5 * sp, cx = 1 - 0.5 * sx;
+  for (int i = 0; i < kCoeffs; ++i) k[i] = 0.0;
+  k[kForce] = -P.G / units;
+  k[kN5] = (1 - sn) / 12;
+  k[kN7] = (1 - sn) / 4;
+  k[kNb1] = sn / 8;
+  k[kNb2] = cn / 4;
+  k[kON] = (1 - sn) / 36;
+  k[kQs] = sq;
+  if (op == kOrth) {
+    k[kQa] = (1 - sq) / 40;
+    k[kQb1] = sq / 60;
+    k[kQb2] = cq / 60;
+    // e = 19 (A + 2 B) - 30 drho, A and B the axis and diagonal sums of f
+    k[kE1] = (1 - se) * 19 / 2394;
+    k[kE2] = (-30 * (1 - se) - 11 * se) / 2394;
+    k[kE3] = 19 * se / 2394;
+    k[kE4] = 38 * ce / 2394;
+    k[kE5] = 19 * ce * sig / 2394;
+    // eps = 12 drho - 16 A - 11 B
+    k[kO1] = -16 * (1 - sx) / 252;
+    k[kO2] = -11 * (1 - sx) / 252;
+    k[kO3] = (12 * (1 - sx) + 3 * sx) / 252;
+    k[kO4] = -5.5 * sx / 252;
+    k[kO5] = -11 * cx / 252;
+    k[kO6] = -16 * cx * sig / 252;
+    // pi_xx over 72 (a, s/2, c) and pi_ww over 24 (three times those)
+    k[kP1] = (1 - sp) / 72;
+    k[kP2] = 0.5 * sp / 72;
+    k[kP3] = cp / 72;
+    k[kOm] = (1 - sm) / 8;
+  } else {
+    k[kQa] = (1 - sq) / 2;
+    k[kQb1] = sq / 12;
+    k[kQb2] = cq / 12;
+    k[kE1] = (1 - se) / 6;
+    k[kE2] = se / 6;
+    k[kE4] = 2 * ce / 6;
+    k[kE5] = ce * sig / 6;
+    if (op == kNonOrth) {
+      k[kP1] = (1 - sp) / 4;
+      k[kP2] = sp / 36;  // drho
+      k[kP3] = sp / 24;  // usq
+      k[kP4] = cp / 6;   // F . u
+      k[kP5] = sp / 12;  // rho u_i^2
+    } else {             // D3Q15: corner moments over 8
+      k[kON] = (1 - sn) / 8;
+      k[kNb1] = sn / 16;
+      k[kNb2] = cn / 8;
+      k[kQb1] = sq / 24;
+      k[kQb2] = cq / 24;
+      k[kP1] = (1 - sp) / 8;
+      k[kP2] = sp / 72;
+      k[kP3] = sp / 144;
+      k[kP4] = cp / 18;
+    }
+  }
+  return c64;
+}
+
 // x-y tile shapes of the single-pass kernel.
 enum Tile { kTile32x4 = 0, kTile32x8 = 1, kTile64x4 = 2 };
 

@@ -13,6 +13,7 @@
 
 #include <algorithm>
 
+#include "lbm_collide64.cuh"
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
 #include "lbm_q15.cuh"
@@ -115,7 +116,7 @@ template <int PREC, int OP, bool SIGMA, int Q>
 __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::S *__restrict__ g_in,
                                                     typename Types<PREC>::S *__restrict__ g_out,
                                                     const typename Types<PREC>::Psi *__restrict__ psi,
-                                                    const KParams P) {
+                                                    const KParams P, const Coeffs64 C) {
   using S = typename Types<PREC>::S;
   using T = typename Types<PREC>::T;
   int x, y, z;
@@ -129,6 +130,18 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
   for (int a = 1; a < Q; ++a) p[a] = (T)__ldg(psi + Lat<Q>::dst(nb, a));
   p[0] = (T)__ldg(psi + nb.self);
   T Sx, Sy, Sz;
+  auto out = [&](int a, T v) { Lat<Q>::store(g_out + (size_t)a * P.n + nb.self, a, v); };
+  if constexpr (PREC == kF64) {
+    psi_sums64<Q>(p, Sx, Sy, Sz);
+    const double k = C.k[kForce] * p[0], S2 = SIGMA ? Sx * Sx + Sy * Sy + Sz * Sz : 0.0;
+    if constexpr (Q == 15)
+      collide_q15_64(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
+    else if constexpr (OP == kNonOrth)
+      collide_nonorth64(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
+    else
+      collide_orth64(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
+    return;
+  }
   Lat<Q>::gradient(p, Sx, Sy, Sz);
   const T k = -Phys<T>::G(P) * p[0];
   const T Fx = k * Sx, Fy = k * Sy, Fz = k * Sz;
@@ -142,7 +155,7 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
   else
     collide_orth<T>(f, Phys<T>::rho_ref(P), Fx, Fy, Fz, dS4, r);
 #pragma unroll
-  for (int a = 0; a < Q; ++a) Lat<Q>::store(g_out + (size_t)a * P.n + nb.self, a, f[a]);
+  for (int a = 0; a < Q; ++a) out(a, f[a]);
 }
 
 // ------------------------------------------------------------------ observables
@@ -158,6 +171,9 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
 // their sums on the FP32 units, exactly (split_scale), which leaves 29 FP64
 // instructions per node.
 
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+
 // sum_a v_a e_a (axis entries times axw) and, with R, r = sum_a v_a.
 template <int Q, bool R, typename T>
 __device__ __forceinline__ void moment_sums(const T v[Q], T axw, T &r, T &x, T &y, T &z) {
@@ -170,14 +186,14 @@ __device__ __forceinline__ void moment_sums(const T v[Q], T axw, T &r, T &x, T &
   }
   if constexpr (Q == 19) {
     const T d1516 = v[15] - v[16], d1718 = v[17] - v[18];
-    x = axw * d12 + ((d78 + d910) + (d1112 + d1314));
-    y = axw * d34 + ((d78 - d910) + (d1516 + d1718));
-    z = axw * d56 + ((d1112 - d1314) + (d1516 - d1718));
+    x = mad(axw, d12, (d78 + d910) + (d1112 + d1314));
+    y = mad(axw, d34, (d78 - d910) + (d1516 + d1718));
+    z = mad(axw, d56, (d1112 - d1314) + (d1516 - d1718));
   } else {
     const T ab = d78 + d910, cd = d1112 - d1314;
-    x = axw * d12 + (ab + cd);
-    y = axw * d34 + (ab - cd);
-    z = axw * d56 + ((d78 - d910) + (d1112 + d1314));
+    x = mad(axw, d12, ab + cd);
+    y = mad(axw, d34, ab - cd);
+    z = mad(axw, d56, (d78 - d910) + (d1112 + d1314));
   }
 }
 
@@ -290,7 +306,7 @@ __global__ void moments_kernel(const typename Types<PREC>::S *__restrict__ g,
   node_moments<PREC, Q>(g, psi, P, nb, rho, rux, ruy, ruz);
   if (rho_out) rho_out[nb.self] = rho;
   if (u_out) {
-    const double inv = 1.0 / rho;
+    const double inv = recip(rho);
     u_out[nb.self] = rux * inv;
     u_out[(size_t)P.n + nb.self] = ruy * inv;
     u_out[2 * (size_t)P.n + nb.self] = ruz * inv;
@@ -314,7 +330,7 @@ __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<
     acc[1] += rux;
     acc[2] += ruy;
     acc[3] += ruz;
-    const double inv = 1.0 / rho;
+    const double inv = recip(rho);
     double u2 = (rux * rux + ruy * ruy + ruz * ruz) * (inv * inv);
     if (__double2hiint(rho) < 0) u2 = -u2;  // a negative density never holds the maximum
     acc[4] = (u2 > acc[4] || u2 != u2) ? u2 : acc[4];
@@ -351,7 +367,7 @@ __global__ void __launch_bounds__(256) max_du_kernel(const typename Types<PREC>:
     const Nbhd nb(x, y, z, P);
     double rho, rux, ruy, ruz;
     node_moments<PREC, Q>(g, psi, P, nb, rho, rux, ruy, ruz);
-    const double inv = 1.0 / rho;
+    const double inv = recip(rho);
     const double u[3] = {rux * inv, ruy * inv, ruz * inv};
     double d2 = 0.0;
 #pragma unroll
@@ -506,11 +522,17 @@ cudaError_t fused_dispatch(const KParams &P, bool sigma, const void *g_in, void 
                            const Launch &L) {
   using S = typename Types<PREC>::S;
   using Psi = typename Types<PREC>::Psi;
-  const dim3 grid = node_grid(P, L), block(L.bx, L.by);
+  // FP64: blocks of one warp.  Every warp holds the SM's FP64 unit for the same time, so the last round is
+  // shortest when warps are dealt out singly: 32^3 steps 28.7 -> 26.7 us (orthogonal; blocks of four warps
+  // leave 8 on some SMs, single ones 7), no difference from 64^3 on.
+  Launch Lf = L;
+  if (PREC == kF64) Lf.by = 1;
+  const dim3 grid = node_grid(P, Lf), block(Lf.bx, Lf.by);
+  const Coeffs64 C = coeffs64(P, Q == 15 ? kNonOrthQ15 : OP);
   if (sigma)
-    fused_kernel<PREC, OP, true, Q><<<grid, block, 0, L.stream>>>((const S *)g_in, (S *)g_out, (const Psi *)psi, P);
+    fused_kernel<PREC, OP, true, Q><<<grid, block, 0, L.stream>>>((const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
   else
-    fused_kernel<PREC, OP, false, Q><<<grid, block, 0, L.stream>>>((const S *)g_in, (S *)g_out, (const Psi *)psi, P);
+    fused_kernel<PREC, OP, false, Q><<<grid, block, 0, L.stream>>>((const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
   return cudaGetLastError();
 }
 

@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/lbm.h"
+#include "lbm_collide64.cuh"
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
 
@@ -44,7 +45,7 @@ __global__ void static_psi_kernel(const double *__restrict__ f, double *__restri
 // Collide f_a(x, t) and push f*_a(x, t) to f_out at x + e_a (Eq. 5).
 template <int OP, bool SIGMA>
 __global__ void static_fused_kernel(const double *__restrict__ f_in, double *__restrict__ f_out,
-                                    const double *__restrict__ psi, const KParams P) {
+                                    const double *__restrict__ psi, const KParams P, const lbm::Coeffs64 C) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
   if (x >= P.nx || y >= P.ny) return;
   const Nbhd nb(x, y, z, P);
@@ -55,16 +56,13 @@ __global__ void static_fused_kernel(const double *__restrict__ f_in, double *__r
   for (int a = 1; a < 19; ++a) p[a] = psi[nb.dst(a)];
   p[0] = psi[nb.self];
   double Sx, Sy, Sz;
-  lbm::psi_gradient<double>(p, Sx, Sy, Sz);
-  const double Fx = -P.G * p[0] * Sx, Fy = -P.G * p[0] * Sy, Fz = -P.G * p[0] * Sz;
-  const double dS4 = SIGMA ? P.sigma_coef * (Sx * Sx + Sy * Sy + Sz * Sz) : 0.0;
-  const lbm::Rates<double> r(P);
+  lbm::psi_sums64<19>(p, Sx, Sy, Sz);
+  const double k = C.k[lbm::kForce] * p[0], S2 = SIGMA ? Sx * Sx + Sy * Sy + Sz * Sz : 0.0;
+  auto out = [&](int a, double v) { f_out[(size_t)a * P.n + nb.dst(a)] = v; };
   if (OP == lbm::kNonOrth)
-    lbm::collide_nonorth<double>(f, 0.0, Fx, Fy, Fz, dS4, r);
+    lbm::collide_nonorth64(f, 0.0, k * Sx, k * Sy, k * Sz, S2, P, C, out);
   else
-    lbm::collide_orth<double>(f, 0.0, Fx, Fy, Fz, dS4, r);
-#pragma unroll
-  for (int a = 0; a < 19; ++a) f_out[(size_t)a * P.n + nb.dst(a)] = f[a];
+    lbm::collide_orth64(f, 0.0, k * Sx, k * Sy, k * Sz, S2, P, C, out);
 }
 
 // Device address of lbm_static_psi, looked up on the first call on each device
@@ -123,7 +121,8 @@ extern "C" lbm_status lbm_step_static(const lbm_ctx *ctx, const double *f_in, do
   }
   if (e != cudaSuccess) return LBM_ERR_CUDA;
   const double *psi_c = psi;
-  void *fused_args[] = {(void *)&f_in, (void *)&f_out, (void *)&psi_c, (void *)&P};
+  lbm::Coeffs64 C = lbm::coeffs64(P, op);
+  void *fused_args[] = {(void *)&f_in, (void *)&f_out, (void *)&psi_c, (void *)&P, (void *)&C};
   if (op == lbm::kNonOrth)
     e = sigma_on ? launch(static_fused_kernel<lbm::kNonOrth, true>, grid, block, stream, fused_args)
                  : launch(static_fused_kernel<lbm::kNonOrth, false>, grid, block, stream, fused_args);
