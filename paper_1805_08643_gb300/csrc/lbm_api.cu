@@ -168,7 +168,7 @@ void free_queue(lbm_ctx *c) {
 lbm_status ensure_queue(lbm_ctx *c) {
   if (c->q_mem) return LBM_OK;
   int grid = 0;
-  CK(lbm::queue_grid(c->precision, &grid), "work list occupancy");
+  CK(lbm::queue_grid(c->precision, c->P.q, &grid), "work list occupancy");
   std::vector<int4> items;
   if (!lbm::queue_items(c->P, grid, items)) return fail(c, LBM_ERR_ARG, "no valid work list for this box");
   const size_t ib = (items.size() * sizeof(int4) + 255) / 256 * 256;

@@ -82,14 +82,15 @@ __device__ __forceinline__ void gather_psi_pair15(const float *__restrict__ psi,
   row3(nb.rmp, unused, p[11], p[10]);
 }
 
-// Fused pass of one pair on D3Q15 (pull, force from the psi stencil, collision, store).
-template <typename S, bool SIGMA>
+// Fused pass of one pair on D3Q15 (pull, force from the psi stencil, collision,
+// store); FORCE_FIRST as in fused_pair_at.
+template <typename S, bool SIGMA, bool FORCE_FIRST = false>
 __device__ __forceinline__ void fused_pair15_at(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                 const float *__restrict__ psi, const KParams &P, int x, int y, int z) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
   V2 f[q15::kQ];
-  pull_pair15<S>(g_in, (unsigned)P.n, nb, px, f);
+  if (!FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.n, nb, px, f);
   V2 Fx, Fy, Fz, dS4;
   {
     V2 p[q15::kQ];
@@ -102,6 +103,7 @@ __device__ __forceinline__ void fused_pair15_at(const S *__restrict__ g_in, S *_
     Fy = kk * Sy;
     Fz = kk * Sz;
   }
+  if (FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.n, nb, px, f);
   q15::collide<V2>(f, V2((double)P.frho_ref), Fx, Fy, Fz, dS4, Rates<V2>(P));
 #pragma unroll
   for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st2(g_out + (size_t)a * P.n + nb.self, a, f[a]);

@@ -61,7 +61,15 @@ namespace {
 constexpr int TXP = 32;          // pair columns of a tile: 64 nodes
 constexpr int kRows = 4;         // rows of a tile (one warp each)
 constexpr int NTH = TXP * kRows;
-constexpr int kMinBlocks = 6;    // resident blocks per SM the register budget is set for
+// Resident blocks per SM the register budgets are set for.  The fused jobs wait
+// for memory most of the time, so a block more is worth more than the spills it
+// costs, up to a point; taking the force from psi before the populations are
+// pulled (FORCE_FIRST) is what lets a thread live on 72 registers.  256^3 FP32
+// steps, non-orthogonal / D3Q15, at 6, 7 and 8 blocks: 527 / 457, 515 / 444 and
+// 551 / 430 us (192^3: 250 / 229, 220 / 235 and 233 / 190).  Batches stay at 6
+// (848 against 842 us for 64 boxes at 7, with 180 bytes spilled).
+constexpr int kBatchBlocks = 6;
+__host__ __device__ constexpr int min_blocks(int q) { return q == 15 ? 8 : 7; }
 // The psi jobs convert to and from FP64 with the conversion instructions, not
 // the integer path of the psi pass kernel (the same results): this kernel is
 // not bound by the FP64 unit, and the integer work cost 1 % (FP32 storage) and
@@ -95,7 +103,7 @@ __device__ __forceinline__ int next_item(unsigned c, int nitems, unsigned &e) {
 // item: x = fused plane (or -1), y = its tile, z = psi plane (or -1), w = its tile.
 // Q: 19 (both operators) or 15 (the D3Q15 non-orthogonal variant).
 template <typename S, int OP, bool SIGMA, int EOS, bool DF, int Q>
-__global__ void __launch_bounds__(NTH, kMinBlocks)
+__global__ void __launch_bounds__(NTH, min_blocks(Q))
     queue_kernel(const S *__restrict__ g_in, S *__restrict__ g_out, const float *__restrict__ psi_in,
                  float *__restrict__ psi_out, const KParams P, const int4 *__restrict__ items, int nitems,
                  int *__restrict__ done, int stamp, unsigned *__restrict__ err) {
@@ -121,9 +129,9 @@ __global__ void __launch_bounds__(NTH, kMinBlocks)
       const int x = (t % G.ntx) * 2 * TXP + 2 * lane, y = (t / G.ntx) * kRows + row;
       if (x < P.nx && y < P.ny) {
         if constexpr (Q == 15)
-          fused_pair15_at<S, SIGMA>(g_in, g_out, psi_in, P, x, y, z);
+          fused_pair15_at<S, SIGMA, true>(g_in, g_out, psi_in, P, x, y, z);
         else
-          fused_pair_at<S, OP, SIGMA, false>(g_in, g_out, psi_in, P, x, y, z, Rates<V2>(P));
+          fused_pair_at<S, OP, SIGMA, true>(g_in, g_out, psi_in, P, x, y, z, Rates<V2>(P));
       }
       if (lane == 0 && row == 0) s_next[par] = next_item(claim - base, nitems, e);
       __syncthreads();
@@ -213,16 +221,17 @@ cudaError_t by_op(const KParams &P, int op, bool sigma, bool df, const void *g_i
 }
 
 // Resident blocks per SM of the kernels a context launches: the smallest over
-// the instantiations of the storage type, so that a cooperative launch of
-// that many blocks per SM fits whichever one runs.
+// the instantiations of the storage type and lattice, so that a cooperative
+// launch of that many blocks per SM fits whichever one runs.
 template <typename S>
-cudaError_t occupancy_of(int *per_sm) {
+cudaError_t occupancy_of(int q, int *per_sm) {
   using K = void (*)(const S *, S *, const float *, float *, const KParams, const int4 *, int, int *, int, unsigned *);
-  const K ks[] = {queue_kernel<S, kNonOrth, true, kEosCS, false, 19>, queue_kernel<S, kOrth, true, kEosCS, false, 19>,
-                  queue_kernel<S, kNonOrth, false, kEosCS, true, 19>, queue_kernel<S, kOrth, false, kEosExp, false, 19>,
-                  queue_kernel<S, kNonOrth, true, kEosCS, false, 15>, queue_kernel<S, kNonOrth, false, kEosExp, true, 15>};
+  const K k19[] = {queue_kernel<S, kNonOrth, true, kEosCS, false, 19>, queue_kernel<S, kOrth, true, kEosCS, false, 19>,
+                   queue_kernel<S, kNonOrth, false, kEosCS, true, 19>, queue_kernel<S, kOrth, false, kEosExp, false, 19>};
+  const K k15[] = {queue_kernel<S, kNonOrth, true, kEosCS, false, 15>, queue_kernel<S, kNonOrth, false, kEosExp, true, 15>};
   int m = 1 << 30;
-  for (K k : ks) {
+  for (int i = 0; i < (q == 15 ? 2 : 4); ++i) {
+    const K k = q == 15 ? k15[i] : k19[i];
     int v = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k, NTH, 0);
     if (e != cudaSuccess) return e;
@@ -283,7 +292,7 @@ __device__ __forceinline__ void prefetch_boxes(BatchBox *dst, const BatchBox *__
 }
 
 template <typename S, int EOS>
-__global__ void __launch_bounds__(NTH, kMinBlocks)
+__global__ void __launch_bounds__(NTH, kBatchBlocks)
     batch_queue_kernel(const BatchBox *__restrict__ boxes, const int4 *__restrict__ items, int nitems, int parity,
                        int *__restrict__ done, int ndone, unsigned *__restrict__ err) {
   __shared__ BatchBox bb[2][2];  // [item parity][fused job's box, psi job's box]
@@ -409,9 +418,9 @@ bool place_psi_jobs(std::vector<int4> &out, const std::vector<long long> &ready,
 
 bool queue_supported(const KParams &P, int precision) { return precision != kF64 && P.nx % 2 == 0; }
 
-cudaError_t queue_grid(int precision, int *grid) {
+cudaError_t queue_grid(int precision, int q, int *grid) {
   int per_sm = 0, dev = 0, sms = 0;
-  cudaError_t e = precision == kF32 ? occupancy_of<float>(&per_sm) : occupancy_of<__half>(&per_sm);
+  cudaError_t e = precision == kF32 ? occupancy_of<float>(q, &per_sm) : occupancy_of<__half>(q, &per_sm);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
