@@ -73,14 +73,15 @@ lbm_status cuda_fail(lbm_ctx *c, cudaError_t e, const char *where) {
     if (e_ != cudaSuccess) return cuda_fail(c, e_, where); \
   } while (0)
 
-// A population buffer holds Q N stored values, and at least 4N doubles: the
+// A population buffer holds Q N stored values (rows padded to an even length in
+// the FP32-arithmetic forms: KParams::px), and at least 4N doubles: the
 // spare one stages rho and u for lbm_moments (D3Q15 with FP16 storage is 30N bytes).
 size_t pop_bytes(const lbm_ctx *c) {
-  return std::max((size_t)c->P.q * c->P.n * lbm::storage_bytes(c->precision), (size_t)4 * c->P.n * sizeof(double));
+  return std::max((size_t)c->P.q * c->P.np * lbm::storage_bytes(c->precision), (size_t)4 * c->P.n * sizeof(double));
 }
-size_t psi_bytes(const lbm_ctx *c) { return 2 * (size_t)c->P.n * lbm::psi_elem_bytes(c->precision); }
+size_t psi_bytes(const lbm_ctx *c) { return 2 * (size_t)c->P.np * lbm::psi_elem_bytes(c->precision); }
 void *psi_at(lbm_ctx *c, int level) {
-  return (char *)c->psi + (size_t)level * c->P.n * lbm::psi_elem_bytes(c->precision);
+  return (char *)c->psi + (size_t)level * c->P.np * lbm::psi_elem_bytes(c->precision);
 }
 void *cur_psi(lbm_ctx *c) { return psi_at(c, c->pc); }
 
@@ -701,6 +702,8 @@ bool fill_params(const int grid[3], const lbm_eos *eos, double G, const lbm_rate
   P.ny = grid[1];
   P.nz = grid[2];
   P.n = (int)n;
+  P.px = stored_row(precision, grid);
+  P.np = (int)((long long)P.px * grid[1] * grid[2]);
   P.q = op == LBM_OP_NONORTHOGONAL_D3Q15 ? 15 : 19;
   P.G = eos->kind == LBM_EOS_NONE ? 0.0 : G;
   P.half_force = -0.5 * P.G / (P.q == 15 ? 24.0 : 12.0);

@@ -1,9 +1,9 @@
 // Batched boxes: many independent periodic boxes advanced together, the
-// launches of two steps captured in a CUDA graph.  Boxes with an even Nx step
-// on the work list (one cooperative launch) or on the two-pass pair kernels
-// (the fused pass as a flat grid per operator, then psi of the new level over
-// work items); boxes with an odd Nx on the one-node single pass, in the same
-// step graph.  Boxes can join and leave
+// launches of two steps captured in a CUDA graph.  Boxes step on the work list
+// (one cooperative launch) or on the two-pass pair kernels (the fused pass as a
+// flat grid per operator, then psi of the new level over work items); a box
+// whose odd-length rows cannot be padded (stored_row) on the one-node single
+// pass, in the same step graph.  Boxes can join and leave
 // between calls (continuous batching); each box's buffers come from the
 // stream-ordered allocator and count against the batch's HBM budget.
 #include <cuda_runtime.h>
@@ -64,7 +64,7 @@ struct lbm_batch {
   bool dirty = true;         // descriptors / items need uploading, graphs re-capturing
   bool pair = false;         // the captured step is the two-pass pair kernels
   bool wl = false;           // ... or the work-list single pass
-  bool odd = false;          // ... and the one-node single pass for the odd-Nx boxes
+  bool odd = false;          // ... and the one-node single pass for boxes with rows of odd length
   int *d_done = nullptr;     // its completion counters, cleared before every launch
   int *d_fmap = nullptr;     // two-pass step: the box of every block of the flat fused grids
   long long cap_fmap = 0;
@@ -96,10 +96,11 @@ lbm_status bfail(lbm_batch *b, lbm_status s, const std::string &m) {
                    std::string(where) + ": " + cudaGetErrorString(e_));                          \
   } while (0)
 
-size_t box_bytes(int precision, long long n) {
-  const size_t pop = (size_t)19 * n * lbm::storage_bytes(precision);
+// n nodes, np stored ones (KParams::np).
+size_t box_bytes(int precision, long long n, long long np) {
+  const size_t pop = (size_t)19 * np * lbm::storage_bytes(precision);
   auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-  return 2 * up(pop) + 2 * up((size_t)n * 4) + up((size_t)3 * n * 4);
+  return 2 * up(pop) + 2 * up((size_t)np * 4) + up((size_t)3 * n * 4);
 }
 
 // Ints after a work list's completion counters for the blocks' item-claim counter (at offset 16).
@@ -135,10 +136,10 @@ lbm_status rebuild(lbm_batch *b) {
     if (b->boxes[i].live && b->boxes[i].initialised) order.push_back({(long long)b->boxes[i].d.P.n, i});
   }
   std::sort(order.begin(), order.end(), [](auto &x, auto &y) { return x.first > y.first || (x.first == y.first && x.second < y.second); });
-  // boxes with an even Nx step on the two-node kernels (the work list, or the two-pass pair kernels);
-  // boxes with an odd Nx on the one-node single pass; one step graph runs both groups
+  // boxes whose stored rows have an even length (KParams::px) step on the two-node kernels (the work list, or
+  // the two-pass pair kernels); the others on the one-node single pass; one step graph runs both groups
   std::vector<std::pair<long long, int>> even, odd;
-  for (auto &o : order) (b->boxes[o.second].d.P.nx % 2 == 0 ? even : odd).push_back(o);
+  for (auto &o : order) (b->boxes[o.second].d.P.px % 2 == 0 ? even : odd).push_back(o);
   const bool wl = !even.empty() && b->tile == kTileWorkList;
   const int tile = b->tile == kTileWorkList ? lbm::kTile32x8 : b->tile;  // of the tile-shaped kernels
   std::vector<int4> items;
@@ -156,7 +157,7 @@ lbm_status rebuild(lbm_batch *b) {
     }
   };
   if (wl) {
-    // the work list over the even-Nx boxes in this order; each box's counters start at its qbase
+    // the work list over the even group in this order; each box's counters start at its qbase
     BCK(lbm::batch_queue_grid(b->precision, b->eos, &b->wl_grid), "work list occupancy");
     std::vector<const KParams *> ps;
     for (auto &o : even) ps.push_back(&b->boxes[o.second].d.P);
@@ -182,7 +183,7 @@ lbm_status rebuild(lbm_batch *b) {
         const unsigned zt = (unsigned)(side ? it.w : it.y);
         const long long z = zt & 0xffffu, t = zt >> 16;
         const long long T = lbm::batch_queue_tiles(P);
-        if (slot >= nb || !b->boxes[slot].live || P.nx % 2 != 0 || z >= P.nz || t >= T ||
+        if (slot >= nb || !b->boxes[slot].live || P.px % 2 != 0 || z >= P.nz || t >= T ||
             desc[slot].qbase + P.nz * T > nc)
           return bfail(b, LBM_ERR_ARG, "work list does not match the box table");
       }
@@ -248,13 +249,15 @@ lbm_status rebuild(lbm_batch *b) {
     if (b->pair) BCK(lbm::batch_pair_occupancy(b->precision, b->eos, tile, pair_per_sm), "pair kernel occupancy");
     const int per_sm = tile == lbm::kTile32x4 ? 4 : 2;
     const int n_odd = b->nitems - n_even;
+    bool padded = false;
+    for (auto &o : even) padded = padded || b->boxes[o.second].d.P.px != b->boxes[o.second].d.P.nx;
     const int grid_odd = std::min(b->grid_blocks * per_sm, std::max(n_odd, 1));
     auto step = [&](int parity) {
       cudaError_t e = cudaSuccess;
       if (wl) {
         e = cudaMemsetAsync(b->d_done, 0, sizeof(int) * (size_t)(b->ndone + kClaimInts), b->stream);
         if (e == cudaSuccess)
-          e = lbm::launch_batch_queue(b->precision, b->eos, b->d_boxes, b->d_items, n_even, parity, b->wl_grid,
+          e = lbm::launch_batch_queue(b->precision, b->eos, padded, b->d_boxes, b->d_items, n_even, parity, b->wl_grid,
                                       b->d_done, (int)b->ndone, b->d_err, b->stream);
       } else if (n_even) {
         e = lbm::launch_batch_pair(b->precision, b->eos, tile, b->d_boxes, b->d_items, n_even, b->d_fmap,
@@ -324,7 +327,8 @@ extern "C" {
 
 size_t lbm_batch_box_bytes(int precision, const int grid[3]) {
   if (!grid || grid[0] < 3 || grid[1] < 3 || grid[2] < 3) return 0;
-  return box_bytes(precision, (long long)grid[0] * grid[1] * grid[2]);
+  return box_bytes(precision, (long long)grid[0] * grid[1] * grid[2],
+                   (long long)lbm::stored_row(precision, grid) * grid[1] * grid[2]);
 }
 
 lbm_status lbm_batch_create(int precision, int eos_kind, size_t hbm_budget_bytes, void *cuda_stream,
@@ -370,12 +374,12 @@ lbm_status lbm_batch_add(lbm_batch *b, const int grid[3], const lbm_eos *eos, do
   KParams P;
   if (op == LBM_OP_NONORTHOGONAL_D3Q15) return bfail(b, LBM_ERR_ARG, "batches hold D3Q19 boxes");
   if (!lbm::fill_params(grid, eos, G, rates, op, b->precision, sigma, &P)) return bfail(b, LBM_ERR_ARG, "bad box");
-  const size_t bytes = box_bytes(b->precision, P.n);
+  const size_t bytes = box_bytes(b->precision, P.n, P.np);
   if (b->used + bytes > b->budget) return bfail(b, LBM_ERR_OOM, "HBM budget of the batch exceeded");
   HostBox h;
   BCK(cudaMallocAsync(&h.mem, bytes, b->stream), "box buffers");
-  const size_t pop = (((size_t)19 * P.n * lbm::storage_bytes(b->precision)) + 255) / 256 * 256;
-  const size_t ps = (((size_t)P.n * 4) + 255) / 256 * 256;
+  const size_t pop = (((size_t)19 * P.np * lbm::storage_bytes(b->precision)) + 255) / 256 * 256;
+  const size_t ps = (((size_t)P.np * 4) + 255) / 256 * 256;
   char *m = (char *)h.mem;
   h.live = true;
   h.precision = b->precision;

@@ -24,7 +24,9 @@ struct Nbhd {
   int r00, rm0, rp0, r0m, r0p, rmm, rpp, rmp, rpm;  // nx*(y' + ny*z')
   int self;
 
-  __device__ __forceinline__ Nbhd(int x_, int y, int z, const KParams &P) {
+  // pitch: the row length of the array the offsets are for, KParams::px (stored arrays) or nx (public ones)
+  __device__ __forceinline__ Nbhd(int x_, int y, int z, const KParams &P) : Nbhd(x_, y, z, P, P.px) {}
+  __device__ __forceinline__ Nbhd(int x_, int y, int z, const KParams &P, int pitch) {
     x_ = LBM_IDX(x_, P.nx);  // debug build: the node must lie in the box
     y = LBM_IDX(y, P.ny);
     z = LBM_IDX(z, P.nz);
@@ -33,7 +35,7 @@ struct Nbhd {
     xp = x_ == P.nx - 1 ? 0 : x_ + 1;
     const int ym = y == 0 ? P.ny - 1 : y - 1, yp = y == P.ny - 1 ? 0 : y + 1;
     const int zm = z == 0 ? P.nz - 1 : z - 1, zp = z == P.nz - 1 ? 0 : z + 1;
-    const int nx = P.nx, nxy = P.nx * P.ny;
+    const int nx = pitch, nxy = pitch * P.ny;
     const int z0 = z * nxy, zM = zm * nxy, zP = zp * nxy;
     r00 = y * nx + z0;  rm0 = ym * nx + z0;  rp0 = yp * nx + z0;
     r0m = y * nx + zM;  r0p = y * nx + zP;

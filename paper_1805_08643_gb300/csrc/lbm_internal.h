@@ -21,6 +21,13 @@ enum : unsigned { kErrEosDomain = 1u, kErrNonFinite = 2u, kErrTimeout = 4u };
 struct KParams {
   int nx, ny, nz;
   int n;             // nx * ny * nz (< 2^31)
+  // The stored arrays (populations, psi): px is the length of an x row in them,
+  // np = px * ny * nz the distance from one direction to the next.  px = nx but
+  // for an odd nx in the FP32-arithmetic forms, whose two-node kernels want rows
+  // that start on a pair: there px = nx + 1 and the last element of a row repeats
+  // its first (the periodic neighbour of node nx - 1), kept by whoever writes
+  // node 0.  Arrays of the public interface (rho, u, f) have rows of nx.
+  int px, np;
   int q;             // lattice: 19 (D3Q19, both operators) or 15 (D3Q15 non-orthogonal)
   double G;          // interaction strength, Eq. 15
   double half_force; // -G/2 times the diagonal (D3Q15: corner) weight of Eq. 15, 1/12 (1/24)
@@ -59,6 +66,13 @@ struct KParams {
   int spin_limit;
   int wait_bias;
 };
+
+// KParams::px of a box: rows of an odd nx get one element more where the
+// two-node kernels run, unless that leaves the index range (19 np < 2^32).
+inline int stored_row(int precision, const int grid[3]) {
+  const long long padded = (long long)(grid[0] + 1) * grid[1] * grid[2];
+  return precision != kF64 && grid[0] % 2 != 0 && 19 * padded < (1LL << 32) ? grid[0] + 1 : grid[0];
+}
 
 constexpr int kDefaultSpinLimit = 1 << 22;
 
@@ -331,7 +345,8 @@ int batch_tile_width(int nx);               // 64, 32 or 16: tiles of tw x (256 
 void batch_queue_geometry(BatchBox &d);     // sets d.tw and the geometry fields from d.P
 int batch_queue_tiles(const KParams &P);   // tile jobs per plane of a box in a batch work list
 cudaError_t batch_queue_grid(int precision, int eos, int *grid);
-cudaError_t launch_batch_queue(int precision, int eos, const BatchBox *boxes, const int4 *items, int nitems,
+// odd: some box has rows padded for an odd Nx.
+cudaError_t launch_batch_queue(int precision, int eos, bool odd, const BatchBox *boxes, const int4 *items, int nitems,
                                int parity, int grid, int *done, int ndone, unsigned *err, cudaStream_t s);
 
 // Debug build (-DLBM_BOUNDS_CHECK): OR of the bounds-error words of every

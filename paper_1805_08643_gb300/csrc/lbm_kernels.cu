@@ -69,6 +69,14 @@ __device__ __forceinline__ void pull_q(const S *__restrict__ g, int n, const Nbh
   for (int a = 0; a < Q; ++a) f[a] = (T)Lat<Q>::load(g + (size_t)a * n + Lat<Q>::src(nb, a), a);
 }
 
+// Stores one node's population of direction a, and its copy at the end of a padded row.
+template <int Q, typename S, typename T>
+__device__ __forceinline__ void store_node(S *__restrict__ g, int a, const KParams &P, const Nbhd &nb, T v) {
+  S *at = g + (size_t)a * P.np + nb.self;
+  Lat<Q>::store(at, a, v);
+  if (P.px != P.nx && nb.x == 0) Lat<Q>::store(at + P.nx, a, v);
+}
+
 __device__ __forceinline__ bool node_of_thread(const KParams &P, int &x, int &y, int &z) {
   x = blockIdx.x * blockDim.x + threadIdx.x;
   y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -87,7 +95,7 @@ __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S 
   if (!node_of_thread(P, x, y, z)) return;
   const Nbhd nb(x, y, z, P);
   T f[Q];
-  pull_q<Q, S, T>(g, P.n, nb, f);
+  pull_q<Q, S, T>(g, P.np, nb, f);
   T drho;
   if constexpr (Q == 15) {
     drho = q15::drho(f);
@@ -123,14 +131,14 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
   if (!node_of_thread(P, x, y, z)) return;
   const Nbhd nb(x, y, z, P);
   T f[Q];
-  pull_q<Q, S, T>(g_in, P.n, nb, f);
+  pull_q<Q, S, T>(g_in, P.np, nb, f);
   // interaction force, Eq. 15
   T p[Q];
 #pragma unroll
   for (int a = 1; a < Q; ++a) p[a] = (T)__ldg(psi + Lat<Q>::dst(nb, a));
   p[0] = (T)__ldg(psi + nb.self);
   T Sx, Sy, Sz;
-  auto out = [&](int a, T v) { Lat<Q>::store(g_out + (size_t)a * P.n + nb.self, a, v); };
+  auto out = [&](int a, T v) { Lat<Q>::store(g_out + (size_t)a * P.np + nb.self, a, v); };
   if constexpr (PREC == kF64) {
     psi_sums64<Q>(p, Sx, Sy, Sz);
     const double k = C.k[kForce] * p[0], S2 = SIGMA ? Sx * Sx + Sy * Sy + Sz * Sz : 0.0;
@@ -263,7 +271,7 @@ __device__ __forceinline__ void node_moments(const typename Types<PREC>::S *__re
   // the sums of Eq. 15 with the diagonal (corner) weight taken out: axis entries weigh 2 (8) times as much
   constexpr float axw = Q == 19 ? 2.0f : 8.0f;
   T f[Q], p[Q];
-  pull_q<Q, S, T>(g, P.n, nb, f);
+  pull_q<Q, S, T>(g, P.np, nb, f);
 #pragma unroll
   for (int a = 1; a < Q; ++a) p[a] = psi[Lat<Q>::dst(nb, a)];
   p[0] = psi[nb.self];
@@ -304,12 +312,13 @@ __global__ void moments_kernel(const typename Types<PREC>::S *__restrict__ g,
   const Nbhd nb(x, y, z, P);
   double rho, rux, ruy, ruz;
   node_moments<PREC, Q>(g, psi, P, nb, rho, rux, ruy, ruz);
-  if (rho_out) rho_out[nb.self] = rho;
+  const int i = x + P.nx * (y + P.ny * z);
+  if (rho_out) rho_out[i] = rho;
   if (u_out) {
     const double inv = recip(rho);
-    u_out[nb.self] = rux * inv;
-    u_out[(size_t)P.n + nb.self] = ruy * inv;
-    u_out[2 * (size_t)P.n + nb.self] = ruz * inv;
+    u_out[i] = rux * inv;
+    u_out[(size_t)P.n + i] = ruy * inv;
+    u_out[2 * (size_t)P.n + i] = ruz * inv;
   }
 }
 
@@ -455,11 +464,11 @@ __global__ void state_from_rho_kernel(const double *__restrict__ rho, typename T
   using S = typename Types<PREC>::S;
   int x, y, z;
   if (!node_of_thread(P, x, y, z)) return;
-  const Nbhd nb(x, y, z, P);
+  const Nbhd nb(x, y, z, P), pub(x, y, z, P, P.nx);
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
-    const double v = Lat<Q>::w(a) * (rho[Lat<Q>::dst(nb, a)] - P.rho_ref);
-    Lat<Q>::store(g + (size_t)a * P.n + nb.self, a, (typename Types<PREC>::T)v);
+    const double v = Lat<Q>::w(a) * (rho[Lat<Q>::dst(pub, a)] - P.rho_ref);
+    store_node<Q>(g, a, P, nb, (typename Types<PREC>::T)v);
   }
 }
 
@@ -471,11 +480,12 @@ __global__ void get_populations_kernel(const typename Types<PREC>::S *__restrict
   int x, y, z;
   if (!node_of_thread(P, x, y, z)) return;
   const Nbhd nb(x, y, z, P);
+  const int i = x + P.nx * (y + P.ny * z);
 #pragma unroll
   for (int a = 0; a < Q; ++a)
     if (a >= a_lo && a < a_hi)
-      out[(size_t)(a - a_lo) * P.n + nb.self] =
-          Lat<Q>::w(a) * P.rho_ref + (double)Lat<Q>::load(g + (size_t)a * P.n + Lat<Q>::src(nb, a), a);
+      out[(size_t)(a - a_lo) * P.n + i] =
+          Lat<Q>::w(a) * P.rho_ref + (double)Lat<Q>::load(g + (size_t)a * P.np + Lat<Q>::src(nb, a), a);
 }
 
 // Reverse of the above: g_a(y) = f_a(y + e_a) - w_a rho_ref.
@@ -485,12 +495,12 @@ __global__ void set_populations_kernel(const double *__restrict__ f, typename Ty
   using S = typename Types<PREC>::S;
   int x, y, z;
   if (!node_of_thread(P, x, y, z)) return;
-  const Nbhd nb(x, y, z, P);
+  const Nbhd nb(x, y, z, P), pub(x, y, z, P, P.nx);
 #pragma unroll
   for (int a = 0; a < Q; ++a)
     if (a >= a_lo && a < a_hi) {
-      const double v = f[(size_t)(a - a_lo) * P.n + Lat<Q>::dst(nb, a)] - Lat<Q>::w(a) * P.rho_ref;
-      Lat<Q>::store(g + (size_t)a * P.n + nb.self, a, (typename Types<PREC>::T)v);
+      const double v = f[(size_t)(a - a_lo) * P.n + Lat<Q>::dst(pub, a)] - Lat<Q>::w(a) * P.rho_ref;
+      store_node<Q>(g, a, P, nb, (typename Types<PREC>::T)v);
     }
 }
 

@@ -1,5 +1,5 @@
 // Two-pass kernels for the FP32-arithmetic forms with two x-adjacent nodes per
-// thread (Nx even).
+// thread (rows of even length, KParams::px).
 //
 // A thread owns the pair (x, x+1), x even.  Populations that arrive along
 // e_x = 0 come from an aligned pair (x, x+1) of the source row: one 64-bit
@@ -65,13 +65,13 @@ __global__ void __launch_bounds__(128) psi_pair_kernel(const S *__restrict__ g, 
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[19];
-  pull_pair<S>(g, (unsigned)P.n, nb, px, f);
+  pull_pair<S>(g, (unsigned)P.np, nb, px, f);
   unsigned e = 0;
-  *(float2 *)(psi + nb.self) = psi_pair<EOS, DF>(drho_pair(f), P, e);
+  store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(drho_pair(f), P, px.x), P, e));
   if (e) atomicOr(err, e);
 }
 
-template <typename S, int OP, bool SIGMA>
+template <typename S, int OP, bool SIGMA, bool ODD>
 __global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                          const float *__restrict__ psi, const KParams P) {
   PairX px;
@@ -79,12 +79,11 @@ __global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[19];
-  pull_pair<S>(g_in, (unsigned)P.n, nb, px, f);
+  pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
   V2 p[19];
   gather_psi_pair(psi, nb, px, p);
   force_collide_pair<OP, SIGMA>(f, p, P, Rates<V2>(P), OP);
-#pragma unroll
-  for (int a = 0; a < 19; ++a) PairIO<S>::st2(g_out + (size_t)a * P.n + nb.self, a, f[a]);
+  store_pair_f<S, ODD>(g_out, P, px.x, (unsigned)nb.self, f);
 }
 
 // ------------------------------------------------------------------ D3Q15
@@ -98,23 +97,23 @@ __global__ void __launch_bounds__(128) psi_pair15_kernel(const S *__restrict__ g
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[q15::kQ];
-  pull_pair15<S>(g, (unsigned)P.n, nb, px, f);
+  pull_pair15<S>(g, (unsigned)P.np, nb, px, f);
   unsigned e = 0;
-  *(float2 *)(psi + nb.self) = psi_pair<EOS, DF>(q15::drho(f), P, e);
+  store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(q15::drho(f), P, px.x), P, e));
   if (e) atomicOr(err, e);
 }
 
-template <typename S, bool SIGMA>
+template <typename S, bool SIGMA, bool ODD>
 __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                            const float *__restrict__ psi, const KParams P) {
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
-  fused_pair15_at<S, SIGMA>(g_in, g_out, psi, P, px.x, y, z);
+  fused_pair15_at<S, SIGMA, false, ODD>(g_in, g_out, psi, P, px.x, y, z);
 }
 
 dim3 pair_grid(const KParams &P, const Launch &L) {
-  return dim3((P.nx / 2 + 31) / 32, (P.ny + L.by - 1) / L.by, P.nz);
+  return dim3((P.px / 2 + 31) / 32, (P.ny + L.by - 1) / L.by, P.nz);
 }
 
 template <typename S, bool DF>
@@ -138,7 +137,7 @@ cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsign
   return cudaGetLastError();
 }
 
-template <typename S>
+template <typename S, bool ODD>
 cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void *g_in, void *g_out,
                                 const void *psi, const Launch &L) {
   const dim3 grid = pair_grid(P, L), block(32, L.by);
@@ -146,14 +145,14 @@ cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void
   S *go = (S *)g_out;
   const float *pp = (const float *)psi;
   if (P.q == 15) {
-    if (sigma) fused_pair15_kernel<S, true><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-    else fused_pair15_kernel<S, false><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
+    if (sigma) fused_pair15_kernel<S, true, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
+    else fused_pair15_kernel<S, false, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
   } else if (op == kNonOrth) {
-    if (sigma) fused_pair_kernel<S, kNonOrth, true><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-    else fused_pair_kernel<S, kNonOrth, false><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
+    if (sigma) fused_pair_kernel<S, kNonOrth, true, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
+    else fused_pair_kernel<S, kNonOrth, false, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
   } else {
-    if (sigma) fused_pair_kernel<S, kOrth, true><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-    else fused_pair_kernel<S, kOrth, false><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
+    if (sigma) fused_pair_kernel<S, kOrth, true, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
+    else fused_pair_kernel<S, kOrth, false, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
   }
   return cudaGetLastError();
 }
@@ -191,8 +190,8 @@ __global__ void __launch_bounds__(TXP *TY) batch_psi_kernel(const BatchBox *__re
     for (int z = w.z; z < w.w; ++z) {
       const Nbhd nb(x, y, z, P);
       V2 f[19];
-      pull_pair<S>(g, (unsigned)P.n, nb, px, f);
-      *(float2 *)(psi + nb.self) = psi_pair<EOS, false>(drho_pair(f), P, e);
+      pull_pair<S>(g, (unsigned)P.np, nb, px, f);
+      store_pair_psi<true>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, false>(pad_lane<true>(drho_pair(f), P, x), P, e));
     }
   }
   if (e) atomicOr(err, e);
@@ -222,7 +221,7 @@ __global__ void __launch_bounds__(TXP *TY, kFlatFusedThreadsPerSM / (TXP * TY)) 
   const int x = (t % ntx) * (2 * TXP) + 2 * threadIdx.x, y = (t / ntx) * TY + threadIdx.y;
   if (x >= P.nx || y >= P.ny || z >= P.nz) return;
   const int in = bb.cur ^ parity;
-  fused_pair_at<S, OP, true, false>((const S *)bb.g[in], (S *)bb.g[in ^ 1], bb.psi[in], P, x, y, z, Rates<V2>(P));
+  fused_pair_at<S, OP, true, false, true>((const S *)bb.g[in], (S *)bb.g[in ^ 1], bb.psi[in], P, x, y, z, Rates<V2>(P));
 }
 
 // The fused and psi kernels of one step for a storage type and tile shape;
@@ -286,7 +285,7 @@ cudaError_t batch_pair_dispatch(int precision, int tile, int eos, const BatchBox
 
 }  // namespace
 
-bool pair_supported(const KParams &P, int precision) { return precision != kF64 && P.nx % 2 == 0; }
+bool pair_supported(const KParams &P, int precision) { return precision != kF64 && P.px % 2 == 0; }
 
 cudaError_t batch_pair_occupancy(int precision, int eos, int tile, int per_sm[2]) {
   const int none[2] = {0, 0};
@@ -310,8 +309,10 @@ cudaError_t launch_psi_pair(const KParams &P, int precision, const void *g, void
 
 cudaError_t launch_fused_pair(const KParams &P, int precision, int op, bool sigma, const void *g_in, void *g_out,
                               const void *psi, const Launch &L) {
-  if (precision == kF32) return fused_pair_dispatch<float>(P, op, sigma, g_in, g_out, psi, L);
-  return fused_pair_dispatch<__half>(P, op, sigma, g_in, g_out, psi, L);
+  const bool odd = P.px != P.nx;
+  auto launch = precision == kF32 ? (odd ? fused_pair_dispatch<float, true> : fused_pair_dispatch<float, false>)
+                                  : (odd ? fused_pair_dispatch<__half, true> : fused_pair_dispatch<__half, false>);
+  return launch(P, op, sigma, g_in, g_out, psi, L);
 }
 
 }  // namespace lbm

@@ -83,7 +83,7 @@ __device__ __forceinline__ void fused_plane(const S *__restrict__ g_in, S *__res
                                             int z, const Rates<V2> &r) {
   const int x = (t % T.nx_t) * 2 * TXP + 2 * threadIdx.x, y = (t / T.nx_t) * TYR + threadIdx.y;
   if (x >= P.nx || y >= P.ny) return;
-  fused_pair_at<S, OP, SIGMA>(g_in, g_out, psi, P, x, y, z, r);
+  fused_pair_at<S, OP, SIGMA, true, false>(g_in, g_out, psi, P, x, y, z, r);
 }
 
 template <typename S, int EOS, bool DF>
@@ -91,7 +91,7 @@ __device__ __forceinline__ void psi_plane(const S *__restrict__ g, float *__rest
                                           const Tiles &T, int t, int z, unsigned &e) {
   const int x = (t % T.nx_t) * 2 * TXP + 2 * threadIdx.x, y = (t / T.nx_t) * TYR + threadIdx.y;
   if (x >= P.nx || y >= P.ny) return;
-  psi_pair_at_l2<S, EOS, DF>(g, psi, P, x, y, z, e);
+  psi_pair_at_l2<S, EOS, DF, true, false>(g, psi, P, x, y, z, e);
 }
 
 // Block b works on z chunk b / per_chunk ([z0, z1), at least three planes) and

@@ -64,19 +64,20 @@ __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *_
   const bool active = tid < NE;
   const int lx = tid % EX, ly = tid / EX;
   const int nx = P.nx, ny = P.ny, nz = P.nz;
-  const unsigned n = (unsigned)P.n, nxy = (unsigned)(nx * ny);
+  const int px = P.px;  // row length of the stored arrays
+  const unsigned n = (unsigned)P.np, nxy = (unsigned)(px * ny);
   const int gx = wrap(x0 + lx - 1, nx), gy = wrap(y0 + ly - 1, ny);
   const bool interior = active && lx >= 1 && lx <= BX && ly >= 1 && ly <= BY && x0 + lx - 1 < nx &&
                         y0 + ly - 1 < ny;
   const Rates<float> r(P);
   const float rho_ref = P.frho_ref, mG = -P.fG;
 
-  // In-plane offsets (y' nx + x') of the pull sources x - e_a of this node: the
+  // In-plane offsets (y' px + x') of the pull sources x - e_a of this node: the
   // nine (x - ex, y - ey) combinations, computed once.  Element offsets are
   // unsigned 32-bit: 19 N < 2^32 for every box the library accepts.
   const int xm = gx == 0 ? nx - 1 : gx - 1, xp = gx == nx - 1 ? 0 : gx + 1;
   const int ym = gy == 0 ? ny - 1 : gy - 1, yp = gy == ny - 1 ? 0 : gy + 1;
-  const unsigned r0 = (unsigned)(gy * nx), rm = (unsigned)(ym * nx), rp = (unsigned)(yp * nx);
+  const unsigned r0 = (unsigned)(gy * px), rm = (unsigned)(ym * px), rp = (unsigned)(yp * px);
   const unsigned o_00 = r0 + gx, o_m0 = r0 + xm, o_p0 = r0 + xp;  // (x-ex) with ey = 0
   const unsigned o_0m = rm + gx, o_0p = rp + gx;                 // ex = 0, y - ey = y-1 / y+1
   const unsigned o_mm = rm + xm, o_pp = rp + xp, o_mp = rp + xm, o_pm = rm + xp;
@@ -89,7 +90,7 @@ __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *_
   for (int k = 0; k < KPSI; ++k) {
     const int q = tid + k * NT;
     psi_ok[k] = q < NP;
-    psi_xy[k] = psi_ok[k] ? (unsigned)(wrap(x0 - 2 + q % PX, nx) + nx * wrap(y0 - 2 + q / PX, ny)) : 0u;
+    psi_xy[k] = psi_ok[k] ? (unsigned)(wrap(x0 - 2 + q % PX, nx) + px * wrap(y0 - 2 + q / PX, ny)) : 0u;
   }
   auto psi_slot = [&](int zp) { return sm_psi + (zp & 3) * NP; };
   auto zwrap = [&](int zp) { return zp < 0 ? zp + nz : (zp >= nz ? zp - nz : zp); };
@@ -169,6 +170,10 @@ __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *_
         const unsigned self = (unsigned)zz * nxy + o_00;
 #pragma unroll
         for (int a = 0; a < 19; ++a) Storage<S>::store(g_out + (unsigned)a * n + self, a, f[a]);
+        if (px != nx && gx == 0) {  // the copy of node 0 at the end of a padded row
+#pragma unroll
+          for (int a = 0; a < 19; ++a) Storage<S>::store(g_out + (unsigned)a * n + self + nx, a, f[a]);
+        }
       }
 #pragma unroll
       for (int a = 1; a < 19; ++a) buf[(a - 1) * NE + tid] = f[a];

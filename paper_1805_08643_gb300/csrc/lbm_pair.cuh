@@ -1,5 +1,5 @@
 // Pair access for the kernels that give each thread two x-adjacent nodes
-// (x even, Nx even): loads and stores of stored populations as pairs, the pull
+// (x even, rows of even length: KParams::px): loads and stores of stored populations as pairs, the pull
 // of both nodes' 19 populations (Eq. 5), their density, psi, force and
 // collision on packed FP32 pairs (V2).
 #pragma once
@@ -17,6 +17,7 @@ template <> struct PairIO<float> {
   static __device__ __forceinline__ float ld1(const float *p) { return __ldg(p); }
   static __device__ __forceinline__ V2 decode(float2 v, int a) { (void)a; return V2(v); }
   static __device__ __forceinline__ void st2(float *p, int a, V2 v) { (void)a; *(float2 *)p = v.v; }
+  static __device__ __forceinline__ void st1(float *p, int a, V2 v) { (void)a; *p = v.v.x; }  // the first lane
 };
 template <> struct PairIO<__half> {
   static __device__ __forceinline__ float2 ld2(const __half *p) { return __half22float2(__ldg((const __half2 *)p)); }
@@ -24,6 +25,9 @@ template <> struct PairIO<__half> {
   static __device__ __forceinline__ V2 decode(float2 v, int a) { return V2(v) * V2(lattice_w(a)); }
   static __device__ __forceinline__ void st2(__half *p, int a, V2 v) {
     *(__half2 *)p = __float22half2_rn(V2(v * V2((double)lattice_inv_w(a))).v);
+  }
+  static __device__ __forceinline__ void st1(__half *p, int a, V2 v) {
+    *p = __float2half_rn(V2(v * V2((double)lattice_inv_w(a))).v.x);
   }
 };
 
@@ -46,7 +50,10 @@ __device__ __forceinline__ constexpr int ex_of(int a) {
   return (a == 1 || a == 7 || a == 9 || a == 11 || a == 13) ? 1 : (a == 2 || a == 8 || a == 10 || a == 12 || a == 14) ? -1 : 0;
 }
 
-// x positions of a pair: x (even), x - 1 and x + 2 wrapped periodically.
+// x positions of a pair: x (even), x - 1 and x + 2 wrapped periodically.  With
+// an odd Nx the last pair holds node Nx - 1 and the row's pad, which repeats
+// node 0, so x + 1 is read where it stands there too; the pad's own lane
+// computes on whatever its neighbours hold and is not stored.
 struct PairX {
   int x, xm1, xp2;
 };
@@ -69,6 +76,47 @@ __device__ __forceinline__ void pull_pair(const S *__restrict__ g, unsigned n, c
       v = make_float2(PairIO<S>::ld1(rowp + px.x + 1), PairIO<S>::ld1(rowp + px.xp2));
     f[a] = PairIO<S>::decode(v, a);
   }
+}
+
+// Stores a pair (two-lane values v of direction a, or psi) at p: both lanes, or
+// in a row padded for an odd Nx the nodes there are, node 0 once more in the
+// pad.  Kernels that only see even boxes leave ODD out (it costs registers).
+template <bool ODD, typename St2, typename St1>
+__device__ __forceinline__ void store_pair(const KParams &P, int x, St2 &&st2, St1 &&st1) {
+  if (!ODD || P.px == P.nx) {
+    st2();
+  } else {
+    if (x + 1 < P.nx) st2();
+    else st1(0);
+    if (x == 0) st1(P.nx);
+  }
+}
+
+// Stores the 19 results of a pair.
+template <typename S, bool ODD>
+__device__ __forceinline__ void store_pair_f(S *__restrict__ g, const KParams &P, int x, unsigned self, const V2 f[19]) {
+  store_pair<ODD>(
+      P, x,
+      [&] {
+#pragma unroll
+        for (int a = 0; a < 19; ++a) PairIO<S>::st2(g + (size_t)a * P.np + self, a, f[a]);
+      },
+      [&](int off) {
+#pragma unroll
+        for (int a = 0; a < 19; ++a) PairIO<S>::st1(g + (size_t)a * P.np + self + off, a, f[a]);
+      });
+}
+template <bool ODD>
+__device__ __forceinline__ void store_pair_psi(float *__restrict__ psi, const KParams &P, int x, unsigned self,
+                                               float2 v) {
+  store_pair<ODD>(P, x, [&] { *(float2 *)(psi + self) = v; }, [&](int off) { psi[self + off] = v.x; });
+}
+
+// rho - rho_ref of a pair for the EOS: the pad's lane repeats its neighbour, so that it flags nothing of its own.
+template <bool ODD>
+__device__ __forceinline__ V2 pad_lane(V2 drho, const KParams &P, int x) {
+  if (ODD && x + 1 >= P.nx) drho.v.y = drho.v.x;
+  return drho;
 }
 
 // rho - rho_ref of both nodes: the sum of the pulled deviations (Eq. 6).
@@ -149,7 +197,7 @@ __device__ __forceinline__ PairX pair_x(const KParams &P, int x) {
 // which keeps the registers of the single-pass kernels down.  The arithmetic
 // and its order are those of fused_pair_kernel, so the results are equal bit
 // for bit.
-template <typename S, int OP, bool SIGMA, bool FORCE_FIRST = true>
+template <typename S, int OP, bool SIGMA, bool FORCE_FIRST, bool ODD>
 __device__ __forceinline__ void fused_pair_at(const S *__restrict__ g_in, S *__restrict__ g_out,
                                               const float *__restrict__ psi, const KParams &P, int x, int y, int z,
                                               const Rates<V2> &r) {
@@ -158,7 +206,7 @@ __device__ __forceinline__ void fused_pair_at(const S *__restrict__ g_in, S *__r
   V2 f[19];
   // without FORCE_FIRST both sets of loads are issued before either is used
   // (one memory round trip, more registers)
-  if (!FORCE_FIRST) pull_pair<S>(g_in, (unsigned)P.n, nb, px, f);
+  if (!FORCE_FIRST) pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
   V2 Fx, Fy, Fz, dS4;
   {
     V2 p[19];
@@ -181,15 +229,14 @@ __device__ __forceinline__ void fused_pair_at(const S *__restrict__ g_in, S *__r
     p[18] = row1(nb.rmp);
     force_pair<SIGMA>(p, P, Fx, Fy, Fz, dS4);
   }
-  if (FORCE_FIRST) pull_pair<S>(g_in, (unsigned)P.n, nb, px, f);
+  if (FORCE_FIRST) pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
   collide_pair<OP>(f, Fx, Fy, Fz, dS4, P, r, OP);
-#pragma unroll
-  for (int a = 0; a < 19; ++a) PairIO<S>::st2(g_out + (size_t)a * P.n + nb.self, a, f[a]);
+  store_pair_f<S, ODD>(g_out, P, x, (unsigned)nb.self, f);
 }
 
 // psi of one pair from populations written earlier in the same launch (the
 // psi pass of psi_pair_kernel, pulls through L2).
-template <typename S, int EOS, bool DF, bool ICVT = true>
+template <typename S, int EOS, bool DF, bool ICVT, bool ODD>
 __device__ __forceinline__ void psi_pair_at_l2(const S *__restrict__ g, float *__restrict__ psi, const KParams &P,
                                                int x, int y, int z, unsigned &e) {
   const PairX px = pair_x(P, x);
@@ -197,7 +244,7 @@ __device__ __forceinline__ void psi_pair_at_l2(const S *__restrict__ g, float *_
   V2 f[19];
 #pragma unroll
   for (int a = 0; a < 19; ++a) {
-    const S *rowp = g + (size_t)a * P.n + src_row(nb, a);
+    const S *rowp = g + (size_t)a * P.np + src_row(nb, a);
     float2 v;
     if (ex_of(a) == 0)
       v = L2Load<S>::ld2(rowp + px.x);
@@ -207,7 +254,7 @@ __device__ __forceinline__ void psi_pair_at_l2(const S *__restrict__ g, float *_
       v = make_float2(L2Load<S>::ld1(rowp + px.x + 1), L2Load<S>::ld1(rowp + px.xp2));
     f[a] = PairIO<S>::decode(v, a);
   }
-  *(float2 *)(psi + nb.self) = psi_pair<EOS, DF, ICVT>(drho_pair(f), P, e);
+  store_pair_psi<ODD>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, DF, ICVT>(pad_lane<ODD>(drho_pair(f), P, x), P, e));
 }
 
 // Cross-block signalling inside one launch: a release increment of a

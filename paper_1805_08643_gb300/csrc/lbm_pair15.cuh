@@ -16,11 +16,15 @@ namespace lbm {
 template <typename S> struct PairIO15 {
   static __device__ __forceinline__ V2 decode(float2 v, int a) { return PairIO<S>::decode(v, a); }
   static __device__ __forceinline__ void st2(S *p, int a, V2 v) { PairIO<S>::st2(p, a, v); }
+  static __device__ __forceinline__ void st1(S *p, int a, V2 v) { PairIO<S>::st1(p, a, v); }
 };
 template <> struct PairIO15<__half> {
   static __device__ __forceinline__ V2 decode(float2 v, int a) { return V2(v) * V2(q15::w(a)); }
   static __device__ __forceinline__ void st2(__half *p, int a, V2 v) {
     *(__half2 *)p = __float22half2_rn(V2(v * V2((double)q15::inv_w(a))).v);
+  }
+  static __device__ __forceinline__ void st1(__half *p, int a, V2 v) {
+    *p = __float2half_rn(V2(v * V2((double)q15::inv_w(a))).v.x);
   }
 };
 
@@ -84,13 +88,13 @@ __device__ __forceinline__ void gather_psi_pair15(const float *__restrict__ psi,
 
 // Fused pass of one pair on D3Q15 (pull, force from the psi stencil, collision,
 // store); FORCE_FIRST as in fused_pair_at.
-template <typename S, bool SIGMA, bool FORCE_FIRST = false>
+template <typename S, bool SIGMA, bool FORCE_FIRST, bool ODD>
 __device__ __forceinline__ void fused_pair15_at(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                 const float *__restrict__ psi, const KParams &P, int x, int y, int z) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
   V2 f[q15::kQ];
-  if (!FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.n, nb, px, f);
+  if (!FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.np, nb, px, f);
   V2 Fx, Fy, Fz, dS4;
   {
     V2 p[q15::kQ];
@@ -103,21 +107,30 @@ __device__ __forceinline__ void fused_pair15_at(const S *__restrict__ g_in, S *_
     Fy = kk * Sy;
     Fz = kk * Sz;
   }
-  if (FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.n, nb, px, f);
+  if (FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.np, nb, px, f);
   q15::collide<V2>(f, V2((double)P.frho_ref), Fx, Fy, Fz, dS4, Rates<V2>(P));
+  store_pair<ODD>(
+      P, x,
+      [&] {
 #pragma unroll
-  for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st2(g_out + (size_t)a * P.n + nb.self, a, f[a]);
+        for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st2(g_out + (size_t)a * P.np + nb.self, a, f[a]);
+      },
+      [&](int off) {
+#pragma unroll
+        for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st1(g_out + (size_t)a * P.np + nb.self + off, a, f[a]);
+      });
 }
 
 // psi of one pair on D3Q15 from populations written earlier in the same launch (pulls through L2).
-template <typename S, int EOS, bool DF, bool ICVT = true>
+template <typename S, int EOS, bool DF, bool ICVT, bool ODD>
 __device__ __forceinline__ void psi_pair15_at_l2(const S *__restrict__ g, float *__restrict__ psi, const KParams &P,
                                                  int x, int y, int z, unsigned &e) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
   V2 f[q15::kQ];
-  pull_pair15<S, L2Load<S>>(g, (unsigned)P.n, nb, px, f);
-  *(float2 *)(psi + nb.self) = psi_pair<EOS, DF, ICVT>(q15::drho(f), P, e);
+  pull_pair15<S, L2Load<S>>(g, (unsigned)P.np, nb, px, f);
+  store_pair_psi<ODD>(psi, P, x, (unsigned)nb.self,
+                      psi_pair<EOS, DF, ICVT>(pad_lane<ODD>(q15::drho(f), P, x), P, e));
 }
 
 }  // namespace lbm

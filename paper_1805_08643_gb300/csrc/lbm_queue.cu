@@ -129,9 +129,9 @@ __global__ void __launch_bounds__(NTH, min_blocks(Q))
       const int x = (t % G.ntx) * 2 * TXP + 2 * lane, y = (t / G.ntx) * kRows + row;
       if (x < P.nx && y < P.ny) {
         if constexpr (Q == 15)
-          fused_pair15_at<S, SIGMA, true>(g_in, g_out, psi_in, P, x, y, z);
+          fused_pair15_at<S, SIGMA, true, false>(g_in, g_out, psi_in, P, x, y, z);
         else
-          fused_pair_at<S, OP, SIGMA, true>(g_in, g_out, psi_in, P, x, y, z, Rates<V2>(P));
+          fused_pair_at<S, OP, SIGMA, true, false>(g_in, g_out, psi_in, P, x, y, z, Rates<V2>(P));
       }
       if (lane == 0 && row == 0) s_next[par] = next_item(claim - base, nitems, e);
       __syncthreads();
@@ -166,9 +166,9 @@ __global__ void __launch_bounds__(NTH, min_blocks(Q))
       const int x = tx * 2 * TXP + 2 * lane, y = ty * kRows + row;
       if (x < P.nx && y < P.ny) {
         if constexpr (Q == 15)
-          psi_pair15_at_l2<S, EOS, DF, kIntCvt>(g_out, psi_out, P, x, y, z, e);
+          psi_pair15_at_l2<S, EOS, DF, kIntCvt, false>(g_out, psi_out, P, x, y, z, e);
         else
-          psi_pair_at_l2<S, EOS, DF, kIntCvt>(g_out, psi_out, P, x, y, z, e);
+          psi_pair_at_l2<S, EOS, DF, kIntCvt, false>(g_out, psi_out, P, x, y, z, e);
       }
     }
     k = kn;
@@ -291,7 +291,8 @@ __device__ __forceinline__ void prefetch_boxes(BatchBox *dst, const BatchBox *__
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <typename S, int EOS>
+// ODD: some box has an odd Nx (rows padded to an even length, KParams::px).
+template <typename S, int EOS, bool ODD>
 __global__ void __launch_bounds__(NTH, kBatchBlocks)
     batch_queue_kernel(const BatchBox *__restrict__ boxes, const int4 *__restrict__ items, int nitems, int parity,
                        int *__restrict__ done, int ndone, unsigned *__restrict__ err) {
@@ -324,9 +325,9 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
         const S *gi = (const S *)B.g[in];
         S *go = (S *)B.g[in ^ 1];
         if (B.op == kNonOrth)
-          fused_pair_at<S, kNonOrth, true, false>(gi, go, B.psi[in], P, x, y, z, Rates<V2>(P));
+          fused_pair_at<S, kNonOrth, true, false, ODD>(gi, go, B.psi[in], P, x, y, z, Rates<V2>(P));
         else
-          fused_pair_at<S, kOrth, true, false>(gi, go, B.psi[in], P, x, y, z, Rates<V2>(P));
+          fused_pair_at<S, kOrth, true, false, ODD>(gi, go, B.psi[in], P, x, y, z, Rates<V2>(P));
       }
       __syncthreads();
       if (tid == 0) counter_release_add(done + LBM_IDX(B.qbase + z * B.T + t, ndone), 1);
@@ -365,7 +366,7 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
       if (!__all_sync(0xffffffffu, ok)) e |= kErrTimeout;
       const int in = B.cur ^ parity;
       const int x = tx * B.tw + 2 * (tid & ((1 << B.hshift) - 1)), y = ty * B.th + (tid >> B.hshift);
-      if (x < P.nx && y < P.ny) psi_pair_at_l2<S, EOS, false, kIntCvt>((const S *)B.g[in ^ 1], B.psi[in ^ 1], P, x, y, z, e);
+      if (x < P.nx && y < P.ny) psi_pair_at_l2<S, EOS, false, kIntCvt, ODD>((const S *)B.g[in ^ 1], B.psi[in ^ 1], P, x, y, z, e);
     }
     __syncthreads();  // s_next and s_it are written; rewritten only after the next item's first barrier
     k = s_next;
@@ -375,23 +376,23 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
   if (e) atomicOr(err, e);
 }
 
-template <typename S, int EOS>
+template <typename S, int EOS, bool ODD>
 cudaError_t batch_launch(const BatchBox *boxes, const int4 *items, int nitems, int parity, int grid, int *done,
                          int ndone, unsigned *err, cudaStream_t s, int *per_sm) {
-  auto kern = batch_queue_kernel<S, EOS>;
+  auto kern = batch_queue_kernel<S, EOS, ODD>;
   if (per_sm) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, NTH, 0);
   void *args[] = {(void *)&boxes, (void *)&items, (void *)&nitems, (void *)&parity,
                   (void *)&done,  (void *)&ndone, (void *)&err};
   return cudaLaunchCooperativeKernel((const void *)kern, dim3(grid), dim3(TXP, kRows), args, 0, s);
 }
 
-template <typename S>
+template <typename S, bool ODD>
 cudaError_t batch_by_eos(int eos, const BatchBox *boxes, const int4 *items, int nitems, int parity, int grid,
                          int *done, int ndone, unsigned *err, cudaStream_t s, int *per_sm) {
   switch (eos) {
-    case kEosCS: return batch_launch<S, kEosCS>(boxes, items, nitems, parity, grid, done, ndone, err, s, per_sm);
-    case kEosExp: return batch_launch<S, kEosExp>(boxes, items, nitems, parity, grid, done, ndone, err, s, per_sm);
-    default: return batch_launch<S, kEosNone>(boxes, items, nitems, parity, grid, done, ndone, err, s, per_sm);
+    case kEosCS: return batch_launch<S, kEosCS, ODD>(boxes, items, nitems, parity, grid, done, ndone, err, s, per_sm);
+    case kEosExp: return batch_launch<S, kEosExp, ODD>(boxes, items, nitems, parity, grid, done, ndone, err, s, per_sm);
+    default: return batch_launch<S, kEosNone, ODD>(boxes, items, nitems, parity, grid, done, ndone, err, s, per_sm);
   }
 }
 
@@ -526,7 +527,7 @@ bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std:
   for (size_t b = 0; b < boxes.size(); ++b) {
     const KParams &P = *boxes[b];
     const BatchGeo G = batch_geo(P, batch_tile_width(P.nx));
-    if (P.nz < 3 || P.nx % 2 != 0 || P.nz > 0xffff || G.T > 0xffff || grid < 1) return false;
+    if (P.nz < 3 || P.px % 2 != 0 || P.nz > 0xffff || G.T > 0xffff || grid < 1) return false;
     first[b + 1] = first[b] + (long long)P.nz * G.T;
     if (first[b + 1] >= (1LL << 30)) return false;
     base[b] = (int)first[b];
@@ -587,8 +588,8 @@ bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std:
 cudaError_t batch_queue_grid(int precision, int eos, int *grid) {
   int per_sm = 0, dev = 0, sms = 0;
   cudaError_t e = precision == kF32
-                      ? batch_by_eos<float>(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm)
-                      : batch_by_eos<__half>(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm);
+                      ? batch_by_eos<float, true>(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm)
+                      : batch_by_eos<__half, true>(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
@@ -597,13 +598,12 @@ cudaError_t batch_queue_grid(int precision, int eos, int *grid) {
   return cudaSuccess;
 }
 
-cudaError_t launch_batch_queue(int precision, int eos, const BatchBox *boxes, const int4 *items, int nitems,
+cudaError_t launch_batch_queue(int precision, int eos, bool odd, const BatchBox *boxes, const int4 *items, int nitems,
                                int parity, int grid, int *done, int ndone, unsigned *err, cudaStream_t s) {
-  if (precision == kF32)
-    return batch_by_eos<float>(eos, boxes, items, nitems, parity, grid, done, ndone, err, s, nullptr);
-  if (precision == kF16)
-    return batch_by_eos<__half>(eos, boxes, items, nitems, parity, grid, done, ndone, err, s, nullptr);
-  return cudaErrorInvalidValue;
+  if (precision != kF32 && precision != kF16) return cudaErrorInvalidValue;
+  auto launch = precision == kF32 ? (odd ? batch_by_eos<float, true> : batch_by_eos<float, false>)
+                                  : (odd ? batch_by_eos<__half, true> : batch_by_eos<__half, false>);
+  return launch(eos, boxes, items, nitems, parity, grid, done, ndone, err, s, nullptr);
 }
 
 }  // namespace lbm
