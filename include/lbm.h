@@ -67,8 +67,8 @@ typedef enum {
  * from the D3Q19 rows each vector equals (their mean where several coincide;
  * zero for e_x e_y e_z), rates 1, s_e, s_nu x5, s_q x4, s_pi, and Eq. 15 weights
  * 1/3 (axes), 1/24 (corners).  A D3Q15 context runs the two-pass step (the
- * two-node kernels for the FP32-arithmetic forms with an even Nx, the one-node
- * kernels otherwise) or, for those forms, the work-list step (mode 5 of
+ * two-node kernels for the FP32-arithmetic forms, the one-node kernels for
+ * LBM_F64) or, for those forms, the work-list step (mode 5 of
  * lbm_set_tuning; the default with LBM_F32 storage); the other single-pass
  * variants, the no-alloc step (lbm_step_static) and batches are D3Q19 only. */
 typedef enum {
@@ -114,8 +114,9 @@ lbm_status lbm_create(const int grid[3], const lbm_eos *eos, double G,
                       void *cuda_stream, lbm_ctx **out);
 
 /* Bytes of the three device buffers a context needs: each of the two
- * population buffers (Q N stored values, and never less than 4N doubles: the
- * spare one stages rho and u for lbm_moments), the psi buffer (two time levels
+ * population buffers (Q N stored values, rows of an odd Nx one element longer in
+ * the FP32-arithmetic forms, and never less than 4N doubles: the spare one
+ * stages rho and u for lbm_moments), the psi buffer (two time levels
  * of psi), and the scratch buffer (reductions and the error word). */
 lbm_status lbm_buffer_bytes(const lbm_ctx *ctx, size_t *population_bytes,
                             size_t *psi_bytes, size_t *scratch_bytes);
@@ -208,9 +209,10 @@ lbm_status lbm_kernel_times(lbm_ctx *ctx, double *ms_psi, long long *n_psi,
  * call in this mode allocates a small device array of progress flags (one int
  * per 64x4 tile and plane), freed by lbm_destroy.  5 (same forms; also
  * on D3Q15) runs each step as one cooperative launch over an ordered work list: each
- * item is the fused pass of one 64x4 tile of one plane plus the psi pass of
- * the next step for another tile, placed (and checked, on the host) at least
- * half a wave of the grid after the 27 fused tiles it reads; the FP64 EOS of the
+ * item is the fused pass of one tile of one plane (128 node pairs in row order;
+ * 64x4 nodes where Nx > 512) plus the psi pass of the next step for another tile,
+ * placed (and checked, on the host) at least half a wave of the grid after the
+ * fused tiles it reads; the FP64 EOS of the
  * psi work overlaps the fused work's HBM stream and the populations it pulls
  * come from L2 (Eqs. 3-6 in 2 x Q x s + 8 bytes per node); results equal the
  * two-pass step bit for bit; the first step in this mode allocates the item
@@ -281,10 +283,9 @@ lbm_status lbm_step_static(const lbm_ctx *ctx, const double *f_in, double *f_out
 
 /* ------------------------------------------------------------------ batches
  * Many independent periodic boxes advanced together: every step runs
- * persistent launches over a table of work items (one x-y tile of one box and
- * a range of z planes each, largest boxes first): when every box has an even
- * Nx, the fused pass and then the psi pass of the new state on the two-node
- * kernels of lbm_step; otherwise one launch of the single-pass kernel.
+ * persistent launches over tables of work items of all boxes (a tile of one box
+ * each, largest boxes first), on the two-node kernels of lbm_step: the work
+ * list, or the fused pass and then the psi pass of the new state.
  * lbm_batch_step replays the launches of two steps as a CUDA graph.  Boxes
  * may differ in size, operator, temperature, G, rates and sigma; they share the
  * precision (LBM_F32 or LBM_F32_STORE_F16) and the kind of EOS.  Boxes join
@@ -319,7 +320,7 @@ lbm_status lbm_batch_init_droplet(lbm_batch *b, int id, const double centre[3], 
 lbm_status lbm_batch_init_flat(lbm_batch *b, int id, int axis, double lo, double hi, double W, double rho_l,
                                double rho_v);
 
-/* Step of the batch's boxes with an even Nx: 3 (the default) the work-list
+/* Step of the batch's boxes: 3 (the default) the work-list
  * single pass (one cooperative launch per step over tile jobs of all boxes:
  * fused jobs and the next step's psi jobs, each box's psi jobs half a wave of
  * the grid behind the fused jobs they read; its completion counters, 4 bytes
@@ -327,8 +328,10 @@ lbm_status lbm_batch_init_flat(lbm_batch *b, int id, int axis, double lo, double
  * two-pass pair kernels with that tile shape (32x4, 32x8, 64x4): the fused pass
  * as a flat grid of one block per plane of a tile, one launch per operator (a
  * block-to-box table of 4 bytes per block), then the psi pass over work items
- * of a tile through z planes.  Boxes with an odd Nx run the one-node single
- * pass in the same step, tile shape as chosen (32x8 under 3).  For box id >= 0,
+ * of a tile through z planes.  Boxes with an odd Nx step like
+ * the others (their stored rows hold one element more), but for boxes so large
+ * that the longer rows would leave the index range (19 N near 2^32): those run
+ * the one-node single pass in the same step, tile shape as chosen (32x8 under 3).  For box id >= 0,
  * z_planes sets its planes per work item of the psi pass and the single pass
  * (0 = automatic).  Results do not depend on the choice (the work list and the
  * two-pass kernels are equal bit for bit). */

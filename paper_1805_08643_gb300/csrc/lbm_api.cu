@@ -382,7 +382,7 @@ lbm_status lbm_step(lbm_ctx *c, int n) {
       // the counters advance only with launches that run (each one claims every item once)
       const int stamp = c->q_stamp + 1;
       CK(timed(c, 1, [&] {
-           return lbm::launch_queue(c->P, c->precision, c->op, c->sigma_on, c->eos_f2, gin, gout, pin, pout, c->q,
+           return lbm::launch_queue(c->P, c->precision, c->op, c->eos_f2, gin, gout, pin, pout, c->q,
                                     stamp, err_word(c), c->L.stream);
          }),
          "single-pass kernel");

@@ -167,7 +167,7 @@ lbm_status rebuild(lbm_batch *b) {
     for (size_t k = 0; k < even.size(); ++k) {
       BatchBox &d = b->boxes[even[k].second].d;
       d.qbase = base[k];
-      lbm::batch_queue_geometry(d);
+      d.map = lbm::tile_map(d.P);
       desc[even[k].second] = d;
     }
     // the list numbers boxes in `even`; the kernel reads the descriptor table by slot: renumber, then
@@ -182,7 +182,7 @@ lbm_status rebuild(lbm_batch *b) {
         const KParams &P = desc[slot].P;
         const unsigned zt = (unsigned)(side ? it.w : it.y);
         const long long z = zt & 0xffffu, t = zt >> 16;
-        const long long T = lbm::batch_queue_tiles(P);
+        const long long T = desc[slot].map.T;
         if (slot >= nb || !b->boxes[slot].live || P.px % 2 != 0 || z >= P.nz || t >= T ||
             desc[slot].qbase + P.nz * T > nc)
           return bfail(b, LBM_ERR_ARG, "work list does not match the box table");

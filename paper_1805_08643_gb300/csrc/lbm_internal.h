@@ -244,6 +244,17 @@ enum Tile { kTile32x4 = 0, kTile32x8 = 1, kTile64x4 = 2 };
 cudaError_t launch_onepass(const KParams &P, int precision, int op, bool sigma, int tile, int zc, const void *g_in,
                            void *g_out, const void *psi_in, void *psi_out, unsigned *err, cudaStream_t s);
 
+// Which node pairs of a plane a work-list tile job covers: 128 consecutive
+// pairs of the plane in row order (lin), or 64 x 4 nodes.
+struct TileMap {
+  int lin;
+  int T;         // tiles per plane
+  int W, M;      // pairs per row and per plane
+  int ntx, nty;  // 64 x 4 tiles along x and y
+  unsigned m;    // lin: ceil(2^32 / W), so that v / W is (v m) >> 32 for every pair v of a plane
+};
+TileMap tile_map(const KParams &P);
+
 // One box of a batch as the batched kernel sees it (copied to shared memory
 // per work item).  g[k] / psi[k]: the two time levels; cur: which level holds
 // the state at the batch's parity 0.
@@ -255,12 +266,7 @@ struct alignas(16) BatchBox {  // 16-byte aligned: copied to shared memory in 16
   int cur;
   int qbase;  // first completion counter of this box in the batch work list, or (two-pass step) its first
               // block of the flat fused grid
-  int tw;     // its tile width there (batch_tile_width)
-  // the rest of its work-list tile geometry (batch_queue_geometry): tiles along x and y and per plane, tile
-  // height, log2 of the node pairs across a tile, and ntx_m = ceil(2^32 / ntx), so that t / ntx is
-  // (t * ntx_m) >> 32 for every tile index t < 2^16
-  int ntx, nty, T, th, hshift;
-  unsigned long long ntx_m;
+  TileMap map;  // its tiles there
 };
 
 // Persistent single-pass launch over the work items (box, tx | ty << 16, z0, z1)
@@ -329,7 +335,7 @@ cudaError_t queue_grid(int precision, int q, int *grid);
 size_t queue_counters(const KParams &P);
 bool queue_items(const KParams &P, int grid, std::vector<int4> &out);
 // stamp: 1 + the number of earlier launches on these counters.
-cudaError_t launch_queue(const KParams &P, int precision, int op, bool sigma, bool df, const void *g_in, void *g_out,
+cudaError_t launch_queue(const KParams &P, int precision, int op, bool df, const void *g_in, void *g_out,
                          const void *psi_in, void *psi_out, const QueueState &q, int stamp, unsigned *err,
                          cudaStream_t s);
 
@@ -341,9 +347,6 @@ cudaError_t launch_queue(const KParams &P, int precision, int op, bool sigma, bo
 // launch starts (the step graph clears them).
 bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std::vector<int4> &out,
                        std::vector<int> &base, long long *ncounters);
-int batch_tile_width(int nx);               // 64, 32 or 16: tiles of tw x (256 / tw) nodes
-void batch_queue_geometry(BatchBox &d);     // sets d.tw and the geometry fields from d.P
-int batch_queue_tiles(const KParams &P);   // tile jobs per plane of a box in a batch work list
 cudaError_t batch_queue_grid(int precision, int eos, int *grid);
 // odd: some box has rows padded for an odd Nx.
 cudaError_t launch_batch_queue(int precision, int eos, bool odd, const BatchBox *boxes, const int4 *items, int nitems,

@@ -2,13 +2,13 @@
 // Nx even): one persistent launch per step runs both passes of the two-pass
 // step as interleaved work.
 //
-// Work item k is a pair of tile jobs (64 x 4 nodes of one plane, one node
-// pair per thread):
+// Work item k is a pair of tile jobs (128 node pairs of one plane that follow
+// each other in row order, one per thread; see tile_map):
 //   fused job (z, tile): the fused pass (Eqs. 4-6 and 15, pull streaming of
 //     Eq. 5): reads f(t) and psi(t), writes f*(t); then counts itself done;
 //   psi job (z', tile'): the psi pass of the next step: rho(t+1) from the
 //     pulled f*(t) (Eq. 6), the EOS, psi(t+1).  It needs the fused jobs of
-//     planes z'-1..z'+1 on the tile and its eight neighbours (periodic) and
+//     planes z'-1..z'+1 on its rows and the rows next to them (periodic) and
 //     pulls their output through L2, where it still is.
 // The host builds the list (and checks it): fused jobs plane by plane; each
 // psi job in the first free item at least half a wave of the grid (grid / 2
@@ -33,8 +33,9 @@
 //
 // What this buys over two launches: the psi jobs' FP64 EOS runs on the same
 // SMs while the fused jobs stream HBM, and the populations they pull come from
-// L2 (writer and reader are about two planes plus half a wave of tiles apart): DRAM traffic per node is f(t) read and f*(t) written once plus psi
-// read and written once (2 x 19 x s + 8 bytes) against 3 x 19 x s + 8.  The
+// L2 (writer and reader are about two planes plus half a wave of tiles apart):
+// DRAM traffic per node is f(t) read and f*(t) written once plus psi read and
+// written once (2 x 19 x s + 8 bytes) against 3 x 19 x s + 8.  The
 // arithmetic and its order are those of the two-pass kernels, so the results
 // are equal bit for bit.
 //
@@ -76,16 +77,74 @@ __host__ __device__ constexpr int min_blocks(int q) { return q == 15 ? 8 : 7; }
 // 3 % (FP16) of a 256^3 step on GB300.
 constexpr bool kIntCvt = false;
 
-struct TileGeo {
-  int ntx, nty, T;  // tiles along x, along y, per plane
-};
+// The pair of thread tid in tile t of a plane: true if there is one.
+__device__ __forceinline__ bool tile_node(const TileMap &G, bool lin, const KParams &P, int t, int tid, int &x,
+                                          int &y) {
+  if (lin) {
+    const unsigned p = (unsigned)t * NTH + tid;
+    y = (int)__umulhi(p, G.m);
+    x = 2 * ((int)p - y * G.W);
+    return (int)p < G.M;
+  }
+  const int ty = t / G.ntx;
+  x = (t - ty * G.ntx) * 2 * TXP + 2 * (tid & (TXP - 1));
+  y = ty * kRows + tid / TXP;
+  return x < P.nx && y < P.ny;
+}
 
-__host__ __device__ inline TileGeo tile_geo(const KParams &P) {
-  TileGeo g;
-  g.ntx = (P.nx + 2 * TXP - 1) / (2 * TXP);
-  g.nty = (P.ny + kRows - 1) / kRows;
-  g.T = g.ntx * g.nty;
-  return g;
+// The tiles a psi job of tile t reads in planes z - 1, z, z + 1: lane's share
+// (dz, tile), false if it has none.  64 x 4 tiles: the 3 x 3 around it.  lin: all
+// tiles of the rows from one before its first to one after its last (a pair at
+// the end of a row reads the row's other end), at most kMaxLin of them, which
+// follow each other modulo T.
+constexpr int kMaxLin = 10;
+__host__ __device__ __forceinline__ bool dep_of_lane(const TileMap &G, bool lin, int t, int lane, int &dz,
+                                                               int &tile) {
+  if (lin) {
+    const int a = t * NTH, b = a + NTH < G.M ? a + NTH - 1 : G.M - 1;
+    const int ya = (int)(((unsigned long long)(unsigned)a * G.m) >> 32);
+    const int yb = (int)(((unsigned long long)(unsigned)b * G.m) >> 32);
+    int s = (ya - 1) * G.W, e = (yb + 2) * G.W - 1;
+    const bool all = e - s + 1 + NTH >= G.M;  // the range meets itself
+    if (s < 0) s += G.M;
+    if (e >= G.M) e -= G.M;
+    const int first = all ? 0 : s / NTH;
+    int cnt = all ? G.T : e / NTH - first + 1;
+    if (cnt <= 0) cnt += G.T;
+    dz = lane / kMaxLin - 1;
+    const int j = lane % kMaxLin;
+    tile = first + j;
+    if (tile >= G.T) tile -= G.T;
+    return dz <= 1 && j < cnt;
+  }
+  const int ty = t / G.ntx, tx = t - ty * G.ntx;
+  int xx = tx + lane % 3 - 1, yy = ty + (lane / 3) % 3 - 1;
+  xx = xx < 0 ? xx + G.ntx : (xx >= G.ntx ? xx - G.ntx : xx);
+  yy = yy < 0 ? yy + G.nty : (yy >= G.nty ? yy - G.nty : yy);
+  dz = lane / 9 - 1;
+  tile = yy * G.ntx + xx;
+  return lane < 27;
+}
+
+// Polls, by the lanes that have one, the counters of the fused jobs a psi job
+// reads until each shows `target`; false (on every lane) if one gave up.
+__device__ __forceinline__ bool wait_for_fused(const TileMap &G, bool lin, const KParams &P, const int *__restrict__ done,
+                                               int base, int count, int z, int t, int lane, int target) {
+  bool ok = true;
+  int dz, tile;
+  if (dep_of_lane(G, lin, t, lane, dz, tile)) {
+    int zz = z + dz;
+    zz = zz < 0 ? zz + P.nz : (zz >= P.nz ? zz - P.nz : zz);
+    const int *c = done + LBM_IDX(base + zz * G.T + tile, count);
+    for (int n = 0; counter_acquire(c) < target; ++n) {
+      if (n >= P.spin_limit) {
+        ok = false;
+        break;
+      }
+      __nanosleep(32);
+    }
+  }
+  return __all_sync(0xffffffffu, ok);
 }
 
 // The item claim number c of this launch names: gridDim.x + c.  Every launch
@@ -101,13 +160,13 @@ __device__ __forceinline__ int next_item(unsigned c, int nitems, unsigned &e) {
 }
 
 // item: x = fused plane (or -1), y = its tile, z = psi plane (or -1), w = its tile.
-// Q: 19 (both operators) or 15 (the D3Q15 non-orthogonal variant).
-template <typename S, int OP, bool SIGMA, int EOS, bool DF, int Q>
+// Q: 19 (both operators) or 15 (the D3Q15 non-orthogonal variant).  LIN: TileMap::lin.
+// The Eq. 16 term is compiled in (a zero coefficient switches it off).
+template <typename S, int OP, bool LIN, int EOS, bool DF, int Q>
 __global__ void __launch_bounds__(NTH, min_blocks(Q))
     queue_kernel(const S *__restrict__ g_in, S *__restrict__ g_out, const float *__restrict__ psi_in,
-                 float *__restrict__ psi_out, const KParams P, const int4 *__restrict__ items, int nitems,
-                 int *__restrict__ done, int stamp, unsigned *__restrict__ err) {
-  const TileGeo G = tile_geo(P);
+                 float *__restrict__ psi_out, const KParams P, const TileMap G, const int4 *__restrict__ items,
+                 int nitems, int *__restrict__ done, int stamp, unsigned *__restrict__ err) {
   const int lane = threadIdx.x, row = threadIdx.y;
   unsigned e = 0;
   // the claimed next item, by item parity: thread 0 writes slot i & 1 before item i's barrier and the block
@@ -126,12 +185,12 @@ __global__ void __launch_bounds__(NTH, min_blocks(Q))
     if (it.x >= 0) {
       int z = it.x, t = it.y;
       asm volatile("" : "+r"(z), "+r"(t));  // keep the row offsets out of the registers across items
-      const int x = (t % G.ntx) * 2 * TXP + 2 * lane, y = (t / G.ntx) * kRows + row;
-      if (x < P.nx && y < P.ny) {
+      int x, y;
+      if (tile_node(G, LIN, P, t, row * TXP + lane, x, y)) {
         if constexpr (Q == 15)
-          fused_pair15_at<S, SIGMA, true, false>(g_in, g_out, psi_in, P, x, y, z);
+          fused_pair15_at<S, true, true, false>(g_in, g_out, psi_in, P, x, y, z);
         else
-          fused_pair_at<S, OP, SIGMA, true, false>(g_in, g_out, psi_in, P, x, y, z, Rates<V2>(P));
+          fused_pair_at<S, OP, true, true, false>(g_in, g_out, psi_in, P, x, y, z, Rates<V2>(P));
       }
       if (lane == 0 && row == 0) s_next[par] = next_item(claim - base, nitems, e);
       __syncthreads();
@@ -145,26 +204,9 @@ __global__ void __launch_bounds__(NTH, min_blocks(Q))
     if (it.z >= 0) {
       int z = it.z, t = it.w;
       asm volatile("" : "+r"(z), "+r"(t));
-      const int tx = t % G.ntx, ty = t / G.ntx;
-      bool ok = true;
-      if (lane < 27) {  // fused jobs of planes z-1..z+1 on the 3 x 3 tiles around (tx, ty)
-        int zz = z + lane / 9 - 1, xx = tx + lane % 3 - 1, yy = ty + (lane / 3) % 3 - 1;
-        zz = zz < 0 ? zz + P.nz : (zz >= P.nz ? zz - P.nz : zz);
-        xx = xx < 0 ? xx + G.ntx : (xx >= G.ntx ? xx - G.ntx : xx);
-        yy = yy < 0 ? yy + G.nty : (yy >= G.nty ? yy - G.nty : yy);
-        const int *c = done + LBM_IDX(zz * G.T + yy * G.ntx + xx, P.nz * G.T);
-        const int target = stamp + P.wait_bias;
-        for (int n = 0; counter_acquire(c) < target; ++n) {
-          if (n >= P.spin_limit) {
-            ok = false;
-            break;
-          }
-          __nanosleep(32);
-        }
-      }
-      if (!__all_sync(0xffffffffu, ok)) e |= kErrTimeout;
-      const int x = tx * 2 * TXP + 2 * lane, y = ty * kRows + row;
-      if (x < P.nx && y < P.ny) {
+      if (!wait_for_fused(G, LIN, P, done, 0, P.nz * G.T, z, t, lane, stamp + P.wait_bias)) e |= kErrTimeout;
+      int x, y;
+      if (tile_node(G, LIN, P, t, row * TXP + lane, x, y)) {
         if constexpr (Q == 15)
           psi_pair15_at_l2<S, EOS, DF, kIntCvt, false>(g_out, psi_out, P, x, y, z, e);
         else
@@ -176,47 +218,48 @@ __global__ void __launch_bounds__(NTH, min_blocks(Q))
   if (e) atomicOr(err, e);
 }
 
-template <typename S, int OP, bool SIGMA, int EOS, bool DF, int Q>
+template <typename S, int OP, bool LIN, int EOS, bool DF, int Q>
 cudaError_t launch_kernel(const KParams &P, const void *g_in, void *g_out, const void *psi_in, void *psi_out,
                           const QueueState &q, int stamp, unsigned *err, cudaStream_t s) {
-  auto kern = queue_kernel<S, OP, SIGMA, EOS, DF, Q>;
+  auto kern = queue_kernel<S, OP, LIN, EOS, DF, Q>;
   const S *gi = (const S *)g_in;
   S *go = (S *)g_out;
   const float *pi = (const float *)psi_in;
   float *po = (float *)psi_out;
   KParams Pc = P;
+  TileMap G = tile_map(P);
   const int4 *items = q.items;
   int nitems = q.nitems, *done = q.done;
-  void *args[] = {(void *)&gi,    (void *)&go,     (void *)&pi,   (void *)&po,    (void *)&Pc,
+  void *args[] = {(void *)&gi,    (void *)&go,     (void *)&pi,   (void *)&po,    (void *)&Pc,   (void *)&G,
                   (void *)&items, (void *)&nitems, (void *)&done, (void *)&stamp, (void *)&err};
   return cudaLaunchCooperativeKernel((const void *)kern, dim3(q.grid), dim3(TXP, kRows), args, 0, s);
 }
 
-template <typename S, int OP, bool SIGMA, int Q = 19>
+template <typename S, int OP, bool LIN, int Q = 19>
 cudaError_t by_eos(const KParams &P, bool df, const void *g_in, void *g_out, const void *psi_in, void *psi_out,
                    const QueueState &q, int stamp, unsigned *err, cudaStream_t s) {
   switch (P.eos) {
     case kEosCS:
-      return df ? launch_kernel<S, OP, SIGMA, kEosCS, true, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
-                : launch_kernel<S, OP, SIGMA, kEosCS, false, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
+      return df ? launch_kernel<S, OP, LIN, kEosCS, true, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
+                : launch_kernel<S, OP, LIN, kEosCS, false, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
     case kEosExp:
-      return df ? launch_kernel<S, OP, SIGMA, kEosExp, true, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
-                : launch_kernel<S, OP, SIGMA, kEosExp, false, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
+      return df ? launch_kernel<S, OP, LIN, kEosExp, true, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
+                : launch_kernel<S, OP, LIN, kEosExp, false, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
     default:
-      return launch_kernel<S, OP, SIGMA, kEosNone, false, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
+      return launch_kernel<S, OP, LIN, kEosNone, false, Q>(P, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
   }
 }
 
 template <typename S>
-cudaError_t by_op(const KParams &P, int op, bool sigma, bool df, const void *g_in, void *g_out, const void *psi_in,
+cudaError_t by_op(const KParams &P, int op, bool lin, bool df, const void *g_in, void *g_out, const void *psi_in,
                   void *psi_out, const QueueState &q, int stamp, unsigned *err, cudaStream_t s) {
   if (P.q == 15)
-    return sigma ? by_eos<S, kNonOrth, true, 15>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
+    return lin ? by_eos<S, kNonOrth, true, 15>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
                  : by_eos<S, kNonOrth, false, 15>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
   if (op == kNonOrth)
-    return sigma ? by_eos<S, kNonOrth, true>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
+    return lin ? by_eos<S, kNonOrth, true>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
                  : by_eos<S, kNonOrth, false>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
-  return sigma ? by_eos<S, kOrth, true>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
+  return lin ? by_eos<S, kOrth, true>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s)
                : by_eos<S, kOrth, false>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
 }
 
@@ -225,7 +268,8 @@ cudaError_t by_op(const KParams &P, int op, bool sigma, bool df, const void *g_i
 // launch of that many blocks per SM fits whichever one runs.
 template <typename S>
 cudaError_t occupancy_of(int q, int *per_sm) {
-  using K = void (*)(const S *, S *, const float *, float *, const KParams, const int4 *, int, int *, int, unsigned *);
+  using K = void (*)(const S *, S *, const float *, float *, const KParams, const TileMap, const int4 *, int, int *, int,
+                     unsigned *);
   const K k19[] = {queue_kernel<S, kNonOrth, true, kEosCS, false, 19>, queue_kernel<S, kOrth, true, kEosCS, false, 19>,
                    queue_kernel<S, kNonOrth, false, kEosCS, true, 19>, queue_kernel<S, kOrth, false, kEosExp, false, 19>};
   const K k15[] = {queue_kernel<S, kNonOrth, true, kEosCS, false, 15>, queue_kernel<S, kNonOrth, false, kEosExp, true, 15>};
@@ -248,29 +292,7 @@ cudaError_t occupancy_of(int q, int *per_sm) {
 // buffered), so it is there when the item starts; a fused job of box B
 // reads level in = B.cur ^ parity and writes in ^ 1, the psi job evaluates psi
 // of level in ^ 1.  Both operators and the Eq. 16 term (zero coefficient when
-// off) are compiled in.  Tiles are tw x (256 / tw) nodes, tw = 64, 32 or 16 per
-// box (batch_tile_width): 128 threads, one node pair each, and on the small
-// boxes of a batch (edges 32, 48, 96, ...) no idle half tiles.
-struct BatchGeo {
-  int tw, th, ntx, nty, T;  // tile width and height, tiles along x and y, per plane
-};
-
-__host__ __device__ inline BatchGeo batch_geo(const KParams &P, int tw) {
-  BatchGeo g;
-  g.tw = tw;
-  g.th = 2 * NTH / tw;
-  g.ntx = (P.nx + tw - 1) / tw;
-  g.nty = (P.ny + g.th - 1) / g.th;
-  g.T = g.ntx * g.nty;
-  return g;
-}
-
-// Tile row of tile t of a box: t / ntx by a multiply with the descriptor's
-// ceil(2^32 / ntx) instead of a division (exact for t * ntx < 2^32).
-__device__ __forceinline__ int tile_row(int t, const BatchBox &B) {
-  return (int)(((unsigned long long)(unsigned)t * B.ntx_m) >> 32);
-}
-
+// off) are compiled in.
 // Copy box descriptors to shared memory with asynchronous 16-byte copies (one
 // commit group per call), so that the next item's descriptors arrive while the
 // current item runs.
@@ -319,9 +341,8 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
       int z = (int)((unsigned)it.y & 0xffffu), t = (int)((unsigned)it.y >> 16);
       asm volatile("" : "+r"(z), "+r"(t));
       const int in = B.cur ^ parity;
-      const int ty = tile_row(t, B), tx = t - ty * B.ntx;
-      const int x = tx * B.tw + 2 * (tid & ((1 << B.hshift) - 1)), y = ty * B.th + (tid >> B.hshift);
-      if (x < P.nx && y < P.ny) {
+      int x, y;
+      if (tile_node(B.map, B.map.lin, P, t, tid, x, y)) {
         const S *gi = (const S *)B.g[in];
         S *go = (S *)B.g[in ^ 1];
         if (B.op == kNonOrth)
@@ -330,7 +351,7 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
           fused_pair_at<S, kOrth, true, false, ODD>(gi, go, B.psi[in], P, x, y, z, Rates<V2>(P));
       }
       __syncthreads();
-      if (tid == 0) counter_release_add(done + LBM_IDX(B.qbase + z * B.T + t, ndone), 1);
+      if (tid == 0) counter_release_add(done + LBM_IDX(B.qbase + z * B.map.T + t, ndone), 1);
     }
     if (threadIdx.y == 0) {  // the next item and its descriptors (buffer (i + 1) & 1 was item i - 1's)
       const int kn = (int)min((unsigned)gridDim.x + __shfl_sync(0xffffffffu, claim, 0), (unsigned)nitems);
@@ -346,27 +367,12 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
       const KParams &P = B.P;
       int z = (int)((unsigned)it.w & 0xffffu), t = (int)((unsigned)it.w >> 16);
       asm volatile("" : "+r"(z), "+r"(t));
-      const int ty = tile_row(t, B), tx = t - ty * B.ntx, lane = threadIdx.x;
-      bool ok = true;
-      if (lane < 27) {  // fused jobs of planes z-1..z+1 on the 3 x 3 tiles around (tx, ty)
-        int zz = z + lane / 9 - 1, xx = tx + lane % 3 - 1, yy = ty + (lane / 3) % 3 - 1;
-        zz = zz < 0 ? zz + P.nz : (zz >= P.nz ? zz - P.nz : zz);
-        xx = xx < 0 ? xx + B.ntx : (xx >= B.ntx ? xx - B.ntx : xx);
-        yy = yy < 0 ? yy + B.nty : (yy >= B.nty ? yy - B.nty : yy);
-        const int *c = done + LBM_IDX(B.qbase + zz * B.T + yy * B.ntx + xx, ndone);
-        const int target = 1 + P.wait_bias;  // counters are cleared before every launch
-        for (int n = 0; counter_acquire(c) < target; ++n) {
-          if (n >= P.spin_limit) {
-            ok = false;
-            break;
-          }
-          __nanosleep(32);
-        }
-      }
-      if (!__all_sync(0xffffffffu, ok)) e |= kErrTimeout;
+      // counters are cleared before every launch
+      if (!wait_for_fused(B.map, B.map.lin, P, done, B.qbase, ndone, z, t, threadIdx.x, 1 + P.wait_bias)) e |= kErrTimeout;
       const int in = B.cur ^ parity;
-      const int x = tx * B.tw + 2 * (tid & ((1 << B.hshift) - 1)), y = ty * B.th + (tid >> B.hshift);
-      if (x < P.nx && y < P.ny) psi_pair_at_l2<S, EOS, false, kIntCvt, ODD>((const S *)B.g[in ^ 1], B.psi[in ^ 1], P, x, y, z, e);
+      int x, y;
+      if (tile_node(B.map, B.map.lin, P, t, tid, x, y))
+        psi_pair_at_l2<S, EOS, false, kIntCvt, ODD>((const S *)B.g[in ^ 1], B.psi[in ^ 1], P, x, y, z, e);
     }
     __syncthreads();  // s_next and s_it are written; rewritten only after the next item's first barrier
     k = s_next;
@@ -396,14 +402,21 @@ cudaError_t batch_by_eos(int eos, const BatchBox *boxes, const int4 *items, int 
   }
 }
 
+// The psi jobs in order of the last fused job they read (stable).
+std::vector<long long> by_ready(const std::vector<long long> &ready) {
+  std::vector<long long> start(ready.size() + 1, 0), order(ready.size());
+  for (long long r : ready) ++start[r + 1];
+  for (size_t k = 1; k < start.size(); ++k) start[k] += start[k - 1];
+  for (size_t p = 0; p < ready.size(); ++p) order[start[ready[p]]++] = (long long)p;
+  return order;
+}
+
 // Psi jobs go to the first free item at least `lag` items after the last of
 // the fused jobs they read (ready[]); fused job j sits in item j.  Checks the
 // result as the single-box list does.
 bool place_psi_jobs(std::vector<int4> &out, const std::vector<long long> &ready, const std::vector<int2> &job,
                     long long nf, long long lag) {
-  std::vector<long long> order((size_t)nf);
-  for (long long p = 0; p < nf; ++p) order[p] = p;
-  std::stable_sort(order.begin(), order.end(), [&](long long a, long long b) { return ready[a] < ready[b]; });
+  const std::vector<long long> order = by_ready(ready);
   long long next = 0;
   for (long long p : order) {
     const long long k = std::max(next, ready[p] + lag);
@@ -416,6 +429,49 @@ bool place_psi_jobs(std::vector<int4> &out, const std::vector<long long> &ready,
 }
 
 }  // namespace
+
+// 128 consecutive pairs of the plane leave no lane idle and start on a sector
+// wherever the row does, whatever Nx is; 64 x 4 tiles leave lanes idle where Nx
+// is no multiple of 64 or Ny of 4 (80 x 80: 38 %, 200 x 180: 22 %), and tiles
+// narrowed to 16 nodes start off a 32-byte sector in most rows.  They are also
+// the faster ones where 64 x 4 fits: per step, 64 x 4 / consecutive, 80^3 36.9 /
+// 25.5 us, 160^3 184 / 136, 192^3 259 / 220, 200 x 180 x 256 (orthogonal) 379 /
+// 304, 256^3 530 / 518; a batch of six boxes of edges 62 to 140 314 / 257 (16-
+// and 32-node tiles: 301).  A psi job then waits for whole rows around its
+// tile; past 512 nodes a row that is more tiles than a warp has lanes to poll
+// with, and the 64 x 4 tiles take over.
+TileMap tile_map(const KParams &P) {
+  TileMap G{};
+  G.W = P.px / 2;
+  G.M = G.W * P.ny;
+  G.ntx = (P.nx + 2 * TXP - 1) / (2 * TXP);
+  G.nty = (P.ny + kRows - 1) / kRows;
+  const long long rows = NTH / G.W + 4;  // rows a psi job of a tile of consecutive pairs reads, at most
+  if (P.px % 2 == 0 && (rows * G.W + NTH - 1) / NTH + 2 <= kMaxLin && (long long)G.M * G.W < (1LL << 32)) {
+    G.lin = 1;
+    G.T = (G.M + NTH - 1) / NTH;
+    G.m = (unsigned)(((1ull << 32) + G.W - 1) / G.W);
+  } else {
+    G.T = G.ntx * G.nty;
+  }
+  return G;
+}
+
+// For every tile, the last of the tiles a psi job of it reads in a plane.
+static std::vector<int> last_tiles(const TileMap &G) {
+  std::vector<int> last((size_t)G.T, 0);
+  for (int t = 0; t < G.T; ++t)
+    for (int lane = 0; lane < 32; ++lane) {
+      int dz, tile;
+      if (dep_of_lane(G, G.lin != 0, t, lane, dz, tile)) last[t] = std::max(last[t], tile);
+    }
+  return last;
+}
+// Position (z T + tile) of the last fused job that psi job (z, t) reads: in
+// plane z + 1, or in the last plane where the box wraps.
+static long long last_read(const TileMap &G, const std::vector<int> &last, int nz, int z, int t) {
+  return (long long)(z == 0 || z == nz - 1 ? nz - 1 : z + 1) * G.T + last[t];
+}
 
 bool queue_supported(const KParams &P, int precision) { return precision != kF64 && P.nx % 2 == 0; }
 
@@ -430,31 +486,22 @@ cudaError_t queue_grid(int precision, int q, int *grid) {
   return cudaSuccess;
 }
 
-size_t queue_counters(const KParams &P) { return (size_t)P.nz * tile_geo(P).T + 32; }  // + the claim counter
+size_t queue_counters(const KParams &P) { return (size_t)P.nz * tile_map(P).T + 32; }  // + the claim counter
 
 bool queue_items(const KParams &P, int grid, std::vector<int4> &out) {
-  const TileGeo G = tile_geo(P);
+  const TileMap G = tile_map(P);
   const long long nf = (long long)P.nz * G.T;
   if (P.nz < 3 || grid < 1 || nf >= (1LL << 30)) return false;
   // fused job j = (j / T, j % T); psi job (z, t) is ready after the last of the
-  // 27 fused jobs it reads and goes to the first free item >= ready + lag, half
+  // fused jobs it reads and goes to the first free item >= ready + lag, half
   // a wave of the grid later (at least one item)
   const long long lag = std::max(1, grid / 2);
+  const std::vector<int> last = last_tiles(G);
   std::vector<long long> ready((size_t)nf);
   for (long long p = 0; p < nf; ++p) {
-    const int z = (int)(p / G.T), t = (int)(p % G.T), tx = t % G.ntx, ty = t / G.ntx;
-    long long r = -1;
-    for (int dz = -1; dz <= 1; ++dz)
-      for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int zz = (z + dz + P.nz) % P.nz, yy = (ty + dy + G.nty) % G.nty, xx = (tx + dx + G.ntx) % G.ntx;
-          r = std::max(r, (long long)zz * G.T + yy * G.ntx + xx);
-        }
-    ready[p] = r;
+    ready[p] = last_read(G, last, P.nz, (int)(p / G.T), (int)(p % G.T));
   }
-  std::vector<long long> order((size_t)nf);
-  for (long long p = 0; p < nf; ++p) order[p] = p;
-  std::stable_sort(order.begin(), order.end(), [&](long long a, long long b) { return ready[a] < ready[b]; });
+  const std::vector<long long> order = by_ready(ready);
   out.assign((size_t)nf, make_int4(-1, -1, -1, -1));
   for (long long j = 0; j < nf; ++j) out[j] = make_int4((int)(j / G.T), (int)(j % G.T), -1, -1);
   long long next = 0;  // first item that may still take a psi job
@@ -487,36 +534,13 @@ bool queue_items(const KParams &P, int grid, std::vector<int4> &out) {
   return true;
 }
 
-cudaError_t launch_queue(const KParams &P, int precision, int op, bool sigma, bool df, const void *g_in, void *g_out,
+cudaError_t launch_queue(const KParams &P, int precision, int op, bool df, const void *g_in, void *g_out,
                          const void *psi_in, void *psi_out, const QueueState &q, int stamp, unsigned *err,
                          cudaStream_t s) {
   if (!queue_supported(P, precision)) return cudaErrorInvalidValue;
-  if (precision == kF32) return by_op<float>(P, op, sigma, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
-  return by_op<__half>(P, op, sigma, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
-}
-
-int batch_tile_width(int nx) {
-  // the widest of 64, 32, 16 with the fewest idle columns in the last tile
-  int best = 64;
-  long long waste = (long long)(nx + 63) / 64 * 64 - nx;
-  for (int tw : {32, 16}) {
-    const long long w = (long long)(nx + tw - 1) / tw * tw - nx;
-    if (w < waste) best = tw, waste = w;
-  }
-  return best;
-}
-
-int batch_queue_tiles(const KParams &P) { return batch_geo(P, batch_tile_width(P.nx)).T; }
-
-void batch_queue_geometry(BatchBox &d) {
-  d.tw = batch_tile_width(d.P.nx);
-  const BatchGeo G = batch_geo(d.P, d.tw);
-  d.ntx = G.ntx;
-  d.nty = G.nty;
-  d.T = G.T;
-  d.th = G.th;
-  d.hshift = d.tw == 64 ? 5 : (d.tw == 32 ? 4 : 3);  // log2 of the node pairs across a tile
-  d.ntx_m = ((1ull << 32) + (unsigned long long)G.ntx - 1) / (unsigned long long)G.ntx;
+  const bool lin = tile_map(P).lin != 0;
+  if (precision == kF32) return by_op<float>(P, op, lin, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
+  return by_op<__half>(P, op, lin, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
 }
 
 bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std::vector<int4> &out,
@@ -526,7 +550,7 @@ bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std:
   base.assign(boxes.size(), 0);
   for (size_t b = 0; b < boxes.size(); ++b) {
     const KParams &P = *boxes[b];
-    const BatchGeo G = batch_geo(P, batch_tile_width(P.nx));
+    const TileMap G = tile_map(P);
     if (P.nz < 3 || P.px % 2 != 0 || P.nz > 0xffff || G.T > 0xffff || grid < 1) return false;
     first[b + 1] = first[b] + (long long)P.nz * G.T;
     if (first[b + 1] >= (1LL << 30)) return false;
@@ -539,22 +563,15 @@ bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std:
   std::vector<int2> job((size_t)nf);  // (box, z | tile << 16) of psi job p (same numbering as fused job p)
   for (size_t b = 0; b < boxes.size(); ++b) {
     const KParams &P = *boxes[b];
-    const BatchGeo G = batch_geo(P, batch_tile_width(P.nx));
+    const TileMap G = tile_map(P);
+    const std::vector<int> last = last_tiles(G);
     for (int z = 0; z < P.nz; ++z)
       for (int t = 0; t < G.T; ++t) {
         const long long j = first[b] + (long long)z * G.T + t;
         const int zt = (int)((unsigned)z | ((unsigned)t << 16));
         out[j] = make_int4((int)b, zt, -1, -1);
         job[j] = make_int2((int)b, zt);
-        const int tx = t % G.ntx, ty = t / G.ntx;
-        long long r = -1;
-        for (int dz = -1; dz <= 1; ++dz)
-          for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-              const int zz = (z + dz + P.nz) % P.nz, yy = (ty + dy + G.nty) % G.nty, xx = (tx + dx + G.ntx) % G.ntx;
-              r = std::max(r, first[b] + (long long)zz * G.T + yy * G.ntx + xx);
-            }
-        ready[j] = r;
+        ready[j] = first[b] + last_read(G, last, P.nz, z, t);
       }
   }
   if (!place_psi_jobs(out, ready, job, nf, std::max(1, grid / 2))) return false;
@@ -568,7 +585,7 @@ bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std:
       if (b >= (int)boxes.size()) return false;
       const unsigned zt = (unsigned)(side ? it.w : it.y);
       const int z = (int)(zt & 0xffffu), t = (int)(zt >> 16);
-      const BatchGeo G = batch_geo(*boxes[b], batch_tile_width(boxes[b]->nx));
+      const TileMap G = tile_map(*boxes[b]);
       if (z >= boxes[b]->nz || t >= G.T) return false;
       const long long j = first[b] + (long long)z * G.T + t;
       if (!side) {
