@@ -16,6 +16,17 @@
 
 namespace lbm {
 
+// ------------------------------------------------------------------ chained launches
+// First statement of a kernel launched by launch_chained: lets the next
+// launch's blocks in (they come only once every block of this grid has started)
+// and waits until the grid before this one has completed and its writes are
+// visible.  Every such kernel waits, so a grid completes only after all before
+// it: what it overwrites has been read.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ------------------------------------------------------------------ addressing
 // Periodic neighbours of a node and the row offsets (y, z part of the index)
 // of the nine (y', z') combinations a D3Q19 stencil touches.

@@ -89,6 +89,7 @@ template <int PREC, int EOS, bool DF, int Q>
 __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S *__restrict__ g,
                                                   typename Types<PREC>::Psi *__restrict__ psi,
                                                   const KParams P, unsigned *__restrict__ err) {
+  chain_wait();
   using S = typename Types<PREC>::S;
   using T = typename Types<PREC>::T;
   int x, y, z;
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
                                                     typename Types<PREC>::S *__restrict__ g_out,
                                                     const typename Types<PREC>::Psi *__restrict__ psi,
                                                     const KParams P, const Coeffs64 C) {
+  chain_wait();
   using S = typename Types<PREC>::S;
   using T = typename Types<PREC>::T;
   int x, y, z;
@@ -515,16 +517,12 @@ cudaError_t psi_dispatch(const KParams &P, const void *g, void *psi, unsigned *e
   const dim3 grid = node_grid(P, L), block(L.bx, L.by);
   switch (P.eos) {
     case kEosCS:
-      psi_kernel<PREC, kEosCS, DF, Q><<<grid, block, 0, L.stream>>>((const S *)g, (Psi *)psi, P, err);
-      break;
+      return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosCS, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
     case kEosExp:
-      psi_kernel<PREC, kEosExp, DF, Q><<<grid, block, 0, L.stream>>>((const S *)g, (Psi *)psi, P, err);
-      break;
+      return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosExp, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
     default:
-      psi_kernel<PREC, kEosNone, DF, Q><<<grid, block, 0, L.stream>>>((const S *)g, (Psi *)psi, P, err);
-      break;
+      return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosNone, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
   }
-  return cudaGetLastError();
 }
 
 template <int PREC, int OP, int Q>
@@ -539,11 +537,8 @@ cudaError_t fused_dispatch(const KParams &P, bool sigma, const void *g_in, void 
   if (PREC == kF64) Lf.by = 1;
   const dim3 grid = node_grid(P, Lf), block(Lf.bx, Lf.by);
   const Coeffs64 C = coeffs64(P, Q == 15 ? kNonOrthQ15 : OP);
-  if (sigma)
-    fused_kernel<PREC, OP, true, Q><<<grid, block, 0, L.stream>>>((const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
-  else
-    fused_kernel<PREC, OP, false, Q><<<grid, block, 0, L.stream>>>((const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
-  return cudaGetLastError();
+  return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), sigma ? fused_kernel<PREC, OP, true, Q> : fused_kernel<PREC, OP, false, Q>, grid, block, L.stream,
+                        (const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
 }
 
 }  // namespace

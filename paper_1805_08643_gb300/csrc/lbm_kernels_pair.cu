@@ -60,6 +60,7 @@ __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int 
 template <typename S, int EOS, bool DF>
 __global__ void __launch_bounds__(128) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                        const KParams P, unsigned *__restrict__ err) {
+  chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
@@ -74,6 +75,7 @@ __global__ void __launch_bounds__(128) psi_pair_kernel(const S *__restrict__ g, 
 template <typename S, int OP, bool SIGMA, bool ODD>
 __global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                          const float *__restrict__ psi, const KParams P) {
+  chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
@@ -92,6 +94,7 @@ __global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g
 template <typename S, int EOS, bool DF>
 __global__ void __launch_bounds__(128) psi_pair15_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                          const KParams P, unsigned *__restrict__ err) {
+  chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
@@ -106,6 +109,7 @@ __global__ void __launch_bounds__(128) psi_pair15_kernel(const S *__restrict__ g
 template <typename S, bool SIGMA, bool ODD>
 __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                            const float *__restrict__ psi, const KParams P) {
+  chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
@@ -123,18 +127,16 @@ cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsign
   float *pp = (float *)psi;
   if (P.q == 15) {
     switch (P.eos) {
-      case kEosCS: psi_pair15_kernel<S, kEosCS, DF><<<grid, block, 0, L.stream>>>(gg, pp, P, err); break;
-      case kEosExp: psi_pair15_kernel<S, kEosExp, DF><<<grid, block, 0, L.stream>>>(gg, pp, P, err); break;
-      default: psi_pair15_kernel<S, kEosNone, false><<<grid, block, 0, L.stream>>>(gg, pp, P, err); break;
+      case kEosCS: return launch_chained(P.n >= kChainPairs, psi_pair15_kernel<S, kEosCS, DF>, grid, block, L.stream, gg, pp, P, err);
+      case kEosExp: return launch_chained(P.n >= kChainPairs, psi_pair15_kernel<S, kEosExp, DF>, grid, block, L.stream, gg, pp, P, err);
+      default: return launch_chained(P.n >= kChainPairs, psi_pair15_kernel<S, kEosNone, false>, grid, block, L.stream, gg, pp, P, err);
     }
-    return cudaGetLastError();
   }
   switch (P.eos) {
-    case kEosCS: psi_pair_kernel<S, kEosCS, DF><<<grid, block, 0, L.stream>>>(gg, pp, P, err); break;
-    case kEosExp: psi_pair_kernel<S, kEosExp, DF><<<grid, block, 0, L.stream>>>(gg, pp, P, err); break;
-    default: psi_pair_kernel<S, kEosNone, false><<<grid, block, 0, L.stream>>>(gg, pp, P, err); break;
+    case kEosCS: return launch_chained(P.n >= kChainPairs, psi_pair_kernel<S, kEosCS, DF>, grid, block, L.stream, gg, pp, P, err);
+    case kEosExp: return launch_chained(P.n >= kChainPairs, psi_pair_kernel<S, kEosExp, DF>, grid, block, L.stream, gg, pp, P, err);
+    default: return launch_chained(P.n >= kChainPairs, psi_pair_kernel<S, kEosNone, false>, grid, block, L.stream, gg, pp, P, err);
   }
-  return cudaGetLastError();
 }
 
 template <typename S, bool ODD>
@@ -144,17 +146,11 @@ cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void
   const S *gi = (const S *)g_in;
   S *go = (S *)g_out;
   const float *pp = (const float *)psi;
-  if (P.q == 15) {
-    if (sigma) fused_pair15_kernel<S, true, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-    else fused_pair15_kernel<S, false, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-  } else if (op == kNonOrth) {
-    if (sigma) fused_pair_kernel<S, kNonOrth, true, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-    else fused_pair_kernel<S, kNonOrth, false, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-  } else {
-    if (sigma) fused_pair_kernel<S, kOrth, true, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-    else fused_pair_kernel<S, kOrth, false, ODD><<<grid, block, 0, L.stream>>>(gi, go, pp, P);
-  }
-  return cudaGetLastError();
+  auto run = [&](auto kernel) { return launch_chained(P.n >= kChainPairs, kernel, grid, block, L.stream, gi, go, pp, P); };
+  if (P.q == 15) return sigma ? run(fused_pair15_kernel<S, true, ODD>) : run(fused_pair15_kernel<S, false, ODD>);
+  if (op == kNonOrth)
+    return sigma ? run(fused_pair_kernel<S, kNonOrth, true, ODD>) : run(fused_pair_kernel<S, kNonOrth, false, ODD>);
+  return sigma ? run(fused_pair_kernel<S, kOrth, true, ODD>) : run(fused_pair_kernel<S, kOrth, false, ODD>);
 }
 
 // Batched boxes, two-pass step, psi pass: work item w = (box, tile_x | tile_y
