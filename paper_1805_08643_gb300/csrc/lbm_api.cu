@@ -240,8 +240,6 @@ lbm_status lbm_create(const int grid[3], const lbm_eos *eos, double G, const lbm
   c->op = op;
   c->sigma_on = sigma != 0.0;
   c->L.stream = (cudaStream_t)cuda_stream;
-  c->L.bx = 32;
-  c->L.by = 4;
   // the default step: the work-list single pass where it applies and is the
   // faster one on GB300 (FP32 storage: it moves 160 instead of 236 bytes per
   // node and overlaps the FP64 EOS with the population stream), else the
@@ -704,6 +702,8 @@ bool fill_params(const int grid[3], const lbm_eos *eos, double G, const lbm_rate
   P.n = (int)n;
   P.px = stored_row(precision, grid);
   P.np = (int)((long long)P.px * grid[1] * grid[2]);
+  P.row_m = row_multiplier(P.nx, (long long)P.nx * grid[1]);
+  P.pair_m = row_multiplier(P.px / 2, (long long)(P.px / 2) * grid[1]);
   P.q = op == LBM_OP_NONORTHOGONAL_D3Q15 ? 15 : 19;
   P.G = eos->kind == LBM_EOS_NONE ? 0.0 : G;
   P.half_force = -0.5 * P.G / (P.q == 15 ? 24.0 : 12.0);

@@ -299,8 +299,6 @@ HostBox *get_box(lbm_batch *b, int id) {
 lbm::Launch launch_of(lbm_batch *b) {
   lbm::Launch L;
   L.stream = b->stream;
-  L.bx = 32;
-  L.by = 4;
   return L;
 }
 

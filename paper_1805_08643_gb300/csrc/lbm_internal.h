@@ -28,6 +28,9 @@ struct KParams {
   // its first (the periodic neighbour of node nx - 1), kept by whoever writes
   // node 0.  Arrays of the public interface (rho, u, f) have rows of nx.
   int px, np;
+  // ceil(2^32 / nx), ceil(2^32 / (px / 2)): a plane's node or pair p lies in row (p m) >> 32; 0 (planes too large
+  // for that): divide
+  unsigned row_m, pair_m;
   int q;             // lattice: 19 (D3Q19, both operators) or 15 (D3Q15 non-orthogonal)
   double G;          // interaction strength, Eq. 15
   double half_force; // -G/2 times the diagonal (D3Q15: corner) weight of Eq. 15, 1/12 (1/24)
@@ -67,6 +70,11 @@ struct KParams {
   int wait_bias;
 };
 
+// ceil(2^32 / d) if (v m) >> 32 is v / d for every v < count, else 0.
+inline unsigned row_multiplier(long long d, long long count) {
+  return d >= 2 && count * d < (1LL << 32) ? (unsigned)(((1ull << 32) + d - 1) / d) : 0u;
+}
+
 // KParams::px of a box: rows of an odd nx get one element more where the
 // two-node kernels run, unless that leaves the index range (19 np < 2^32).
 inline int stored_row(int precision, const int grid[3]) {
@@ -101,8 +109,17 @@ struct DropletChunk {
 
 struct Launch {
   cudaStream_t stream;
-  int bx, by;  // thread-block shape (x, y) of the per-node kernels
 };
+
+// Threads per block of the per-node and per-pair kernels.  A block takes as many
+// consecutive nodes (pairs) of a plane in row order: blocks of 32 x 4 nodes left
+// lanes idle where Nx is no multiple of 32 (pairs: 64), which the kernels bound
+// by the FP64 unit pay in full (72^3 FP64 step 242 -> 187 us, 72^3
+// FP16 20.9 -> 13.4, 65^3 FP32 18.9 -> 14.8).
+constexpr int kThreads = 128;
+inline dim3 plane_grid(int per_plane, int nz, int threads = kThreads) {
+  return dim3((unsigned)((per_plane + threads - 1) / threads), 1, (unsigned)nz);
+}
 
 // Launch of a kernel of the two-pass step that may start while its predecessor
 // in the stream is ending (programmatic stream serialization): its blocks take

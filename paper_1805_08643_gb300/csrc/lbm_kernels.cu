@@ -78,10 +78,11 @@ __device__ __forceinline__ void store_node(S *__restrict__ g, int a, const KPara
 }
 
 __device__ __forceinline__ bool node_of_thread(const KParams &P, int &x, int &y, int &z) {
-  x = blockIdx.x * blockDim.x + threadIdx.x;
-  y = blockIdx.y * blockDim.y + threadIdx.y;
+  const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
+  y = (int)(P.row_m ? __umulhi(p, P.row_m) : p / (unsigned)P.nx);
+  x = (int)p - y * P.nx;
   z = blockIdx.z;
-  return x < P.nx && y < P.ny;
+  return y < P.ny;
 }
 
 // ------------------------------------------------------------------ psi pass
@@ -506,15 +507,13 @@ __global__ void set_populations_kernel(const double *__restrict__ f, typename Ty
     }
 }
 
-dim3 node_grid(const KParams &P, const Launch &L) {
-  return dim3((P.nx + L.bx - 1) / L.bx, (P.ny + L.by - 1) / L.by, P.nz);
-}
+dim3 node_grid(const KParams &P, int threads = kThreads) { return plane_grid(P.nx * P.ny, P.nz, threads); }
 
 template <int PREC, bool DF, int Q>
 cudaError_t psi_dispatch(const KParams &P, const void *g, void *psi, unsigned *err, const Launch &L) {
   using S = typename Types<PREC>::S;
   using Psi = typename Types<PREC>::Psi;
-  const dim3 grid = node_grid(P, L), block(L.bx, L.by);
+  const dim3 grid = node_grid(P), block(kThreads);
   switch (P.eos) {
     case kEosCS:
       return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosCS, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
@@ -533,9 +532,8 @@ cudaError_t fused_dispatch(const KParams &P, bool sigma, const void *g_in, void 
   // FP64: blocks of one warp.  Every warp holds the SM's FP64 unit for the same time, so the last round is
   // shortest when warps are dealt out singly: 32^3 steps 28.7 -> 26.7 us (orthogonal; blocks of four warps
   // leave 8 on some SMs, single ones 7), no difference from 64^3 on.
-  Launch Lf = L;
-  if (PREC == kF64) Lf.by = 1;
-  const dim3 grid = node_grid(P, Lf), block(Lf.bx, Lf.by);
+  constexpr int threads = PREC == kF64 ? 32 : kThreads;
+  const dim3 grid = node_grid(P, threads), block(threads);
   const Coeffs64 C = coeffs64(P, Q == 15 ? kNonOrthQ15 : OP);
   return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), sigma ? fused_kernel<PREC, OP, true, Q> : fused_kernel<PREC, OP, false, Q>, grid, block, L.stream,
                         (const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
@@ -607,7 +605,7 @@ cudaError_t launch_fused(const KParams &P, int precision, int op, bool sigma, co
 
 cudaError_t launch_moments(const KParams &P, int precision, const void *g, const void *psi, double *rho,
                            double *u, const Launch &L) {
-  const dim3 grid = node_grid(P, L), block(L.bx, L.by);
+  const dim3 grid = node_grid(P), block(kThreads);
   LBM_PREC_SWITCH(precision, (moments_kernel<PR, QQ><<<grid, block, 0, L.stream>>>(
                                  (const typename Types<PR>::S *)g, (const typename Types<PR>::Psi *)psi, P, rho, u)));
   return cudaGetLastError();
@@ -634,19 +632,19 @@ cudaError_t launch_max_du(const KParams &P, int precision, const void *g, const 
 
 cudaError_t launch_rho_droplets(const KParams &P, double *rho, const DropletChunk &chunk, double W,
                                 double rho_l, double rho_v, bool first, const Launch &L) {
-  rho_droplets_kernel<<<node_grid(P, L), dim3(L.bx, L.by), 0, L.stream>>>(rho, P, chunk, W, rho_l, rho_v,
+  rho_droplets_kernel<<<node_grid(P), kThreads, 0, L.stream>>>(rho, P, chunk, W, rho_l, rho_v,
                                                                            first ? 1 : 0);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rho_slab(const KParams &P, double *rho, int axis, double lo, double hi, double W,
                             double rho_l, double rho_v, const Launch &L) {
-  rho_slab_kernel<<<node_grid(P, L), dim3(L.bx, L.by), 0, L.stream>>>(rho, P, axis, lo, hi, W, rho_l, rho_v);
+  rho_slab_kernel<<<node_grid(P), kThreads, 0, L.stream>>>(rho, P, axis, lo, hi, W, rho_l, rho_v);
   return cudaGetLastError();
 }
 
 cudaError_t launch_state_from_rho(const KParams &P, int precision, const double *rho, void *g, const Launch &L) {
-  const dim3 grid = node_grid(P, L), block(L.bx, L.by);
+  const dim3 grid = node_grid(P), block(kThreads);
   LBM_PREC_SWITCH(precision, (state_from_rho_kernel<PR, QQ><<<grid, block, 0, L.stream>>>(
                                  rho, (typename Types<PR>::S *)g, P)));
   return cudaGetLastError();
@@ -654,7 +652,7 @@ cudaError_t launch_state_from_rho(const KParams &P, int precision, const double 
 
 cudaError_t launch_get_populations(const KParams &P, int precision, const void *g, double *out, int a_lo,
                                    int a_hi, const Launch &L) {
-  const dim3 grid = node_grid(P, L), block(L.bx, L.by);
+  const dim3 grid = node_grid(P), block(kThreads);
   LBM_PREC_SWITCH(precision, (get_populations_kernel<PR, QQ><<<grid, block, 0, L.stream>>>(
                                  (const typename Types<PR>::S *)g, out, P, a_lo, a_hi)));
   return cudaGetLastError();
@@ -662,7 +660,7 @@ cudaError_t launch_get_populations(const KParams &P, int precision, const void *
 
 cudaError_t launch_set_populations(const KParams &P, int precision, const double *f, void *g, int a_lo,
                                    int a_hi, const Launch &L) {
-  const dim3 grid = node_grid(P, L), block(L.bx, L.by);
+  const dim3 grid = node_grid(P), block(kThreads);
   LBM_PREC_SWITCH(precision, (set_populations_kernel<PR, QQ><<<grid, block, 0, L.stream>>>(
                                  f, (typename Types<PR>::S *)g, P, a_lo, a_hi)));
   return cudaGetLastError();

@@ -47,14 +47,11 @@ __device__ __forceinline__ void gather_psi_pair(const float *__restrict__ psi, c
 }
 
 __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int &y, int &z) {
-  const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  y = blockIdx.y * blockDim.y + threadIdx.y;
+  const unsigned p = blockIdx.x * blockDim.x + threadIdx.x, W = (unsigned)P.px / 2;
+  y = (int)(P.pair_m ? __umulhi(p, P.pair_m) : p / W);
   z = blockIdx.z;
-  if (x >= P.nx || y >= P.ny) return false;
-  px.x = x;
-  px.xm1 = x == 0 ? P.nx - 1 : x - 1;
-  px.xp2 = x + 2 >= P.nx ? x + 2 - P.nx : x + 2;
-  return true;
+  px = pair_x(P, 2 * (int)(p - y * W));
+  return y < P.ny;
 }
 
 template <typename S, int EOS, bool DF>
@@ -116,13 +113,11 @@ __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__
   fused_pair15_at<S, SIGMA, false, ODD>(g_in, g_out, psi, P, px.x, y, z);
 }
 
-dim3 pair_grid(const KParams &P, const Launch &L) {
-  return dim3((P.px / 2 + 31) / 32, (P.ny + L.by - 1) / L.by, P.nz);
-}
+dim3 pair_grid(const KParams &P) { return plane_grid(P.px / 2 * P.ny, P.nz); }
 
 template <typename S, bool DF>
 cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsigned *err, const Launch &L) {
-  const dim3 grid = pair_grid(P, L), block(32, L.by);
+  const dim3 grid = pair_grid(P), block(kThreads);
   const S *gg = (const S *)g;
   float *pp = (float *)psi;
   if (P.q == 15) {
@@ -142,7 +137,7 @@ cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsign
 template <typename S, bool ODD>
 cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void *g_in, void *g_out,
                                 const void *psi, const Launch &L) {
-  const dim3 grid = pair_grid(P, L), block(32, L.by);
+  const dim3 grid = pair_grid(P), block(kThreads);
   const S *gi = (const S *)g_in;
   S *go = (S *)g_out;
   const float *pp = (const float *)psi;
