@@ -148,9 +148,10 @@ lbm_status lbm_init_field(lbm_ctx *ctx, const double *rho, int on_device, double
 
 /* Advance n >= 1 time steps (asynchronous on the context's stream).  Each step
  * is the form's step kernels (lbm_set_tuning): by default, for FP32 storage
- * with an even Nx, one cooperative launch of the work-list single pass;
+ * with an even Nx, one cooperative launch of the work-list single pass (small
+ * boxes, up to about 10^6 nodes: one launch for up to 256 steps of a call);
  * otherwise two kernels, the psi pass and the fused force + collision +
- * pull-streaming pass.  A work-list launch carries the context's launch count
+ * pull-streaming pass.  A work-list launch carries the context's step count
  * (its completion and item-claim counters advance with every launch), so steps
  * must not be captured into a CUDA graph and replayed: a replayed launch finds
  * its counters out of step, stops early and reports LBM_ERR_TIMEOUT at the next
@@ -215,7 +216,10 @@ lbm_status lbm_kernel_times(lbm_ctx *ctx, double *ms_psi, long long *n_psi,
  * fused tiles it reads; the FP64 EOS of the
  * psi work overlaps the fused work's HBM stream and the populations it pulls
  * come from L2 (Eqs. 3-6 in 2 x Q x s + 8 bytes per node); results equal the
- * two-pass step bit for bit; the first step in this mode allocates the item
+ * two-pass step bit for bit.  Small boxes take the same jobs through up to 256
+ * steps in one launch, every thread block keeping its tiles, a counter per tile
+ * and kind of job saying how far each is (one step per launch while
+ * lbm_set_profiling is on).  The first step in this mode allocates the item
  * table and counters (about 20 bytes per tile and plane), freed by
  * lbm_destroy.  tile picks the x-y tile of
  * the single-pass kernel (0: 32x4, 1: 32x8, 2: 64x4); z_planes the z planes

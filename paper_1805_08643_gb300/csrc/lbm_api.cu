@@ -41,6 +41,7 @@ struct lbm_ctx {
   lbm::QueueState q{};      // its item table and counters (one allocation: q_mem)
   void *q_mem = nullptr;
   int q_stamp = 0;
+  int steps_grid = 0;       // small box: grid of the several-steps kernel (q.done: its counters), 0: the list
   bool eos_f2 = false;      // EOS radicand in compensated FP32 pairs (psi pass)
   int tile = 1, zc = 0;     // its tile shape and z planes per CTA (0 = automatic)
   bool owns = false, have_buffers = false, initialized = false, psi_valid = false;
@@ -163,12 +164,25 @@ void free_queue(lbm_ctx *c) {
   c->q_mem = nullptr;
   c->q = lbm::QueueState{};
   c->q_stamp = 0;
+  c->steps_grid = 0;
 }
 
 // Item table and counters of the work-list single pass (zeroed counters).
 lbm_status ensure_queue(lbm_ctx *c) {
   if (c->q_mem) return LBM_OK;
   int grid = 0;
+  CK(lbm::steps_grid(c->P, c->precision, &grid), "several-steps occupancy");
+  if (grid > 0) {
+    const size_t bytes = lbm::steps_counters(c->P) * sizeof(int);
+    void *m = nullptr;
+    CK(cudaMalloc(&m, bytes), "cudaMalloc(work list)");
+    c->q_mem = m;
+    c->q.done = (int *)m;
+    c->q_stamp = 0;
+    c->steps_grid = grid;
+    CK(cudaMemsetAsync(m, 0, bytes, c->L.stream), "clear work list counters");
+    return LBM_OK;
+  }
   CK(lbm::queue_grid(c->precision, c->P.q, &grid), "work list occupancy");
   std::vector<int4> items;
   if (!lbm::queue_items(c->P, grid, items)) return fail(c, LBM_ERR_ARG, "no valid work list for this box");
@@ -203,6 +217,9 @@ lbm_status finish_init(lbm_ctx *c, const double *rho_dev) {
   c->steps = 0;
   return LBM_OK;
 }
+
+// Steps of a small box per launch: enough for the launch not to matter, and short enough for a launch to end soon.
+constexpr int kMostStepsPerLaunch = 256;
 
 bool finite_positive(double v) { return std::isfinite(v) && v > 0; }
 
@@ -375,10 +392,26 @@ lbm_status lbm_step(lbm_ctx *c, int n) {
   const int zc = c->zc > 0 ? c->zc : auto_zc(c);
   for (int k = 0; k < n; ++k) {
     void *gin = c->g[c->cur], *gout = c->g[c->cur ^ 1];
-    if (c->queued) {
+    if (c->queued && c->steps_grid > 0) {
+      // as many steps as the call, the next check and the length of a launch allow (one if they are timed apart)
+      int m = std::min(n - k, kMostStepsPerLaunch);
+      if (c->check_interval > 0) m = std::min(m, c->check_interval - (int)(c->steps % c->check_interval));
+      if (c->profiling) m = 1;
+      CK(timed(c, 1, [&] {
+           return lbm::launch_steps(c->P, c->op, c->eos_f2, gin, gout, cur_psi(c), psi_at(c, c->pc ^ 1), c->steps_grid,
+                                    c->q.done, m, (int)((unsigned)c->q_stamp + 1u), err_word(c), c->L.stream);
+         }),
+         "several-steps kernel");
+      c->q_stamp = (int)((unsigned)c->q_stamp + (unsigned)m);  // (counts may wrap)
+      c->pc ^= m & 1;
+      c->cur ^= m & 1;
+      c->psi_valid = true;
+      c->steps += m - 1;  // the last one is counted below
+      k += m - 1;
+    } else if (c->queued) {
       void *pin = cur_psi(c), *pout = psi_at(c, c->pc ^ 1);
       // the counters advance only with launches that run (each one claims every item once)
-      const int stamp = c->q_stamp + 1;
+      const int stamp = (int)((unsigned)c->q_stamp + 1u);
       CK(timed(c, 1, [&] {
            return lbm::launch_queue(c->P, c->precision, c->op, c->eos_f2, gin, gout, pin, pout, c->q,
                                     stamp, err_word(c), c->L.stream);

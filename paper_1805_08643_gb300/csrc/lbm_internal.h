@@ -380,6 +380,17 @@ cudaError_t launch_queue(const KParams &P, int precision, int op, bool df, const
                          const void *psi_in, void *psi_out, const QueueState &q, int stamp, unsigned *err,
                          cudaStream_t s);
 
+// Up to nsteps steps of a small box in one launch (FP32 storage, even Nx; the
+// work-list jobs, each block keeping its tiles).  steps_grid gives the grid, 0
+// for a box that is too large or not of that form.  counters: steps_counters
+// ints, zero before the first launch; stamp: 1 + the steps launched on them.
+// The state and psi after nsteps steps are in g_in / psi_in (nsteps even) or
+// g_out / psi_out (odd).
+cudaError_t steps_grid(const KParams &P, int precision, int *grid);
+size_t steps_counters(const KParams &P);
+cudaError_t launch_steps(const KParams &P, int op, bool df, void *g_in, void *g_out, void *psi_in, void *psi_out,
+                         int grid, int *counters, int nsteps, int stamp, unsigned *err, cudaStream_t s);
+
 // The work-list step over a batch (every box D3Q19 with an even Nx): one
 // cooperative launch per step; items hold a fused tile job and a psi tile job
 // of any boxes (x / z: box index or -1, y / w: z | tile << 16).  The list is

@@ -31,6 +31,14 @@ template <> struct PairIO<__half> {
   }
 };
 
+// Plain loads, for arrays that other blocks write in the same launch: coherent
+// after an acquire, where the read-only path of PairIO could return what was
+// there before.
+struct PlainLoad {
+  static __device__ __forceinline__ float2 ld2(const float *p) { return *(const float2 *)p; }
+  static __device__ __forceinline__ float ld1(const float *p) { return *p; }
+};
+
 // Row offset (y', z' part of the node index) of the pull source of direction a.
 __device__ __forceinline__ int src_row(const Nbhd &nb, int a) {
   switch (a) {
@@ -61,19 +69,19 @@ struct PairX {
 // Pull the 19 deviations of nodes x and x + 1 (Eq. 5).  Populations with
 // e_x = 0 come from an aligned pair of the source row, those with e_x = +1
 // from (x-1, x) and those with e_x = -1 from (x+1, x+2), read as two scalars.
-template <typename S>
-__device__ __forceinline__ void pull_pair(const S *__restrict__ g, unsigned n, const Nbhd &nb, const PairX &px,
+template <typename S, typename Ld = PairIO<S>>
+__device__ __forceinline__ void pull_pair(const S *g, unsigned n, const Nbhd &nb, const PairX &px,
                                           V2 f[19]) {
 #pragma unroll
   for (int a = 0; a < 19; ++a) {
     const S *rowp = g + (size_t)a * n + src_row(nb, a);
     float2 v;
     if (ex_of(a) == 0)
-      v = PairIO<S>::ld2(rowp + px.x);
+      v = Ld::ld2(rowp + px.x);
     else if (ex_of(a) > 0)
-      v = make_float2(PairIO<S>::ld1(rowp + px.xm1), PairIO<S>::ld1(rowp + px.x));
+      v = make_float2(Ld::ld1(rowp + px.xm1), Ld::ld1(rowp + px.x));
     else
-      v = make_float2(PairIO<S>::ld1(rowp + px.x + 1), PairIO<S>::ld1(rowp + px.xp2));
+      v = make_float2(Ld::ld1(rowp + px.x + 1), Ld::ld1(rowp + px.xp2));
     f[a] = PairIO<S>::decode(v, a);
   }
 }
@@ -197,27 +205,27 @@ __device__ __forceinline__ PairX pair_x(const KParams &P, int x) {
 // which keeps the registers of the single-pass kernels down.  The arithmetic
 // and its order are those of fused_pair_kernel, so the results are equal bit
 // for bit.
-template <typename S, int OP, bool SIGMA, bool FORCE_FIRST, bool ODD>
-__device__ __forceinline__ void fused_pair_at(const S *__restrict__ g_in, S *__restrict__ g_out,
-                                              const float *__restrict__ psi, const KParams &P, int x, int y, int z,
+// Ld, PsiLd: how populations and psi are read.
+template <typename S, int OP, bool SIGMA, bool FORCE_FIRST, bool ODD, typename Ld = PairIO<S>, typename PsiLd = PairIO<float>>
+__device__ __forceinline__ void fused_pair_at(const S *g_in, S *__restrict__ g_out, const float *psi, const KParams &P, int x, int y, int z,
                                               const Rates<V2> &r) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
   V2 f[19];
   // without FORCE_FIRST both sets of loads are issued before either is used
   // (one memory round trip, more registers)
-  if (!FORCE_FIRST) pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
+  if (!FORCE_FIRST) pull_pair<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
   V2 Fx, Fy, Fz, dS4;
   {
     V2 p[19];
     auto row3 = [&](int row, V2 &c, V2 &plus, V2 &minus) {
-      const float2 m = __ldg((const float2 *)(psi + row + px.x));
-      const float l = __ldg(psi + row + px.xm1), rr = __ldg(psi + row + px.xp2);
+      const float2 m = PsiLd::ld2(psi + row + px.x);
+      const float l = PsiLd::ld1(psi + row + px.xm1), rr = PsiLd::ld1(psi + row + px.xp2);
       c = V2(m);
       plus = V2(m.y, rr);
       minus = V2(l, m.x);
     };
-    auto row1 = [&](int row) { return V2(__ldg((const float2 *)(psi + row + px.x))); };
+    auto row1 = [&](int row) { return V2(PsiLd::ld2(psi + row + px.x)); };
     row3(nb.r00, p[0], p[1], p[2]);
     row3(nb.rp0, p[3], p[7], p[10]);
     row3(nb.rm0, p[4], p[9], p[8]);
@@ -229,7 +237,7 @@ __device__ __forceinline__ void fused_pair_at(const S *__restrict__ g_in, S *__r
     p[18] = row1(nb.rmp);
     force_pair<SIGMA>(p, P, Fx, Fy, Fz, dS4);
   }
-  if (FORCE_FIRST) pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
+  if (FORCE_FIRST) pull_pair<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
   collide_pair<OP>(f, Fx, Fy, Fz, dS4, P, r, OP);
   store_pair_f<S, ODD>(g_out, P, x, (unsigned)nb.self, f);
 }

@@ -46,7 +46,7 @@ __device__ __forceinline__ int src_row15(const Nbhd &nb, int a) {
 // Pull of both nodes' 15 populations; Ld: PairIO<S> (read-only path) or
 // L2Load<S> (populations written earlier in the same launch).
 template <typename S, typename Ld = PairIO<S>>
-__device__ __forceinline__ void pull_pair15(const S *__restrict__ g, unsigned n, const Nbhd &nb, const PairX &px,
+__device__ __forceinline__ void pull_pair15(const S *g, unsigned n, const Nbhd &nb, const PairX &px,
                                             V2 f[q15::kQ]) {
 #pragma unroll
   for (int a = 0; a < q15::kQ; ++a) {
@@ -63,17 +63,18 @@ __device__ __forceinline__ void pull_pair15(const S *__restrict__ g, unsigned n,
 }
 
 // psi(x + e_a) of both nodes, p[a] (Eq. 15 stencil on D3Q15).
-__device__ __forceinline__ void gather_psi_pair15(const float *__restrict__ psi, const Nbhd &nb, const PairX &px,
+template <typename Ld = PairIO<float>>
+__device__ __forceinline__ void gather_psi_pair15(const float *psi, const Nbhd &nb, const PairX &px,
                                                   V2 p[q15::kQ]) {
   // centre pair, and the pairs shifted by +1 and -1 in x
   auto row3 = [&](int row, V2 &c, V2 &plus, V2 &minus) {
-    const float2 m = __ldg((const float2 *)(psi + row + px.x));
-    const float l = __ldg(psi + row + px.xm1), r = __ldg(psi + row + px.xp2);
+    const float2 m = Ld::ld2(psi + row + px.x);
+    const float l = Ld::ld1(psi + row + px.xm1), r = Ld::ld1(psi + row + px.xp2);
     c = V2(m);
     plus = V2(m.y, r);
     minus = V2(l, m.x);
   };
-  auto row1 = [&](int row) { return V2(__ldg((const float2 *)(psi + row + px.x))); };
+  auto row1 = [&](int row) { return V2(Ld::ld2(psi + row + px.x)); };
   V2 unused;
   row3(nb.r00, p[0], p[1], p[2]);
   p[3] = row1(nb.rp0);
@@ -88,17 +89,16 @@ __device__ __forceinline__ void gather_psi_pair15(const float *__restrict__ psi,
 
 // Fused pass of one pair on D3Q15 (pull, force from the psi stencil, collision,
 // store); FORCE_FIRST as in fused_pair_at.
-template <typename S, bool SIGMA, bool FORCE_FIRST, bool ODD>
-__device__ __forceinline__ void fused_pair15_at(const S *__restrict__ g_in, S *__restrict__ g_out,
-                                                const float *__restrict__ psi, const KParams &P, int x, int y, int z) {
+template <typename S, bool SIGMA, bool FORCE_FIRST, bool ODD, typename Ld = PairIO<S>, typename PsiLd = PairIO<float>>
+__device__ __forceinline__ void fused_pair15_at(const S *g_in, S *__restrict__ g_out, const float *psi, const KParams &P, int x, int y, int z) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
   V2 f[q15::kQ];
-  if (!FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.np, nb, px, f);
+  if (!FORCE_FIRST) pull_pair15<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
   V2 Fx, Fy, Fz, dS4;
   {
     V2 p[q15::kQ];
-    gather_psi_pair15(psi, nb, px, p);
+    gather_psi_pair15<PsiLd>(psi, nb, px, p);
     V2 Sx, Sy, Sz;
     q15::psi_gradient<V2>(p, Sx, Sy, Sz);
     const V2 kk = V2((double)-P.fG) * p[0];
@@ -107,7 +107,7 @@ __device__ __forceinline__ void fused_pair15_at(const S *__restrict__ g_in, S *_
     Fy = kk * Sy;
     Fz = kk * Sz;
   }
-  if (FORCE_FIRST) pull_pair15<S>(g_in, (unsigned)P.np, nb, px, f);
+  if (FORCE_FIRST) pull_pair15<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
   q15::collide<V2>(f, V2((double)P.frho_ref), Fx, Fy, Fz, dS4, Rates<V2>(P));
   store_pair<ODD>(
       P, x,

@@ -11,12 +11,12 @@
 //     planes z'-1..z'+1 on its rows and the rows next to them (periodic) and
 //     pulls their output through L2, where it still is.
 // The host builds the list (and checks it): fused jobs plane by plane; each
-// psi job in the first free item at least half a wave of the grid (grid / 2
-// items) after the last fused job it reads.  Half a wave: by the time a block
-// reaches the psi job those fused jobs are normally finished, so the wait is
-// one poll, while writer and reader stay close enough for the populations to
-// be still in L2 (measured on GB300: a whole wave waits less but re-reads about
-// twice as much from DRAM, and is slower; a quarter waits more).
+// psi job in the first free item at least about half a wave of the grid
+// (grid / 2 items) after the last fused job it reads.  Half a wave: by the time
+// a block reaches the psi job those fused jobs are normally finished, so the
+// wait is one poll, while writer and reader stay close enough for the
+// populations to be still in L2 (measured on GB300: a whole wave waits less but
+// re-reads about twice as much from DRAM, and is slower; a quarter waits more).
 //
 // Block b starts with item b; from then on it claims the next unclaimed item
 // (one atomic fetch per item, issued when an item starts and read when it
@@ -55,13 +55,11 @@
 #include "lbm_internal.h"
 #include "lbm_pair.cuh"
 #include "lbm_pair15.cuh"
+#include "lbm_worklist.cuh"
 
 namespace lbm {
 namespace {
 
-constexpr int TXP = 32;          // pair columns of a tile: 64 nodes
-constexpr int kRows = 4;         // rows of a tile (one warp each)
-constexpr int NTH = TXP * kRows;
 // Resident blocks per SM the register budgets are set for.  The fused jobs wait
 // for memory most of the time, so a block more is worth more than the spills it
 // costs, up to a point; taking the force from psi before the populations are
@@ -76,76 +74,6 @@ __host__ __device__ constexpr int min_blocks(int q) { return q == 15 ? 8 : 7; }
 // not bound by the FP64 unit, and the integer work cost 1 % (FP32 storage) and
 // 3 % (FP16) of a 256^3 step on GB300.
 constexpr bool kIntCvt = false;
-
-// The pair of thread tid in tile t of a plane: true if there is one.
-__device__ __forceinline__ bool tile_node(const TileMap &G, bool lin, const KParams &P, int t, int tid, int &x,
-                                          int &y) {
-  if (lin) {
-    const unsigned p = (unsigned)t * NTH + tid;
-    y = (int)__umulhi(p, G.m);
-    x = 2 * ((int)p - y * G.W);
-    return (int)p < G.M;
-  }
-  const int ty = t / G.ntx;
-  x = (t - ty * G.ntx) * 2 * TXP + 2 * (tid & (TXP - 1));
-  y = ty * kRows + tid / TXP;
-  return x < P.nx && y < P.ny;
-}
-
-// The tiles a psi job of tile t reads in planes z - 1, z, z + 1: lane's share
-// (dz, tile), false if it has none.  64 x 4 tiles: the 3 x 3 around it.  lin: all
-// tiles of the rows from one before its first to one after its last (a pair at
-// the end of a row reads the row's other end), at most kMaxLin of them, which
-// follow each other modulo T.
-constexpr int kMaxLin = 10;
-__host__ __device__ __forceinline__ bool dep_of_lane(const TileMap &G, bool lin, int t, int lane, int &dz,
-                                                               int &tile) {
-  if (lin) {
-    const int a = t * NTH, b = a + NTH < G.M ? a + NTH - 1 : G.M - 1;
-    const int ya = (int)(((unsigned long long)(unsigned)a * G.m) >> 32);
-    const int yb = (int)(((unsigned long long)(unsigned)b * G.m) >> 32);
-    int s = (ya - 1) * G.W, e = (yb + 2) * G.W - 1;
-    const bool all = e - s + 1 + NTH >= G.M;  // the range meets itself
-    if (s < 0) s += G.M;
-    if (e >= G.M) e -= G.M;
-    const int first = all ? 0 : s / NTH;
-    int cnt = all ? G.T : e / NTH - first + 1;
-    if (cnt <= 0) cnt += G.T;
-    dz = lane / kMaxLin - 1;
-    const int j = lane % kMaxLin;
-    tile = first + j;
-    if (tile >= G.T) tile -= G.T;
-    return dz <= 1 && j < cnt;
-  }
-  const int ty = t / G.ntx, tx = t - ty * G.ntx;
-  int xx = tx + lane % 3 - 1, yy = ty + (lane / 3) % 3 - 1;
-  xx = xx < 0 ? xx + G.ntx : (xx >= G.ntx ? xx - G.ntx : xx);
-  yy = yy < 0 ? yy + G.nty : (yy >= G.nty ? yy - G.nty : yy);
-  dz = lane / 9 - 1;
-  tile = yy * G.ntx + xx;
-  return lane < 27;
-}
-
-// Polls, by the lanes that have one, the counters of the fused jobs a psi job
-// reads until each shows `target`; false (on every lane) if one gave up.
-__device__ __forceinline__ bool wait_for_fused(const TileMap &G, bool lin, const KParams &P, const int *__restrict__ done,
-                                               int base, int count, int z, int t, int lane, int target) {
-  bool ok = true;
-  int dz, tile;
-  if (dep_of_lane(G, lin, t, lane, dz, tile)) {
-    int zz = z + dz;
-    zz = zz < 0 ? zz + P.nz : (zz >= P.nz ? zz - P.nz : zz);
-    const int *c = done + LBM_IDX(base + zz * G.T + tile, count);
-    for (int n = 0; counter_acquire(c) < target; ++n) {
-      if (n >= P.spin_limit) {
-        ok = false;
-        break;
-      }
-      __nanosleep(32);
-    }
-  }
-  return __all_sync(0xffffffffu, ok);
-}
 
 // The item claim number c of this launch names: gridDim.x + c.  Every launch
 // makes exactly nitems claims, so c < nitems; a claim outside that range
@@ -204,7 +132,8 @@ __global__ void __launch_bounds__(NTH, min_blocks(Q))
     if (it.z >= 0) {
       int z = it.z, t = it.w;
       asm volatile("" : "+r"(z), "+r"(t));
-      if (!wait_for_fused(G, LIN, P, done, 0, P.nz * G.T, z, t, lane, stamp + P.wait_bias)) e |= kErrTimeout;
+      if (!wait_for_jobs(G, LIN, P, done, 0, P.nz * G.T, z, t, lane, stamp + P.wait_bias, P.spin_limit))
+        e |= kErrTimeout;
       int x, y;
       if (tile_node(G, LIN, P, t, row * TXP + lane, x, y)) {
         if constexpr (Q == 15)
@@ -368,7 +297,8 @@ __global__ void __launch_bounds__(NTH, kBatchBlocks)
       int z = (int)((unsigned)it.w & 0xffffu), t = (int)((unsigned)it.w >> 16);
       asm volatile("" : "+r"(z), "+r"(t));
       // counters are cleared before every launch
-      if (!wait_for_fused(B.map, B.map.lin, P, done, B.qbase, ndone, z, t, threadIdx.x, 1 + P.wait_bias)) e |= kErrTimeout;
+      if (!wait_for_jobs(B.map, B.map.lin, P, done, B.qbase, ndone, z, t, threadIdx.x, 1 + P.wait_bias, P.spin_limit))
+        e |= kErrTimeout;
       const int in = B.cur ^ parity;
       int x, y;
       if (tile_node(B.map, B.map.lin, P, t, tid, x, y))
@@ -493,8 +423,7 @@ bool queue_items(const KParams &P, int grid, std::vector<int4> &out) {
   const long long nf = (long long)P.nz * G.T;
   if (P.nz < 3 || grid < 1 || nf >= (1LL << 30)) return false;
   // fused job j = (j / T, j % T); psi job (z, t) is ready after the last of the
-  // fused jobs it reads and goes to the first free item >= ready + lag, half
-  // a wave of the grid later (at least one item)
+  // fused jobs it reads and goes to the first free item >= ready + lag
   const long long lag = std::max(1, grid / 2);
   const std::vector<int> last = last_tiles(G);
   std::vector<long long> ready((size_t)nf);
