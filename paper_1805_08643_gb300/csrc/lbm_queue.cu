@@ -12,7 +12,7 @@
 //     pulls their output through L2, where it still is.
 // The host builds the list (and checks it): fused jobs plane by plane; each
 // psi job in the first free item at least about half a wave of the grid
-// (grid / 2 items) after the last fused job it reads.  Half a wave: by the time
+// (psi_lag items) after the last fused job it reads.  Half a wave: by the time
 // a block reaches the psi job those fused jobs are normally finished, so the
 // wait is one poll, while writer and reader stay close enough for the
 // populations to be still in L2 (measured on GB300: a whole wave waits less but
@@ -341,6 +341,16 @@ std::vector<long long> by_ready(const std::vector<long long> &ready) {
   return order;
 }
 
+// Items between a psi job and the last fused job it reads: 3/8 of a wave of the
+// grid where a plane is large (the populations leave L2 sooner), 5/8 where it
+// is small (more of the list hangs on each plane).  At 1/4, 3/8, 1/2, 5/8 and
+// 3/4: 128^3 89.0, 84.2, 78.4, 74.3 and 73.7 us per step, 160^3 164, 148, 136,
+// 134 and 135, 256^3 558, 514, 518, 526 and 534, 512^3 4.66, 4.32, 4.34, 4.38 and
+// 4.42 ms; 192^3 (144 tiles a plane) 267, 236, 220, 220 and 222.
+long long psi_lag(int grid, int tiles_per_plane) {
+  return std::max(1LL, (long long)grid * (tiles_per_plane < 192 ? 5 : 3) / 8);
+}
+
 // Psi jobs go to the first free item at least `lag` items after the last of
 // the fused jobs they read (ready[]); fused job j sits in item j.  Checks the
 // result as the single-box list does.
@@ -424,7 +434,7 @@ bool queue_items(const KParams &P, int grid, std::vector<int4> &out) {
   if (P.nz < 3 || grid < 1 || nf >= (1LL << 30)) return false;
   // fused job j = (j / T, j % T); psi job (z, t) is ready after the last of the
   // fused jobs it reads and goes to the first free item >= ready + lag
-  const long long lag = std::max(1, grid / 2);
+  const long long lag = psi_lag(grid, G.T);
   const std::vector<int> last = last_tiles(G);
   std::vector<long long> ready((size_t)nf);
   for (long long p = 0; p < nf; ++p) {
