@@ -13,6 +13,8 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
+#include <type_traits>
 
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
@@ -54,6 +56,39 @@ __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int 
   return y < P.ny;
 }
 
+// Force and collision of the two nodes of a pair one after the other in scalar
+// FP32.  The compiler contracts more of the scalar code to FMAs than V2 does; a
+// box with an odd Nx and FP32 storage keeps the rounding it always had (that of
+// the one-node kernels) on the loads and stores of the pair kernels.
+template <int OP, bool SIGMA, int Q>
+__device__ __forceinline__ void force_collide_lanes(V2 f[Q], const V2 p[Q], const KParams &P) {
+  const Rates<float> r(P);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    float fl[Q], pl[Q], Sx, Sy, Sz;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      fl[a] = k == 0 ? f[a].v.x : f[a].v.y;
+      pl[a] = k == 0 ? p[a].v.x : p[a].v.y;
+    }
+    if constexpr (Q == 15)
+      q15::psi_gradient<float>(pl, Sx, Sy, Sz);
+    else
+      psi_gradient<float>(pl, Sx, Sy, Sz);
+    const float kk = -P.fG * pl[0];
+    const float Fx = kk * Sx, Fy = kk * Sy, Fz = kk * Sz;
+    const float dS4 = SIGMA ? P.fsigma_coef * (Sx * Sx + Sy * Sy + Sz * Sz) : 0.f;
+    if constexpr (Q == 15)
+      q15::collide<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
+    else if (OP == kNonOrth)
+      collide_nonorth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
+    else
+      collide_orth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) (k == 0 ? f[a].v.x : f[a].v.y) = fl[a];
+  }
+}
+
 template <typename S, int EOS, bool DF>
 __global__ void __launch_bounds__(128) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                        const KParams P, unsigned *__restrict__ err) {
@@ -81,7 +116,10 @@ __global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g
   pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
   V2 p[19];
   gather_psi_pair(psi, nb, px, p);
-  force_collide_pair<OP, SIGMA>(f, p, P, Rates<V2>(P), OP);
+  if constexpr (ODD && std::is_same<S, float>::value)
+    force_collide_lanes<OP, SIGMA, 19>(f, p, P);
+  else
+    force_collide_pair<OP, SIGMA>(f, p, P, Rates<V2>(P), OP);
   store_pair_f<S, ODD>(g_out, P, px.x, (unsigned)nb.self, f);
 }
 
@@ -110,7 +148,16 @@ __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
-  fused_pair15_at<S, SIGMA, false, ODD>(g_in, g_out, psi, P, px.x, y, z);
+  if constexpr (ODD && std::is_same<S, float>::value) {
+    const Nbhd nb(px.x, y, z, P);
+    V2 f[q15::kQ], p[q15::kQ];
+    pull_pair15<S>(g_in, (unsigned)P.np, nb, px, f);
+    gather_psi_pair15(psi, nb, px, p);
+    force_collide_lanes<kNonOrth, SIGMA, q15::kQ>(f, p, P);
+    store_pair15_f<S, ODD>(g_out, P, px.x, (unsigned)nb.self, f);
+  } else {
+    fused_pair15_at<S, SIGMA, false, ODD>(g_in, g_out, psi, P, px.x, y, z);
+  }
 }
 
 dim3 pair_grid(const KParams &P) { return plane_grid(P.px / 2 * P.ny, P.nz); }

@@ -87,6 +87,22 @@ __device__ __forceinline__ void gather_psi_pair15(const float *psi, const Nbhd &
   row3(nb.rmp, unused, p[11], p[10]);
 }
 
+// Stores the 15 results of a pair.
+template <typename S, bool ODD>
+__device__ __forceinline__ void store_pair15_f(S *__restrict__ g, const KParams &P, int x, unsigned self,
+                                               const V2 f[q15::kQ]) {
+  store_pair<ODD>(
+      P, x,
+      [&] {
+#pragma unroll
+        for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st2(g + (size_t)a * P.np + self, a, f[a]);
+      },
+      [&](int off) {
+#pragma unroll
+        for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st1(g + (size_t)a * P.np + self + off, a, f[a]);
+      });
+}
+
 // Fused pass of one pair on D3Q15 (pull, force from the psi stencil, collision,
 // store); FORCE_FIRST as in fused_pair_at.
 template <typename S, bool SIGMA, bool FORCE_FIRST, bool ODD, typename Ld = PairIO<S>, typename PsiLd = PairIO<float>>
@@ -109,16 +125,7 @@ __device__ __forceinline__ void fused_pair15_at(const S *g_in, S *__restrict__ g
   }
   if (FORCE_FIRST) pull_pair15<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
   q15::collide<V2>(f, V2((double)P.frho_ref), Fx, Fy, Fz, dS4, Rates<V2>(P));
-  store_pair<ODD>(
-      P, x,
-      [&] {
-#pragma unroll
-        for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st2(g_out + (size_t)a * P.np + nb.self, a, f[a]);
-      },
-      [&](int off) {
-#pragma unroll
-        for (int a = 0; a < q15::kQ; ++a) PairIO15<S>::st1(g_out + (size_t)a * P.np + nb.self + off, a, f[a]);
-      });
+  store_pair15_f<S, ODD>(g_out, P, x, (unsigned)nb.self, f);
 }
 
 // psi of one pair on D3Q15 from populations written earlier in the same launch (pulls through L2).

@@ -65,7 +65,8 @@ namespace {
 // costs, up to a point; taking the force from psi before the populations are
 // pulled (FORCE_FIRST) is what lets a thread live on 72 registers.  256^3 FP32
 // steps, non-orthogonal / D3Q15, at 6, 7 and 8 blocks: 527 / 457, 515 / 444 and
-// 551 / 430 us (192^3: 250 / 229, 220 / 235 and 233 / 190).  Batches stay at 6
+// 551 / 430 us (192^3: 250 / 229, 220 / 235 and 233 / 190; with every V2
+// difference one instruction, see operator-; 526 / 431 us as it is).  Batches stay at 6
 // (848 against 842 us for 64 boxes at 7, with 180 bytes spilled).
 constexpr int kBatchBlocks = 6;
 __host__ __device__ constexpr int min_blocks(int q) { return q == 15 ? 8 : 7; }

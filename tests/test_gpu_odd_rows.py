@@ -1,7 +1,7 @@
 """Boxes with an odd Nx in the FP32-arithmetic forms: stored rows get one element more, which repeats node 0, and
-the two-node kernels step them.  The same box on every path (the single box's two passes, a batch's work list and
-tile kernels, in a mix with even boxes) must agree bit for bit in FP32, and the padding must survive every way a
-state is set, read and handed from one kind of step to another."""
+the two-node kernels step them.  The same box on every path (a batch's work list and tile kernels, in a mix with even
+boxes) must agree bit for bit in FP32; the single box's two passes collide an odd box's nodes one by one, with other
+roundings.  The padding must survive every way a state is set, read and handed from one kind of step to another."""
 
 import numpy as np
 import pytest
@@ -50,6 +50,7 @@ def test_batch_steps_odd_boxes_as_the_two_pass_single_box(op, prec):
 
     phys = physics(sigma=0.105)
     rl, rv = coexistence(0.8)
+    first = {}
     for tile in (3, 0, 1, 2) if prec == "f32" else (3,):  # the FP16 tile kernels may differ by half an ulp
         b = Batch(prec, "cs")
         boxes = []
@@ -64,6 +65,9 @@ def test_batch_steps_odd_boxes_as_the_two_pass_single_box(op, prec):
         for i, grid in boxes:
             rho, u = b.moments(i)
             rho1, u1 = _two_pass(grid, op, prec, 7)
+            if prec == "f32" and grid[0] % 2:
+                assert max_abs(rho, rho1) <= 1e-6 and max_abs(u, u1) <= 1e-6, (tile, grid)
+                rho1, u1 = first.setdefault(grid, (rho, u))
             assert np.array_equal(rho, rho1) and np.array_equal(u, u1), (tile, grid)
         b.close()
 
