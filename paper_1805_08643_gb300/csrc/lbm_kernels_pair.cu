@@ -57,19 +57,20 @@ __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int 
 }
 
 // Force and collision of the two nodes of a pair one after the other in scalar
-// FP32.  The compiler contracts more of the scalar code to FMAs than V2 does; a
-// box with an odd Nx and FP32 storage keeps the rounding it always had (that of
-// the one-node kernels) on the loads and stores of the pair kernels.
+// FP32: a loop, since the compiler packs the two copies of an unrolled one and
+// contracts their products otherwise than the one-node kernels' code.  A box with an
+// odd Nx and FP32 storage keeps the rounding it always had (that of the one-node
+// kernels) on the loads and stores of the pair kernels.
 template <int OP, bool SIGMA, int Q>
-__device__ __forceinline__ void force_collide_lanes(V2 f[Q], const V2 p[Q], const KParams &P) {
+__device__ __forceinline__ void force_collide_lanes(V2 f[Q], V2 p[Q], const KParams &P) {
   const Rates<float> r(P);
-#pragma unroll
+#pragma unroll 1
   for (int k = 0; k < 2; ++k) {
     float fl[Q], pl[Q], Sx, Sy, Sz;
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
-      fl[a] = k == 0 ? f[a].v.x : f[a].v.y;
-      pl[a] = k == 0 ? p[a].v.x : p[a].v.y;
+      fl[a] = f[a].v.x;
+      pl[a] = p[a].v.x;
     }
     if constexpr (Q == 15)
       q15::psi_gradient<float>(pl, Sx, Sy, Sz);
@@ -85,7 +86,10 @@ __device__ __forceinline__ void force_collide_lanes(V2 f[Q], const V2 p[Q], cons
     else
       collide_orth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
 #pragma unroll
-    for (int a = 0; a < Q; ++a) (k == 0 ? f[a].v.x : f[a].v.y) = fl[a];
+    for (int a = 0; a < Q; ++a) {  // the other node comes first, then the order is back
+      f[a].v = make_float2(f[a].v.y, fl[a]);
+      p[a].v.x = p[a].v.y;
+    }
   }
 }
 
