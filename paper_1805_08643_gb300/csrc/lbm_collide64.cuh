@@ -17,10 +17,19 @@
 //    rate: the differences d78, d910, ... relax themselves, no moments are formed;
 //  - 2 x + y is written fma(2, x, y) (2 * x + y compiles to two additions), and
 //    the reciprocal takes three instructions (recip).
-// FP64 instructions per node of the fused pass, with the force: 214
-// non-orthogonal (255 moment by moment), 259 orthogonal; at 128^3 the pass takes
-// 852 us (1014) and 1027 us (1235), D3Q15 725 us (808), 0.84 of the unit's rate.
+//  - the linear parts (the forward and inverse chains, the sums of Eq. 15) run on
+//    the integer units, as sums of 64-bit fixed-point numbers: see Fixed.
+// FP64 instructions per node of the fused pass, with the force: 102 non-orthogonal
+// (255 moment by moment, 214 with these formulas in FP64 throughout), 92 orthogonal
+// (304, 259), 85 on D3Q15.  Fused pass at 128^3, FP64 throughout -> as it is: 855 ->
+// 430, 1018 -> 401 and 725 -> 344 us; bound by the FP64 and integer units together
+// (the FP64 instructions alone take 340 us).  More resident warps (96 registers)
+// and larger blocks are within 2 % of it.  Errors of a step's populations against
+// extended precision are those of FP64 throughout within a few per cent (droplets and
+// slabs with noise: 1.4 - 2.5e-16 relative, orthogonal a tenth less than before).
 #pragma once
+
+#include <type_traits>
 
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
@@ -40,301 +49,420 @@ __device__ __forceinline__ Shear64 shear64(const KParams &P, const Coeffs64 &C, 
   return Shear64{a * (1.0 / 12.0), a * 0.25, s * 0.125, 0.25 - s * 0.125, a * (1.0 / 36.0)};
 }
 
+// ------------------------------------------------------------------ linear parts
+// A chain of additions and small integer factors over values of one node, in the
+// numbers of a scale c: doubles (InDouble), or 64-bit fixed-point ones (InFixed).
+// An FP64 addition takes 16 cycles of an SM's FP64 unit for a warp (19 as it runs),
+// a 64-bit integer one a single cycle of the integer units, and the conversions
+// about 6 and 12.
+//
+// InFixed<S>: v 2^(1075 + S - E) for the largest exponent field E of the values the
+// chain starts from, so those have at most 53 + S bits; S is the largest for which
+// the chain's sums of factors, 2^(10 - S) at most, cannot leave 64 bits whatever
+// the values.  Sums are exact.  A value is cut off S bits below the last place of
+// the largest one, and a result is rounded once (to nearest, ties to even), where
+// an FP64 sum rounds each partial result.  What a chain starts from is chosen so
+// that the cut lies below half the last place of its results.
+struct Fixed {
+  long long v;
+};
+__device__ __forceinline__ Fixed operator+(Fixed a, Fixed b) { return {a.v + b.v}; }
+__device__ __forceinline__ Fixed operator-(Fixed a, Fixed b) { return {a.v - b.v}; }
+template <int K> __device__ __forceinline__ Fixed times(Fixed a) { return {a.v * K}; }
+template <int K> __device__ __forceinline__ double times(double a) { return (double)K * a; }
+
+struct InDouble {
+  using Value = double;
+  __device__ __forceinline__ double in(double v) const { return v; }
+  __device__ __forceinline__ double out(double v) const { return v; }
+  __device__ __forceinline__ double out_half(double v) const { return 0.5 * v; }
+  __device__ __forceinline__ double out_twice(double v) const { return 2.0 * v; }
+  static __device__ __forceinline__ double half(double v) { return 0.5 * v; }
+};
+template <int S> struct InFixed {
+  using Value = Fixed;
+  int E;
+  __device__ __forceinline__ Fixed in(double v) const {
+    const int hi = __double2hiint(v);
+    const unsigned d = (unsigned)(E - ((hi >> 20) & 0x7ff));  // a zero is shifted out
+    unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(v)) << S;
+    m >>= min(d, 63u);
+    const long long s = (long long)(hi >> 31);
+    return {((long long)m ^ s) - s};
+  }
+  __device__ __forceinline__ double out(Fixed x) const { return back(x, E); }
+  __device__ __forceinline__ double out_half(Fixed x) const { return back(x, E - 1); }
+  __device__ __forceinline__ double out_twice(Fixed x) const { return back(x, E + 1); }
+  static __device__ __forceinline__ Fixed half(Fixed x) { return {x.v >> 1}; }
+  static __device__ __forceinline__ double back(Fixed x, int E) {
+    const long long s = x.v >> 63;
+    const unsigned long long u = (unsigned long long)((x.v ^ s) - s);
+    const int lz = __clzll((long long)u);
+    const unsigned long long n = u << (lz & 63), m = n >> 11;  // 53 bits, the top one at 2^(E + 11 - S - lz)
+    const unsigned rest = ((unsigned)n & 0x7ffu) + ((unsigned)m & 1u) + 0x3ffu;
+    const unsigned long long r = m + (rest >> 11);  // a carry out of the fraction moves into the exponent
+    const unsigned hi = (unsigned)(r >> 32) + ((unsigned)(E + 10 - S - lz) << 20);
+    return u == 0 ? 0.0 : __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)r);
+  }
+};
+
+// E for the values from index I on; -1 where Fixed is not for them (infinities, NaN, nothing but very small values).
+template <int I = 0, int N>
+__device__ __forceinline__ int top_exponent(const double (&v)[N]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int k = I; k < N; ++k) m = max(m, (unsigned)__double2hiint(v[k]) & 0x7fffffffu);
+  const int e = (int)(m >> 20);
+  if (m == 0) return 128;
+  return e >= 128 && e < 2000 ? e : -1;
+}
+
 // The sums of Eq. 15 in units of the diagonal (D3Q15: corner) weight, where
 // the axes weigh 2 (8).  p[a] = psi(x + e_a).
-template <int Q>
-__device__ __forceinline__ void psi_sums64(const double p[Q], double &Sx, double &Sy, double &Sz) {
-  constexpr double axw = Q == 19 ? 2.0 : 8.0;
-  const double d78 = p[7] - p[8], d910 = p[9] - p[10], d1112 = p[11] - p[12], d1314 = p[13] - p[14];
+template <int Q, typename C>
+__device__ __forceinline__ void psi_sums_l(const double p[Q], const C &c, double &Sx, double &Sy, double &Sz) {
+  using L = typename C::Value;
+  constexpr int axw = Q == 19 ? 2 : 8;
+  L q[Q];
+#pragma unroll
+  for (int a = 1; a < Q; ++a) q[a] = c.in(p[a]);
+  const L d78 = q[7] - q[8], d910 = q[9] - q[10], d1112 = q[11] - q[12], d1314 = q[13] - q[14];
   if constexpr (Q == 19) {
-    const double d1516 = p[15] - p[16], d1718 = p[17] - p[18];
-    Sx = fma(axw, p[1] - p[2], (d78 + d910) + (d1112 + d1314));
-    Sy = fma(axw, p[3] - p[4], (d78 - d910) + (d1516 + d1718));
-    Sz = fma(axw, p[5] - p[6], (d1112 - d1314) + (d1516 - d1718));
+    const L d1516 = q[15] - q[16], d1718 = q[17] - q[18];
+    Sx = c.out(times<axw>(q[1] - q[2]) + ((d78 + d910) + (d1112 + d1314)));
+    Sy = c.out(times<axw>(q[3] - q[4]) + ((d78 - d910) + (d1516 + d1718)));
+    Sz = c.out(times<axw>(q[5] - q[6]) + ((d1112 - d1314) + (d1516 - d1718)));
   } else {
-    const double ab = d78 + d910, cd = d1112 - d1314;
-    Sx = fma(axw, p[1] - p[2], ab + cd);
-    Sy = fma(axw, p[3] - p[4], ab - cd);
-    Sz = fma(axw, p[5] - p[6], (d78 - d910) + (d1112 + d1314));
+    const L ab = d78 + d910, cd = d1112 - d1314;
+    Sx = c.out(times<axw>(q[1] - q[2]) + (ab + cd));
+    Sy = c.out(times<axw>(q[3] - q[4]) + (ab - cd));
+    Sz = c.out(times<axw>(q[5] - q[6]) + ((d78 - d910) + (d1112 + d1314)));
   }
 }
+template <int Q>
+__device__ __forceinline__ void psi_sums64(const double (&p)[Q], double &Sx, double &Sy, double &Sz) {
+  const int E = top_exponent(p);
+  if (E >= 0)
+    psi_sums_l<Q>(p, InFixed<Q == 19 ? 6 : 5>{E}, Sx, Sy, Sz);  // factors up to 12, 24
+  else
+    psi_sums_l<Q>(p, InDouble{}, Sx, Sy, Sz);
+}
 
-// Non-orthogonal operator: forward chains of Eq. 12, equilibria Eq. 13,
-// forcing Eq. 14, the Eq. 16 term from S2 (the squared sum of Eq. 15), inverse
-// chains of App. A.  f holds the deviations f_a - w_a rho_ref; out(a, f*_a)
-// takes the results (deviations again).
-template <typename Out>
-__device__ __forceinline__ void collide_nonorth64(const double f[19], double rho_ref, double Fx, double Fy, double Fz,
-                                                  double S2, const KParams &P, const Coeffs64 &C, Out &&out) {
-  // opposite-pair sums and differences
-  const double s12 = f[1] + f[2], d12 = f[1] - f[2];
-  const double s34 = f[3] + f[4], d34 = f[3] - f[4];
-  const double s56 = f[5] + f[6], d56 = f[5] - f[6];
-  const double s78 = f[7] + f[8], d78 = f[7] - f[8];
-  const double s910 = f[9] + f[10], d910 = f[9] - f[10];
-  const double s1112 = f[11] + f[12], d1112 = f[11] - f[12];
-  const double s1314 = f[13] + f[14], d1314 = f[13] - f[14];
-  const double s1516 = f[15] + f[16], d1516 = f[15] - f[16];
-  const double s1718 = f[17] + f[18], d1718 = f[17] - f[18];
-  // m = M f (Eq. 12), in deviation form (m - rho_ref M w)
-  const double m16 = s78 + s910, m17 = s1112 + s1314, m18 = s1516 + s1718;
-  const double m7 = s78 - s910, m8 = s1112 - s1314, m9 = s1516 - s1718;
-  const double Dx = (d78 + d910) + (d1112 + d1314);  // m11 + m13
-  const double Dy = (d78 - d910) + (d1516 + d1718);  // m10 + m15
-  const double Dz = (d1112 - d1314) + (d1516 - d1718);  // m12 + m14
-  const double syz = s34 + s56, sax = s12 + syz;
-  const double sxx = m16 + m17, sdg = sxx + m18;
-  const double drho = f[0] + sax + sdg;
-  const double m4 = fma(2.0, sdg, sax);
-  const double m5 = fma(2.0, s12 - m18, sxx - syz);
-  const double m6 = (s34 - s56) + (m16 - m17);
-  // macroscopic quantities, Eq. 6
-  const double rho = rho_ref + drho;
-  const double inv_rho = recip(rho);
-  const double rux = (d12 + Dx) + 0.5 * Fx, ruy = (d34 + Dy) + 0.5 * Fy, ruz = (d56 + Dz) + 0.5 * Fz;
-  const double ox = d12 + C.k[kQs] * Dx, oy = d34 + C.k[kQs] * Dy, oz = d56 + C.k[kQs] * Dz;
-  const double ux = rux * inv_rho, uy = ruy * inv_rho, uz = ruz * inv_rho;
-  const double qxx = rux * ux, qyy = ruy * uy, qzz = ruz * uz;  // rho u_i^2
-  const double usq = qxx + qyy + qzz;
-  const double Fux = Fx * ux, Fuy = Fy * uy, Fuz = Fz * uz;
-  const double Fu = Fux + Fuy + Fuz;
-  // relaxed moments (Eq. 4 with Eqs. 11, 13, 14, 16), scaled: e4 = m4* / 6, e5 = m5* / 12, e6 = m6* / 4,
-  // p_k = m_k* / 4
-  const double e4 = C.k[kE1] * m4 + C.k[kE2] * (drho + usq) + C.k[kE4] * Fu + C.k[kE5] * S2;
+// What the nonlinear parts need of a node's collision.
+struct Node64 {
+  double rho, Fx, Fy, Fz, S2;
+  double rux, ruy, ruz, ux, uy, uz, qxx, qyy, qzz, Fux, Fuy, Fuz;
+  // j: momenta of the populations; Eq. 6
+  __device__ __forceinline__ Node64(double rho_, double jx, double jy, double jz, double Fx_, double Fy_, double Fz_,
+                                    double S2_)
+      : rho(rho_), Fx(Fx_), Fy(Fy_), Fz(Fz_), S2(S2_) {
+    const double inv_rho = recip(rho);
+    rux = jx + 0.5 * Fx, ruy = jy + 0.5 * Fy, ruz = jz + 0.5 * Fz;
+    ux = rux * inv_rho, uy = ruy * inv_rho, uz = ruz * inv_rho;
+    qxx = rux * ux, qyy = ruy * uy, qzz = ruz * uz;  // rho u_i^2
+    Fux = Fx * ux, Fuy = Fy * uy, Fuz = Fz * uz;
+  }
+};
+
+// ------------------------------------------------------------------ non-orthogonal operator
+// f* = M^-1 m* (App. A) from drho, e4 = m4* / 6, e5 = m5* / 12, e6 = m6* / 4,
+// p_k = m_k* / 4 (16, 17, 18, 7, 8, 9), twice the odd parts of the axes, and the
+// odd parts of the diagonals.
+template <typename Sc, typename Out>
+__device__ __forceinline__ void inverse_nonorth_l(const double (&v)[19], const Sc &c, Out &&out) {
+  using L = typename Sc::Value;
+  const L e4 = c.in(v[1]), e5 = c.in(v[2]), e6 = c.in(v[3]);
+  const L p16 = c.in(v[4]), p17 = c.in(v[5]), p18 = c.in(v[6]);
+  const L a = p16 + p17;
+  out(0, fma(4.0, c.out(a + p18), fma(-6.0, v[1], v[0])));  // drho in the sums would set their cut
+  auto axis = [&](int k, const L &even2, double odd2) {  // both twice their value
+    const L o = c.in(odd2);
+    out(k, c.out_half(even2 + o));
+    out(k + 1, c.out_half(even2 - o));
+  };
+  const L e45 = e4 - e5;
+  axis(1, times<2>(e4 + times<2>(e5)) - times<4>(a), v[10]);
+  axis(3, times<2>(e45 + e6) - times<4>(p16 + p18), v[11]);
+  axis(5, times<2>(e45 - e6) - times<4>(p17 + p18), v[12]);
+  auto diagonal = [&](int k, const L &p, double shear, double odd1, double odd2) {
+    const L s = c.in(shear), o1 = c.in(odd1), o2 = c.in(odd2), ev = p + s, ew = p - s;
+    out(k, c.out(ev + o1));
+    out(k + 1, c.out(ev - o1));
+    out(k + 2, c.out(ew + o2));
+    out(k + 3, c.out(ew - o2));
+  };
+  diagonal(7, p16, v[7], v[13], v[14]);
+  diagonal(11, p17, v[8], v[15], v[16]);
+  diagonal(15, p18, v[9], v[17], v[18]);
+}
+
+// Forward chains of Eq. 12 (deviation form, m - rho_ref M w), equilibria Eq. 13,
+// forcing Eq. 14, the Eq. 16 term from S2 (the squared sum of Eq. 15).  f_ holds the
+// deviations f_a - w_a rho_ref; out(a, f*_a) takes the results (deviations again).
+template <typename Sc, typename Out>
+__device__ __forceinline__ void collide_nonorth_l(const double (&f_)[19], const Sc &c, double rho_ref, double Fx,
+                                                  double Fy, double Fz, double S2, const KParams &P, const Coeffs64 &C,
+                                                  Out &&out) {
+  using L = typename Sc::Value;
+  L f[19];
+#pragma unroll
+  for (int a = 0; a < 19; ++a) f[a] = c.in(f_[a]);
+  const L s12 = f[1] + f[2], d12 = f[1] - f[2];
+  const L s34 = f[3] + f[4], d34 = f[3] - f[4];
+  const L s56 = f[5] + f[6], d56 = f[5] - f[6];
+  const L s78 = f[7] + f[8], d78 = f[7] - f[8];
+  const L s910 = f[9] + f[10], d910 = f[9] - f[10];
+  const L s1112 = f[11] + f[12], d1112 = f[11] - f[12];
+  const L s1314 = f[13] + f[14], d1314 = f[13] - f[14];
+  const L s1516 = f[15] + f[16], d1516 = f[15] - f[16];
+  const L s1718 = f[17] + f[18], d1718 = f[17] - f[18];
+  const L l16 = s78 + s910, l17 = s1112 + s1314, l18 = s1516 + s1718;
+  const L lx = (d78 + d910) + (d1112 + d1314);    // m11 + m13
+  const L ly = (d78 - d910) + (d1516 + d1718);    // m10 + m15
+  const L lz = (d1112 - d1314) + (d1516 - d1718);  // m12 + m14
+  const L syz = s34 + s56, sax = s12 + syz, sxx = l16 + l17, sdg = sxx + l18;
+  const double drho = c.out(f[0] + sax + sdg);
+  const double Dx = c.out(lx), Dy = c.out(ly), Dz = c.out(lz);
+  const double jx = c.out(d12 + lx), jy = c.out(d34 + ly), jz = c.out(d56 + lz);
+  const Node64 N(rho_ref + drho, jx, jy, jz, Fx, Fy, Fz, S2);
+  const double usq = N.qxx + N.qyy + N.qzz, Fu = N.Fux + N.Fuy + N.Fuz;
+  double v[19];
+  v[0] = drho;
+  // relaxed moments (Eq. 4 with Eqs. 11, 13, 14, 16), scaled as the inverse takes them
+  v[1] = C.k[kE1] * c.out(sax + times<2>(sdg)) + C.k[kE2] * (drho + usq) + C.k[kE4] * Fu + C.k[kE5] * S2;
   // Eq. 13's phi + (rho - rho_ref)/9 and third-axis parts: m16 takes the sum over the axes less the z part, ...
   const double c4 = C.k[kP2] * drho + C.k[kP3] * usq + C.k[kP4] * Fu;
-  const double p16 = C.k[kP1] * m16 + (c4 - (C.k[kP5] * qzz + C.k[kP4] * Fuz));
-  const double p17 = C.k[kP1] * m17 + (c4 - (C.k[kP5] * qyy + C.k[kP4] * Fuy));
-  const double p18 = C.k[kP1] * m18 + (c4 - (C.k[kP5] * qxx + C.k[kP4] * Fux));
-  out(0, (drho - 6.0 * e4) + 4.0 * ((p16 + p17) + p18));
-  const Shear64 n = shear64<19>(P, C, rho);
-  const double Bx = n.b1 * rux + n.b2 * Fx, By = n.b1 * ruy + n.b2 * Fy, Bz = n.b1 * ruz + n.b2 * Fz;
-  const double Gx = ux * Bx, Gy = uy * By, Gz = uz * Bz;
-  const double e5 = fma(-2.0 / 3.0, fma(-2.0, Gx, Gy + Gz), n.n5 * m5);
-  const double e6 = fma(2.0, Gy - Gz, n.n7 * m6);
-  // f* = M^-1 m* (App. A); odd parts: b_i carries Eq. 13/14's rho u_i / 3 and F_i / 3 of the third-order moments
-  const double bx = C.k[kQb1] * rux + C.k[kQb2] * Fx, by = C.k[kQb1] * ruy + C.k[kQb2] * Fy;
-  const double bz = C.k[kQb1] * ruz + C.k[kQb2] * Fz;
-  const double h = 0.5;
-  const double e45 = e4 - e5;
-  {
-    const double even = fma(-2.0, p16 + p17, fma(2.0, e5, e4)), odd = (ox + Fx) - 8.0 * bx;
-    out(1, even + h * odd);
-    out(2, even - h * odd);
+  v[4] = C.k[kP1] * c.out(l16) + (c4 - (C.k[kP5] * N.qzz + C.k[kP4] * N.Fuz));
+  v[5] = C.k[kP1] * c.out(l17) + (c4 - (C.k[kP5] * N.qyy + C.k[kP4] * N.Fuy));
+  v[6] = C.k[kP1] * c.out(l18) + (c4 - (C.k[kP5] * N.qxx + C.k[kP4] * N.Fux));
+  const Shear64 n = shear64<19>(P, C, N.rho);
+  const double Bx = n.b1 * N.rux + n.b2 * Fx, By = n.b1 * N.ruy + n.b2 * Fy, Bz = n.b1 * N.ruz + n.b2 * Fz;
+  const double Gx = N.ux * Bx, Gy = N.uy * By, Gz = N.uz * Bz;
+  v[2] = fma(-2.0 / 3.0, fma(-2.0, Gx, Gy + Gz), n.n5 * c.out(times<2>(s12 - l18) + (sxx - syz)));
+  v[3] = fma(2.0, Gy - Gz, n.n7 * c.out((s34 - s56) + (l16 - l17)));
+  v[7] = n.n7 * c.out(s78 - s910) + N.ux * By + N.uy * Bx;
+  v[8] = n.n7 * c.out(s1112 - s1314) + N.ux * Bz + N.uz * Bx;
+  v[9] = n.n7 * c.out(s1516 - s1718) + N.uy * Bz + N.uz * By;
+  // odd parts: b_i carries Eq. 13/14's rho u_i / 3 and F_i / 3 of the third-order moments; 2 kQa = 1 - s_q
+  const double bx = C.k[kQb1] * N.rux + C.k[kQb2] * Fx, by = C.k[kQb1] * N.ruy + C.k[kQb2] * Fy;
+  const double bz = C.k[kQb1] * N.ruz + C.k[kQb2] * Fz, qa = C.k[kQa], q2 = -C.k[kQ2];
+  v[10] = fma(-8.0, bx, fma(q2, Dx, jx + Fx));
+  v[11] = fma(-8.0, by, fma(q2, Dy, jy + Fy));
+  v[12] = fma(-8.0, bz, fma(q2, Dz, jz + Fz));
+  v[13] = qa * c.out(d78) + (bx + by);
+  v[14] = qa * c.out(d910) + (bx - by);
+  v[15] = qa * c.out(d1112) + (bx + bz);
+  v[16] = qa * c.out(d1314) + (bx - bz);
+  v[17] = qa * c.out(d1516) + (by + bz);
+  v[18] = qa * c.out(d1718) + (by - bz);
+  const int E = std::is_same<Sc, InDouble>::value ? -1 : top_exponent<1>(v);
+  if (E >= 0)
+    inverse_nonorth_l(v, InFixed<6>{E}, out);
+  else
+    inverse_nonorth_l(v, InDouble{}, out);
+}
+
+// ------------------------------------------------------------------ orthogonal operator
+// d'Humieres et al. D3Q19 basis at the Eq. 2 ordering: m = M_o f, m_eq = M_o f_eq,
+// S = M_o G (Guo), f* = M_o^T diag(1/|row|^2) m*.  The Eq. 16 term enters as
+// dS4 * (0, 19, -16, 0, ...), its image in this basis.
+// v: n_k = m_k* / |row k|^2 for k = 0, 1, 2, 9, 10, 11, a third of 12, 16, 17, 18, 13,
+// 15, 14 (xy, xz, yz), then j*/10 and q*/40 of x, y, z.
+template <typename Sc, typename Out>
+__device__ __forceinline__ void inverse_orth_l(const double (&v)[19], const Sc &c, Out &&out) {
+  using L = typename Sc::Value;
+  const L n0 = c.in(v[0]), n1 = c.in(v[1]), n2 = c.in(v[2]);
+  out(0, c.out_twice((c.half(n0) - times<15>(n1)) + times<6>(n2)));
+  const L Ca = (n0 - times<11>(n1)) - times<4>(n2), Cd = (n0 + times<8>(n1)) + n2;
+  const L n9 = c.in(v[3]), n10 = c.in(v[4]), n11 = c.in(v[5]), n12 = c.in(v[6]);
+  // axis parts of the stresses: x gets 2 q9, y and z -q9 +- w11
+  const L q9 = n9 - times<2>(n10), w11 = n11 - times<6>(n12), r9 = n9 + n10, r11 = n11 + times<3>(n12);
+  const L gx = c.in(v[13]), gy = c.in(v[14]), gz = c.in(v[15]), hx = c.in(v[16]), hy = c.in(v[17]), hz = c.in(v[18]);
+  auto pair = [&](int k, const L &even, const L &odd) {
+    out(k, c.out(even + odd));
+    out(k + 1, c.out(even - odd));
+  };
+  pair(1, Ca + times<2>(q9), gx - times<4>(hx));
+  pair(3, (Ca - q9) + w11, gy - times<4>(hy));
+  pair(5, (Ca - q9) - w11, gz - times<4>(hz));
+  const L X = gx + hx, Y = gy + hy, Z = gz + hz, Cr = Cd + r9;
+  const L n16 = c.in(v[7]), n17 = c.in(v[8]), n18 = c.in(v[9]);
+  {  // xy diagonals 7..10: signs of (p_xy, m_x, m_y) are (+,+,-), (+,-,+), (-,+,+), (-,-,-)
+    const L e = Cr + r11, s = c.in(v[10]);
+    pair(7, e + s, (X + Y) + (n16 - n17));
+    pair(9, e - s, (X - Y) + (n16 + n17));
   }
-  {
-    const double even = fma(-2.0, p16 + p18, e45 + e6), odd = (oy + Fy) - 8.0 * by;
-    out(3, even + h * odd);
-    out(4, even - h * odd);
+  {  // xz diagonals 11..14: signs of (p_xz, m_x, m_z) are (+,-,+), (+,+,-), (-,-,-), (-,+,+)
+    const L e = Cr - r11, s = c.in(v[11]);
+    pair(11, e + s, (X + Z) + (n18 - n16));
+    pair(13, e - s, (X - Z) - (n16 + n18));
   }
-  {
-    const double even = fma(-2.0, p17 + p18, e45 - e6), odd = (oz + Fz) - 8.0 * bz;
-    out(5, even + h * odd);
-    out(6, even - h * odd);
-  }
-  {
-    const double p7 = n.n7 * m7 + ux * By + uy * Bx;
-    const double ev = p16 + p7, od = C.k[kQa] * d78 + (bx + by), ew = p16 - p7, oe = C.k[kQa] * d910 + (bx - by);
-    out(7, ev + od);
-    out(8, ev - od);
-    out(9, ew + oe);
-    out(10, ew - oe);
-  }
-  {
-    const double p8 = n.n7 * m8 + ux * Bz + uz * Bx;
-    const double ev = p17 + p8, od = C.k[kQa] * d1112 + (bx + bz), ew = p17 - p8, oe = C.k[kQa] * d1314 + (bx - bz);
-    out(11, ev + od);
-    out(12, ev - od);
-    out(13, ew + oe);
-    out(14, ew - oe);
-  }
-  {
-    const double p9 = n.n7 * m9 + uy * Bz + uz * By;
-    const double ev = p18 + p9, od = C.k[kQa] * d1516 + (by + bz), ew = p18 - p9, oe = C.k[kQa] * d1718 + (by - bz);
-    out(15, ev + od);
-    out(16, ev - od);
-    out(17, ew + oe);
-    out(18, ew - oe);
+  {  // yz diagonals 15..18: signs of (p_yz, m_y, m_z) are (+,+,-), (+,-,+), (-,+,+), (-,-,-)
+    const L e = Cd - times<2>(r9), s = c.in(v[12]);
+    pair(15, e + s, (Y + Z) + (n17 - n18));
+    pair(17, e - s, (Y - Z) + (n17 + n18));
   }
 }
 
-// Orthogonal operator (d'Humieres et al. D3Q19 basis at the Eq. 2 ordering):
-// m = M_o f, m_eq = M_o f_eq, S = M_o G (Guo), f* = M_o^T diag(1/|row|^2) m*.
-// The Eq. 16 term enters as dS4 * (0, 19, -16, 0, ...), its image in this basis.
-template <typename Out>
-__device__ __forceinline__ void collide_orth64(const double f[19], double rho_ref, double Fx, double Fy, double Fz,
-                                                  double S2, const KParams &P, const Coeffs64 &C, Out &&out) {
-  const double s12 = f[1] + f[2], d12 = f[1] - f[2];
-  const double s34 = f[3] + f[4], d34 = f[3] - f[4];
-  const double s56 = f[5] + f[6], d56 = f[5] - f[6];
-  const double s78 = f[7] + f[8], d78 = f[7] - f[8];
-  const double s910 = f[9] + f[10], d910 = f[9] - f[10];
-  const double s1112 = f[11] + f[12], d1112 = f[11] - f[12];
-  const double s1314 = f[13] + f[14], d1314 = f[13] - f[14];
-  const double s1516 = f[15] + f[16], d1516 = f[15] - f[16];
-  const double s1718 = f[17] + f[18], d1718 = f[17] - f[18];
-  const double sxy = s78 + s910, sxz = s1112 + s1314, syz = s1516 + s1718;
-  const double sp = s34 + s56, sm = s34 - s56;
-  const double A = s12 + sp, sxyz = sxy + sxz, B = sxyz + syz;
-  const double drho = f[0] + A + B;
+template <typename Sc, typename Out>
+__device__ __forceinline__ void collide_orth_l(const double (&f_)[19], const Sc &c, double rho_ref, double Fx,
+                                               double Fy, double Fz, double S2, const KParams &P, const Coeffs64 &C,
+                                               Out &&out) {
+  using L = typename Sc::Value;
+  L f[19];
+#pragma unroll
+  for (int a = 0; a < 19; ++a) f[a] = c.in(f_[a]);
+  const L s12 = f[1] + f[2], d12 = f[1] - f[2];
+  const L s34 = f[3] + f[4], d34 = f[3] - f[4];
+  const L s56 = f[5] + f[6], d56 = f[5] - f[6];
+  const L s78 = f[7] + f[8], d78 = f[7] - f[8];
+  const L s910 = f[9] + f[10], d910 = f[9] - f[10];
+  const L s1112 = f[11] + f[12], d1112 = f[11] - f[12];
+  const L s1314 = f[13] + f[14], d1314 = f[13] - f[14];
+  const L s1516 = f[15] + f[16], d1516 = f[15] - f[16];
+  const L s1718 = f[17] + f[18], d1718 = f[17] - f[18];
+  const L sxy = s78 + s910, sxz = s1112 + s1314, syz = s1516 + s1718;
+  const L sp = s34 + s56, sm = s34 - s56, lA = s12 + sp, sxyz = sxy + sxz, lB = sxyz + syz;
   // diagonal parts of the momenta, plane by plane
-  const double x1 = d78 + d910, y1 = d78 - d910;
-  const double x2 = d1112 + d1314, z1 = d1112 - d1314;
-  const double y2 = d1516 + d1718, z2 = d1516 - d1718;
-  const double dx = x1 + x2, dy = y1 + y2, dz = z1 + z2;
-  const double jx = d12 + dx, jy = d34 + dy, jz = d56 + dz;
-  // macroscopic quantities, Eq. 6
-  const double rho = rho_ref + drho;
-  const double inv_rho = recip(rho);
-  const double rux = jx + 0.5 * Fx, ruy = jy + 0.5 * Fy, ruz = jz + 0.5 * Fz;
-  const double ux = rux * inv_rho, uy = ruy * inv_rho, uz = ruz * inv_rho;
-  const double qxx = rux * ux, qyy = ruy * uy, qzz = ruz * uz;
-  const double qp = qyy + qzz, usq = qxx + qp;
-  const double Fux = Fx * ux, Fuy = Fy * uy, Fuz = Fz * uz;
-  const double Fp = Fuy + Fuz, Fu = Fux + Fp;
-  // relaxed moments over the squared row norms: n_k = m_k* / |row k|^2 (the numbers are the rows')
-  const double n0 = 1.0 / 19.0 * drho;
-  const double n1 = C.k[kE1] * fma(2.0, B, A) + C.k[kE2] * drho + C.k[kE3] * usq + C.k[kE4] * Fu + C.k[kE5] * S2;
-  const double n2 = C.k[kO1] * A + C.k[kO2] * B + C.k[kO3] * drho + C.k[kO4] * usq + C.k[kO5] * Fu + C.k[kO6] * S2;
-  out(0, (n0 - 30.0 * n1) + 12.0 * n2);
-  const double Ca = (n0 - 11.0 * n1) - 4.0 * n2;
-  const double Cd = (n0 + 8.0 * n1) + n2;
-  const Shear64 n = shear64<19>(P, C, rho);
-  const double Bx = n.b1 * rux + n.b2 * Fx, By = n.b1 * ruy + n.b2 * Fy, Bz = n.b1 * ruz + n.b2 * Fz;
-  const double Gx = ux * Bx, Gy = uy * By, Gz = uz * Bz;
-  const double a9 = fma(-2.0, s12, sp), b9 = fma(-2.0, syz, sxyz), b11 = sxy - sxz;
-  const double n9 = fma(-2.0 / 9.0, fma(-2.0, Gx, Gy + Gz), n.nx * (b9 - a9));
-  const double n11 = n.n5 * (sm + b11) + 2.0 / 3.0 * (Gy - Gz);
-  const double n10 = C.k[kP1] * fma(2.0, a9, b9) + C.k[kP2] * fma(-2.0, qxx, qp) + C.k[kP3] * fma(-2.0, Fux, Fp);
-  const double n12 = C.k[kP1] * fma(-2.0, sm, b11) + C.k[kP2] * (qzz - qyy) + C.k[kP3] * (Fuz - Fuy);  // a third of it
-  const double q9 = fma(-2.0, n10, n9), w11 = n11 - 6.0 * n12;  // axis parts of the stresses: x gets 2 q9, y and z -q9 +- w11
-  const double r9 = n9 + n10, r11 = n11 + 3.0 * n12;
-  const double n16 = C.k[kOm] * (x1 - x2), n17 = C.k[kOm] * (y2 - y1), n18 = C.k[kOm] * (z1 - z2);
-  // odd parts of an axis: j* / 10 and q* / 40; xo, yo, zo on the axis, X, Y, Z on the diagonals
-  const double gx = 0.1 * (jx + Fx), gy = 0.1 * (jy + Fy), gz = 0.1 * (jz + Fz);
-  const double hx = C.k[kQa] * (dx - 4.0 * d12) - (C.k[kQb1] * rux + C.k[kQb2] * Fx);
-  const double hy = C.k[kQa] * (dy - 4.0 * d34) - (C.k[kQb1] * ruy + C.k[kQb2] * Fy);
-  const double hz = C.k[kQa] * (dz - 4.0 * d56) - (C.k[kQb1] * ruz + C.k[kQb2] * Fz);
-  const double xo = gx - 4.0 * hx, yo = gy - 4.0 * hy, zo = gz - 4.0 * hz;
-  const double X = gx + hx, Y = gy + hy, Z = gz + hz;
-  {
-    const double cx = fma(2.0, q9, Ca), cy = (Ca - q9) + w11, cz = (Ca - q9) - w11;
-    out(1, cx + xo);
-    out(2, cx - xo);
-    out(3, cy + yo);
-    out(4, cy - yo);
-    out(5, cz + zo);
-    out(6, cz - zo);
-  }
-  const double Cr = Cd + r9;
-  // xy diagonals 7..10: signs of (p_xy, m_x, m_y) are (+,+,-), (+,-,+), (-,+,+), (-,-,-)
-  {
-    const double E = Cr + r11, n13 = n.n7 * (s78 - s910) + ux * By + uy * Bx;
-    const double ev = E + n13, od = (X + Y) + (n16 - n17), ew = E - n13, oe = (X - Y) + (n16 + n17);
-    out(7, ev + od);
-    out(8, ev - od);
-    out(9, ew + oe);
-    out(10, ew - oe);
-  }
-  // xz diagonals 11..14: signs of (p_xz, m_x, m_z) are (+,-,+), (+,+,-), (-,-,-), (-,+,+)
-  {
-    const double E = Cr - r11, n15 = n.n7 * (s1112 - s1314) + ux * Bz + uz * Bx;
-    const double ev = E + n15, od = (X + Z) + (n18 - n16), ew = E - n15, oe = (X - Z) - (n16 + n18);
-    out(11, ev + od);
-    out(12, ev - od);
-    out(13, ew + oe);
-    out(14, ew - oe);
-  }
-  // yz diagonals 15..18: signs of (p_yz, m_y, m_z) are (+,+,-), (+,-,+), (-,+,+), (-,-,-)
-  {
-    const double E = fma(-2.0, r9, Cd), n14 = n.n7 * (s1516 - s1718) + uy * Bz + uz * By;
-    const double ev = E + n14, od = (Y + Z) + (n17 - n18), ew = E - n14, oe = (Y - Z) + (n17 + n18);
-    out(15, ev + od);
-    out(16, ev - od);
-    out(17, ew + oe);
-    out(18, ew - oe);
-  }
+  const L x1 = d78 + d910, y1 = d78 - d910, x2 = d1112 + d1314, z1 = d1112 - d1314, y2 = d1516 + d1718, z2 = d1516 - d1718;
+  const L dx = x1 + x2, dy = y1 + y2, dz = z1 + z2;
+  const double drho = c.out(f[0] + lA + lB), A = c.out(lA), B = c.out(lB);
+  const double jx = c.out(d12 + dx), jy = c.out(d34 + dy), jz = c.out(d56 + dz);
+  const Node64 N(rho_ref + drho, jx, jy, jz, Fx, Fy, Fz, S2);
+  const double qp = N.qyy + N.qzz, usq = N.qxx + qp, Fp = N.Fuy + N.Fuz, Fu = N.Fux + Fp;
+  double v[19];
+  v[0] = (1.0 / 19.0) * drho;
+  v[1] = C.k[kE1] * fma(2.0, B, A) + C.k[kE2] * drho + C.k[kE3] * usq + C.k[kE4] * Fu + C.k[kE5] * S2;
+  v[2] = C.k[kO1] * A + C.k[kO2] * B + C.k[kO3] * drho + C.k[kO4] * usq + C.k[kO5] * Fu + C.k[kO6] * S2;
+  const Shear64 n = shear64<19>(P, C, N.rho);
+  const double Bx = n.b1 * N.rux + n.b2 * Fx, By = n.b1 * N.ruy + n.b2 * Fy, Bz = n.b1 * N.ruz + n.b2 * Fz;
+  const double Gx = N.ux * Bx, Gy = N.uy * By, Gz = N.uz * Bz;
+  const L a9 = sp - times<2>(s12), b9 = sxyz - times<2>(syz), b11 = sxy - sxz;
+  v[3] = fma(-2.0 / 9.0, fma(-2.0, Gx, Gy + Gz), n.nx * c.out(b9 - a9));
+  v[4] = C.k[kP1] * c.out(b9 + times<2>(a9)) + C.k[kP2] * fma(-2.0, N.qxx, qp) + C.k[kP3] * fma(-2.0, N.Fux, Fp);
+  v[5] = n.n5 * c.out(sm + b11) + (2.0 / 3.0) * (Gy - Gz);
+  v[6] = C.k[kP1] * c.out(b11 - times<2>(sm)) + C.k[kP2] * (N.qzz - N.qyy) + C.k[kP3] * (N.Fuz - N.Fuy);
+  v[7] = C.k[kOm] * c.out(x1 - x2);
+  v[8] = C.k[kOm] * c.out(y2 - y1);
+  v[9] = C.k[kOm] * c.out(z1 - z2);
+  v[10] = n.n7 * c.out(s78 - s910) + N.ux * By + N.uy * Bx;
+  v[11] = n.n7 * c.out(s1112 - s1314) + N.ux * Bz + N.uz * Bx;
+  v[12] = n.n7 * c.out(s1516 - s1718) + N.uy * Bz + N.uz * By;
+  v[13] = 0.1 * (jx + Fx);
+  v[14] = 0.1 * (jy + Fy);
+  v[15] = 0.1 * (jz + Fz);
+  v[16] = C.k[kQa] * c.out(dx - times<4>(d12)) - (C.k[kQb1] * N.rux + C.k[kQb2] * Fx);
+  v[17] = C.k[kQa] * c.out(dy - times<4>(d34)) - (C.k[kQb1] * N.ruy + C.k[kQb2] * Fy);
+  v[18] = C.k[kQa] * c.out(dz - times<4>(d56)) - (C.k[kQb1] * N.ruz + C.k[kQb2] * Fz);
+  const int E = std::is_same<Sc, InDouble>::value ? -1 : top_exponent(v);
+  if (E >= 0)
+    inverse_orth_l(v, InFixed<5>{E}, out);
+  else
+    inverse_orth_l(v, InDouble{}, out);
 }
 
-// D3Q15 (the basis and readings of lbm_q15.cuh); the four odd corner moments
-// relax with one rate, so the corner differences relax themselves.
-template <typename Out>
-__device__ __forceinline__ void collide_q15_64(const double f[15], double rho_ref, double Fx, double Fy, double Fz,
-                                                  double S2, const KParams &P, const Coeffs64 &C, Out &&out) {
-  // axis pairs
-  const double s12 = f[1] + f[2], d12 = f[1] - f[2];
-  const double s34 = f[3] + f[4], d34 = f[3] - f[4];
-  const double s56 = f[5] + f[6], d56 = f[5] - f[6];
-  // corner pairs -> even (count, e_x e_y, e_x e_z, e_y e_z) moments by two
-  // butterfly stages; corner parts of e_x, e_y, e_z
-  const double s78 = f[7] + f[8], d78 = f[7] - f[8];
-  const double s910 = f[9] + f[10], d910 = f[9] - f[10];
-  const double s1112 = f[11] + f[12], d1112 = f[11] - f[12];
-  const double s1314 = f[13] + f[14], d1314 = f[13] - f[14];
-  const double u1 = s78 + s910, u2 = s1112 + s1314, v1 = s78 - s910, v2 = s1112 - s1314;
-  const double m14 = u1 + u2, m7 = u1 - u2, m8 = v1 + v2, m9 = v1 - v2;
-  const double U1 = d78 + d910, U2 = d1112 - d1314;
-  const double Dx = U1 + U2, Dy = U1 - U2, Dz = (d78 - d910) + (d1112 + d1314);
-  const double syz = s34 + s56, sax = s12 + syz;
-  const double drho = f[0] + sax + m14;
-  const double m4 = sax + 3.0 * m14;
-  const double m5 = fma(-2.0, s12, syz);  // negated, and e5 below
-  const double m6 = s34 - s56;
-  // macroscopic quantities, Eq. 6
-  const double rho = rho_ref + drho;
-  const double inv_rho = recip(rho);
-  const double rux = (d12 + Dx) + 0.5 * Fx, ruy = (d34 + Dy) + 0.5 * Fy, ruz = (d56 + Dz) + 0.5 * Fz;
-  const double ux = rux * inv_rho, uy = ruy * inv_rho, uz = ruz * inv_rho;
-  const double usq = rux * ux + ruy * uy + ruz * uz;  // rho |u|^2
-  const double Fu = Fx * ux + Fy * uy + Fz * uz;
-  // relaxed moments, scaled: e4 = m4* / 6, e5 = -m5* / 12, e6 = m6* / 4, p_k = m_k* / 8
-  const double e4 = C.k[kE1] * m4 + C.k[kE2] * (drho + usq) + C.k[kE4] * Fu + C.k[kE5] * S2;
-  const double p14 = C.k[kP1] * m14 + C.k[kP2] * drho + C.k[kP3] * usq + C.k[kP4] * Fu;
-  out(0, (drho - 6.0 * e4) + 16.0 * p14);
-  const Shear64 n = shear64<15>(P, C, rho);
-  const double Bx = n.b1 * rux + n.b2 * Fx, By = n.b1 * ruy + n.b2 * Fy, Bz = n.b1 * ruz + n.b2 * Fz;
-  const double Gx = ux * Bx, Gy = uy * By, Gz = uz * Bz;
-  const double e5 = fma(4.0 / 3.0, fma(-2.0, Gx, Gy + Gz), n.n5 * m5);
-  const double e6 = n.n7 * m6 + 4.0 * (Gy - Gz);
-  const double p7 = n.nx * m7 + ux * By + uy * Bx;
-  const double p8 = n.nx * m8 + ux * Bz + uz * Bx;
-  const double p9 = n.nx * m9 + uy * Bz + uz * By;
-  // f* = M^-1 m*
-  const double bx = C.k[kQb1] * rux + C.k[kQb2] * Fx, by = C.k[kQb1] * ruy + C.k[kQb2] * Fy;
-  const double bz = C.k[kQb1] * ruz + C.k[kQb2] * Fz;
-  const double h = 0.5;
-  const double c4 = e4 - 4.0 * p14, c45 = c4 + e5;
-  {
-    const double even = fma(-2.0, e5, c4), odd = ((d12 + Fx) + C.k[kQs] * Dx) - 8.0 * bx;
-    out(1, even + h * odd);
-    out(2, even - h * odd);
-  }
-  {
-    const double even = c45 + e6, odd = ((d34 + Fy) + C.k[kQs] * Dy) - 8.0 * by;
-    out(3, even + h * odd);
-    out(4, even - h * odd);
-  }
-  {
-    const double even = c45 - e6, odd = ((d56 + Fz) + C.k[kQs] * Dz) - 8.0 * bz;
-    out(5, even + h * odd);
-    out(6, even - h * odd);
-  }
-  const double q1 = p14 + p7, q2 = p8 + p9, q3 = p14 - p7, q4 = p8 - p9;
-  const double bp = bx + by, bm = bx - by;
-  {
-    const double ev = q1 + q2, od = C.k[kQa] * d78 + (bp + bz), ew = q1 - q2, oe = C.k[kQa] * d910 + (bp - bz);
-    out(7, ev + od);
-    out(8, ev - od);
-    out(9, ew + oe);
-    out(10, ew - oe);
-  }
-  {
-    const double ev = q3 + q4, od = C.k[kQa] * d1112 + (bm + bz), ew = q3 - q4, oe = C.k[kQa] * d1314 - (bm - bz);
-    out(11, ev + od);
-    out(12, ev - od);
-    out(13, ew + oe);
-    out(14, ew - oe);
-  }
+// ------------------------------------------------------------------ D3Q15
+// The basis and readings of lbm_q15.cuh; the four odd corner moments relax with one
+// rate, so the corner differences relax themselves.  v: drho, m4* / 6, -m5* / 12,
+// m6* / 4, m_k* / 8 (14, 7, 8, 9), twice the odd parts of the axes, the odd parts of
+// the corner pairs.
+template <typename Sc, typename Out>
+__device__ __forceinline__ void inverse_q15_l(const double (&v)[15], const Sc &c, Out &&out) {
+  using L = typename Sc::Value;
+  const L e4 = c.in(v[1]), e5 = c.in(v[2]), e6 = c.in(v[3]), p14 = c.in(v[4]);
+  out(0, fma(16.0, v[4], fma(-6.0, v[1], v[0])));
+  auto axis = [&](int k, const L &even, double odd2) {
+    const L e = times<2>(even), o = c.in(odd2);
+    out(k, c.out_half(e + o));
+    out(k + 1, c.out_half(e - o));
+  };
+  const L c4 = e4 - times<4>(p14), c45 = c4 + e5;
+  axis(1, c4 - times<2>(e5), v[8]);
+  axis(3, c45 + e6, v[9]);
+  axis(5, c45 - e6, v[10]);
+  const L p7 = c.in(v[5]), p8 = c.in(v[6]), p9 = c.in(v[7]);
+  const L q1 = p14 + p7, q2 = p8 + p9, q3 = p14 - p7, q4 = p8 - p9;
+  auto corner = [&](int k, const L &even, double odd) {
+    const L o = c.in(odd);
+    out(k, c.out(even + o));
+    out(k + 1, c.out(even - o));
+  };
+  corner(7, q1 + q2, v[11]);
+  corner(9, q1 - q2, v[12]);
+  corner(11, q3 + q4, v[13]);
+  corner(13, q3 - q4, v[14]);
+}
+
+template <typename Sc, typename Out>
+__device__ __forceinline__ void collide_q15_l(const double (&f_)[15], const Sc &c, double rho_ref, double Fx,
+                                              double Fy, double Fz, double S2, const KParams &P, const Coeffs64 &C,
+                                              Out &&out) {
+  using L = typename Sc::Value;
+  L f[15];
+#pragma unroll
+  for (int a = 0; a < 15; ++a) f[a] = c.in(f_[a]);
+  const L s12 = f[1] + f[2], d12 = f[1] - f[2];
+  const L s34 = f[3] + f[4], d34 = f[3] - f[4];
+  const L s56 = f[5] + f[6], d56 = f[5] - f[6];
+  // corner pairs -> even (count, e_x e_y, e_x e_z, e_y e_z) moments by two butterfly stages; corner parts of e_x, ...
+  const L s78 = f[7] + f[8], d78 = f[7] - f[8];
+  const L s910 = f[9] + f[10], d910 = f[9] - f[10];
+  const L s1112 = f[11] + f[12], d1112 = f[11] - f[12];
+  const L s1314 = f[13] + f[14], d1314 = f[13] - f[14];
+  const L u1 = s78 + s910, u2 = s1112 + s1314, v1 = s78 - s910, v2 = s1112 - s1314, l14 = u1 + u2;
+  const L U1 = d78 + d910, U2 = d1112 - d1314;
+  const L lx = U1 + U2, ly = U1 - U2, lz = (d78 - d910) + (d1112 + d1314);
+  const L syz = s34 + s56, sax = s12 + syz;
+  const double drho = c.out(f[0] + sax + l14);
+  const double Dx = c.out(lx), Dy = c.out(ly), Dz = c.out(lz);
+  const double jx = c.out(d12 + lx), jy = c.out(d34 + ly), jz = c.out(d56 + lz);
+  const Node64 N(rho_ref + drho, jx, jy, jz, Fx, Fy, Fz, S2);
+  const double usq = N.qxx + N.qyy + N.qzz, Fu = N.Fux + N.Fuy + N.Fuz;
+  double v[15];
+  v[0] = drho;
+  v[1] = C.k[kE1] * c.out(sax + times<3>(l14)) + C.k[kE2] * (drho + usq) + C.k[kE4] * Fu + C.k[kE5] * S2;
+  v[4] = C.k[kP1] * c.out(l14) + C.k[kP2] * drho + C.k[kP3] * usq + C.k[kP4] * Fu;
+  const Shear64 n = shear64<15>(P, C, N.rho);
+  const double Bx = n.b1 * N.rux + n.b2 * Fx, By = n.b1 * N.ruy + n.b2 * Fy, Bz = n.b1 * N.ruz + n.b2 * Fz;
+  const double Gx = N.ux * Bx, Gy = N.uy * By, Gz = N.uz * Bz;
+  v[2] = fma(4.0 / 3.0, fma(-2.0, Gx, Gy + Gz), n.n5 * c.out(syz - times<2>(s12)));
+  v[3] = fma(4.0, Gy - Gz, n.n7 * c.out(s34 - s56));
+  v[5] = n.nx * c.out(u1 - u2) + N.ux * By + N.uy * Bx;
+  v[6] = n.nx * c.out(v1 + v2) + N.ux * Bz + N.uz * Bx;
+  v[7] = n.nx * c.out(v1 - v2) + N.uy * Bz + N.uz * By;
+  const double bx = C.k[kQb1] * N.rux + C.k[kQb2] * Fx, by = C.k[kQb1] * N.ruy + C.k[kQb2] * Fy;
+  const double bz = C.k[kQb1] * N.ruz + C.k[kQb2] * Fz, qa = C.k[kQa], q2 = -C.k[kQ2], bp = bx + by, bm = bx - by;
+  v[8] = fma(-8.0, bx, fma(q2, Dx, jx + Fx));
+  v[9] = fma(-8.0, by, fma(q2, Dy, jy + Fy));
+  v[10] = fma(-8.0, bz, fma(q2, Dz, jz + Fz));
+  v[11] = qa * c.out(d78) + (bp + bz);
+  v[12] = qa * c.out(d910) + (bp - bz);
+  v[13] = qa * c.out(d1112) + (bm + bz);
+  v[14] = qa * c.out(d1314) - (bm - bz);
+  const int E = std::is_same<Sc, InDouble>::value ? -1 : top_exponent<1>(v);
+  if (E >= 0)
+    inverse_q15_l(v, InFixed<6>{E}, out);
+  else
+    inverse_q15_l(v, InDouble{}, out);
+}
+
+// Collision of a node of operator OP: linear parts in fixed point where the populations allow it.
+template <int OP, int N, typename Out>
+__device__ __forceinline__ void collide64(const double (&f)[N], double rho_ref, double Fx, double Fy, double Fz, double S2,
+                                          const KParams &P, const Coeffs64 &C, Out &&out) {
+  auto run = [&](const auto &scale) {
+    if constexpr (N == 15)
+      collide_q15_l(f, scale, rho_ref, Fx, Fy, Fz, S2, P, C, out);
+    else if constexpr (OP == kNonOrth)
+      collide_nonorth_l(f, scale, rho_ref, Fx, Fy, Fz, S2, P, C, out);
+    else
+      collide_orth_l(f, scale, rho_ref, Fx, Fy, Fz, S2, P, C, out);
+  };
+  const int E = top_exponent(f);
+  if (E >= 0)
+    run(InFixed<5>{E});  // factors up to 32
+  else
+    run(InDouble{});
 }
 
 }  // namespace lbm

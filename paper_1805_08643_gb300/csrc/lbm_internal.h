@@ -127,7 +127,7 @@ inline dim3 plane_grid(int per_plane, int nz, int threads = kThreads) {
 // the predecessor has completed, so only the launch itself overlaps: 64^3 FP16
 // steps 16.4 -> 12.1 us, 127^3 FP32 (odd) 92 -> 84.  Blocks that come in this
 // way fill one SM after the other, so a grid that would not fill the device has
-// to start by itself: FP64 steps of 32^3 (1024 warps) took 44 us chained, 24.6
+// to start by itself: FP64 steps of 32^3 (1024 warps) took 41 us chained, 18.5
 // not.  The two-node kernels chain from 32^3 on (fewer nodes made no
 // difference), the FP64 ones, a third as many warps resident, from 64^3.
 constexpr int kChainPairs = 1 << 15, kChainFP64 = 1 << 18;  // nodes
@@ -192,7 +192,7 @@ enum Coeff {
   // shear rate: a/12, a/4, s/8, c/4, a/36 (D3Q15: s/16, c/8 and a/8 for the last three)
   kN5 = 0, kN7, kNb1, kNb2, kON,
   // odd moments
-  kQs,        // s_q                    (non-orthogonal and D3Q15)
+  kQ2,        // a_q                    (non-orthogonal and D3Q15)
   kQa,        // a_q / 2; orthogonal: a_q / 40
   kQb1, kQb2, // s_q / 12, c_q / 12; orthogonal over 60, D3Q15 over 24
   // energy; non-orthogonal: moment 4 over 6; orthogonal: e over 2394
@@ -224,7 +224,7 @@ inline Coeffs64 coeffs64(const KParams &P, int op) {
   k[kNb1] = sn / 8;
   k[kNb2] = cn / 4;
   k[kON] = (1 - sn) / 36;
-  k[kQs] = sq;
+  k[kQ2] = 1 - sq;
   if (op == kOrth) {
     k[kQa] = (1 - sq) / 40;
     k[kQb1] = sq / 60;

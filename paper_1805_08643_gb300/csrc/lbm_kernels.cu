@@ -143,14 +143,9 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
   T Sx, Sy, Sz;
   auto out = [&](int a, T v) { Lat<Q>::store(g_out + (size_t)a * P.np + nb.self, a, v); };
   if constexpr (PREC == kF64) {
-    psi_sums64<Q>(p, Sx, Sy, Sz);
+    psi_sums64(p, Sx, Sy, Sz);
     const double k = C.k[kForce] * p[0], S2 = SIGMA ? Sx * Sx + Sy * Sy + Sz * Sz : 0.0;
-    if constexpr (Q == 15)
-      collide_q15_64(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
-    else if constexpr (OP == kNonOrth)
-      collide_nonorth64(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
-    else
-      collide_orth64(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
+    collide64<OP>(f, P.rho_ref, k * Sx, k * Sy, k * Sz, S2, P, C, out);
     return;
   }
   Lat<Q>::gradient(p, Sx, Sy, Sz);
@@ -530,8 +525,8 @@ cudaError_t fused_dispatch(const KParams &P, bool sigma, const void *g_in, void 
   using S = typename Types<PREC>::S;
   using Psi = typename Types<PREC>::Psi;
   // FP64: blocks of one warp.  Every warp holds the SM's FP64 unit for the same time, so the last round is
-  // shortest when warps are dealt out singly: 32^3 steps 28.7 -> 26.7 us (orthogonal; blocks of four warps
-  // leave 8 on some SMs, single ones 7), no difference from 64^3 on.
+  // shortest when warps are dealt out singly: 32^3 steps 20.5 -> 18.5 us (blocks of four warps leave 8 on some
+  // SMs, single ones 7), no difference from 64^3 on.
   constexpr int threads = PREC == kF64 ? 32 : kThreads;
   const dim3 grid = node_grid(P, threads), block(threads);
   const Coeffs64 C = coeffs64(P, Q == 15 ? kNonOrthQ15 : OP);

@@ -56,13 +56,10 @@ __global__ void static_fused_kernel(const double *__restrict__ f_in, double *__r
   for (int a = 1; a < 19; ++a) p[a] = psi[nb.dst(a)];
   p[0] = psi[nb.self];
   double Sx, Sy, Sz;
-  lbm::psi_sums64<19>(p, Sx, Sy, Sz);
+  lbm::psi_sums64(p, Sx, Sy, Sz);
   const double k = C.k[lbm::kForce] * p[0], S2 = SIGMA ? Sx * Sx + Sy * Sy + Sz * Sz : 0.0;
   auto out = [&](int a, double v) { f_out[(size_t)a * P.n + nb.dst(a)] = v; };
-  if (OP == lbm::kNonOrth)
-    lbm::collide_nonorth64(f, 0.0, k * Sx, k * Sy, k * Sz, S2, P, C, out);
-  else
-    lbm::collide_orth64(f, 0.0, k * Sx, k * Sy, k * Sz, S2, P, C, out);
+  lbm::collide64<OP>(f, 0.0, k * Sx, k * Sy, k * Sz, S2, P, C, out);
 }
 
 // Device address of lbm_static_psi, looked up on the first call on each device
