@@ -149,8 +149,9 @@ __device__ __forceinline__ PsiT eos_psi(double rho, float rho_f, const KParams &
   if (!(rho_f < P.f_rho_max)) { err |= kErrEosDomain; return nan; }
   const double X = rho * fma(fma(fma(fma(P.q4, rho, P.q3), rho, P.q2), rho, P.q1), rho, P.q0);
   if (sizeof(PsiT) == sizeof(double)) {
-    if (!(X >= 0.0)) { err |= kErrEosDomain; return nan; }
-    if (X == 0.0) return PsiT(0);
+    const long long b = __double_as_longlong(X);  // comparisons on the bits, off the FP64 unit
+    if (b > 0x7ff0000000000000LL || (b < 0 && (b << 1) != 0)) { err |= kErrEosDomain; return nan; }  // NaN, X < 0
+    if ((b << 1) == 0) return PsiT(0);
     const double one_m = fma(-P.b4, rho, 1.0);
     return (PsiT)(X * rsqrt(X * (one_m * one_m * one_m)));
   }

@@ -99,7 +99,9 @@ __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S 
   T f[Q];
   pull_q<Q, S, T>(g, P.np, nb, f);
   T drho;
-  if constexpr (Q == 15) {
+  if constexpr (PREC == kF64) {
+    drho = sum64(f);
+  } else if constexpr (Q == 15) {
     drho = q15::drho(f);
   } else {
     // sum in the order of the forward chain: rest + axis pairs + diagonal pairs
@@ -115,7 +117,7 @@ __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S 
     psi[nb.self] = (typename Types<PREC>::Psi)eos_psi_d<EOS>((float)drho, P, e);
   } else {
     const double rho = P.rho_ref + (double)drho;
-    const float rho_f = sizeof(T) == sizeof(double) ? (float)rho : Phys<T>::rho_ref(P) + (float)drho;
+    const float rho_f = sizeof(T) == sizeof(double) ? narrow_f64(rho) : Phys<T>::rho_ref(P) + (float)drho;
     psi[nb.self] = eos_psi<EOS, typename Types<PREC>::Psi>(rho, rho_f, P, e);
   }
   if (e) atomicOr(err, e);
