@@ -48,7 +48,16 @@ __device__ __forceinline__ void gather_psi_pair(const float *__restrict__ psi, c
   p[18] = row1(nb.rmp);
 }
 
+// R4: a block's 128 pairs as 32 of each of four rows (every block full: rows4).
+template <bool R4 = false>
 __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int &y, int &z) {
+  if (R4) {
+    const unsigned q = blockIdx.x * 32, w = (unsigned)P.px / 2, by = P.pair_m ? __umulhi(q, P.pair_m) : q / w;
+    y = (int)(4 * by + threadIdx.x / 32);
+    z = blockIdx.z;
+    px = pair_x(P, 2 * (int)(q - by * w + threadIdx.x % 32));
+    return true;
+  }
   const unsigned p = blockIdx.x * blockDim.x + threadIdx.x, W = (unsigned)P.px / 2;
   y = (int)(P.pair_m ? __umulhi(p, P.pair_m) : p / W);
   z = blockIdx.z;
@@ -93,8 +102,10 @@ __device__ __forceinline__ void force_collide_lanes(V2 f[Q], V2 p[Q], const KPar
   }
 }
 
+// Twelve blocks an SM (40 registers): 256^3 FP32 217 -> 201 us against 48 registers
+// (the loads in flight need the warps), FP16 183 -> 180.
 template <typename S, int EOS, bool DF>
-__global__ void __launch_bounds__(128) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
+__global__ void __launch_bounds__(128, 12) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                        const KParams P, unsigned *__restrict__ err) {
   chain_wait();
   PairX px;
@@ -108,13 +119,16 @@ __global__ void __launch_bounds__(128) psi_pair_kernel(const S *__restrict__ g, 
   if (e) atomicOr(err, e);
 }
 
-template <typename S, int OP, bool SIGMA, bool ODD>
-__global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
+// Six blocks of 128 an SM (80 registers) for even boxes: FP16 256^3 fused 263 -> 258
+// us, FP32 192^3 orthogonal 164 -> 161; odd FP32 boxes
+// would spill, five there.
+template <typename S, int OP, bool SIGMA, bool ODD, bool R4 = false>
+__global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
                                                          const float *__restrict__ psi, const KParams P) {
   chain_wait();
   PairX px;
   int y, z;
-  if (!pair_of_thread(P, px, y, z)) return;
+  if (!pair_of_thread<R4>(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[19];
   pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
@@ -131,7 +145,7 @@ __global__ void __launch_bounds__(128) fused_pair_kernel(const S *__restrict__ g
 // The same two-node scheme for the D3Q15 variant (lbm_pair15.cuh).
 
 template <typename S, int EOS, bool DF>
-__global__ void __launch_bounds__(128) psi_pair15_kernel(const S *__restrict__ g, float *__restrict__ psi,
+__global__ void __launch_bounds__(128, 12) psi_pair15_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                          const KParams P, unsigned *__restrict__ err) {
   chain_wait();
   PairX px;
@@ -185,6 +199,12 @@ cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsign
   }
 }
 
+// Rows that fill blocks of 32 pairs x 4 rows.  The orthogonal FP16 fused pass, bound
+// by its issue slots, runs better on those (the rows of a block share psi in L1):
+// 256^3 286 -> 272 us.  The non-orthogonal one does not (263 -> 264), FP32 loses
+// (375 -> 401), and the psi pass too (201 -> 208).
+bool rows4(const KParams &P) { return P.px % 64 == 0 && P.ny % 4 == 0; }
+
 template <typename S, bool ODD>
 cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void *g_in, void *g_out,
                                 const void *psi, const Launch &L) {
@@ -196,6 +216,9 @@ cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void
   if (P.q == 15) return sigma ? run(fused_pair15_kernel<S, true, ODD>) : run(fused_pair15_kernel<S, false, ODD>);
   if (op == kNonOrth)
     return sigma ? run(fused_pair_kernel<S, kNonOrth, true, ODD>) : run(fused_pair_kernel<S, kNonOrth, false, ODD>);
+  if constexpr (!ODD && std::is_same<S, __half>::value)
+    if (rows4(P))
+      return sigma ? run(fused_pair_kernel<S, kOrth, true, ODD, true>) : run(fused_pair_kernel<S, kOrth, false, ODD, true>);
   return sigma ? run(fused_pair_kernel<S, kOrth, true, ODD>) : run(fused_pair_kernel<S, kOrth, false, ODD>);
 }
 
