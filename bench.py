@@ -72,13 +72,13 @@ STEP_MIN_BYTES_Q15 = {"f64": 15 * 8 * 2 + 16, "f32": 15 * 4 * 2 + 8, "f16": 15 *
 HEADLINE = ("nonorth", "f32")
 # DRAM bytes per node of the fused pass, from one ncu capture of the current kernel at 256^3 (dram__bytes_read
 # + dram__bytes_write over the nodes); null for forms without such a capture.
-FUSED_DRAM_BYTES = {("nonorth", "f32"): 152.6, ("nonorth", "f16"): 77.4}
+FUSED_DRAM_BYTES = {("nonorth", "f32"): 152.6, ("nonorth", "f16"): 77.3}
 # DRAM bytes per node of one launch of the work-list single pass at 256^3 (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch over the nodes), from a capture of the current kernel only
-QUEUE_DRAM_BYTES = {("nonorth", "f32"): 170.1}
-# FP64 instructions per node of the fused pass (ncu instruction counts at 128^3 over the nodes) and the FP64
+QUEUE_DRAM_BYTES = {("nonorth", "f32"): 175.4}
+# FP64 instructions per node of the fused pass (ncu instruction counts at 64^3 over the nodes) and the FP64
 # issue peak of one GB300: 2 per SM per clock x 152 SMs x 2070 MHz.
-FUSED_FP64_INSTR = {"nonorth": 255.0, "orth": 309.0, "nonorth_d3q15": 207.0}
+FUSED_FP64_INSTR = {"nonorth": 102.0, "orth": 92.0, "nonorth_d3q15": 85.0}
 FP64_PEAK_GINSTR = 2 * 152 * 2070e6 / 1e9
 PREC_TEXT = {"f64": "FP64 compute and storage", "f32": "FP32 compute and storage",
              "f16": "FP32 compute, FP16 storage"}

@@ -29,7 +29,7 @@ bool fill_params(const int grid[3], const lbm_eos *eos, double G, const lbm_rate
 
 namespace {
 
-// lbm_batch_set_tuning's tile value for the work-list single pass (64x4 tile jobs)
+// lbm_batch_set_tuning's tile value for the work-list single pass (tile jobs of 128 pairs)
 constexpr int kTileWorkList = 3;
 
 struct HostBox {

@@ -7,7 +7,7 @@ run on the live state: every candidate step is a real step of the simulation.
 
 from __future__ import annotations
 
-TILES = {0: "32x4", 1: "32x8", 2: "64x4", 3: "work list (64x4 tile jobs)"}
+TILES = {0: "32x4", 1: "32x8", 2: "64x4", 3: "work list (128-pair tile jobs)"}
 WORK_LIST = 3
 
 
