@@ -140,6 +140,8 @@ lbm_status rebuild(lbm_batch *b) {
   // the two-pass pair kernels); the others on the one-node single pass; one step graph runs both groups
   std::vector<std::pair<long long, int>> even, odd;
   for (auto &o : order) (b->boxes[o.second].d.P.px % 2 == 0 ? even : odd).push_back(o);
+  bool padded = false;
+  for (auto &o : even) padded = padded || b->boxes[o.second].d.P.px != b->boxes[o.second].d.P.nx;
   const bool wl = !even.empty() && b->tile == kTileWorkList;
   const int tile = b->tile == kTileWorkList ? lbm::kTile32x8 : b->tile;  // of the tile-shaped kernels
   std::vector<int4> items;
@@ -158,7 +160,7 @@ lbm_status rebuild(lbm_batch *b) {
   };
   if (wl) {
     // the work list over the even group in this order; each box's counters start at its qbase
-    BCK(lbm::batch_queue_grid(b->precision, b->eos, &b->wl_grid), "work list occupancy");
+    BCK(lbm::batch_queue_grid(b->precision, b->eos, padded, &b->wl_grid), "work list occupancy");
     std::vector<const KParams *> ps;
     for (auto &o : even) ps.push_back(&b->boxes[o.second].d.P);
     std::vector<int> base;
@@ -249,8 +251,6 @@ lbm_status rebuild(lbm_batch *b) {
     if (b->pair) BCK(lbm::batch_pair_occupancy(b->precision, b->eos, tile, pair_per_sm), "pair kernel occupancy");
     const int per_sm = tile == lbm::kTile32x4 ? 4 : 2;
     const int n_odd = b->nitems - n_even;
-    bool padded = false;
-    for (auto &o : even) padded = padded || b->boxes[o.second].d.P.px != b->boxes[o.second].d.P.nx;
     const int grid_odd = std::min(b->grid_blocks * per_sm, std::max(n_odd, 1));
     auto step = [&](int parity) {
       cudaError_t e = cudaSuccess;

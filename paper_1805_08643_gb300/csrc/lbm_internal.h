@@ -399,8 +399,8 @@ cudaError_t launch_steps(const KParams &P, int op, bool df, void *g_in, void *g_
 // launch starts (the step graph clears them).
 bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std::vector<int4> &out,
                        std::vector<int> &base, long long *ncounters);
-cudaError_t batch_queue_grid(int precision, int eos, int *grid);
 // odd: some box has rows padded for an odd Nx.
+cudaError_t batch_queue_grid(int precision, int eos, bool odd, int *grid);
 cudaError_t launch_batch_queue(int precision, int eos, bool odd, const BatchBox *boxes, const int4 *items, int nitems,
                                int parity, int grid, int *done, int ndone, unsigned *err, cudaStream_t s);
 

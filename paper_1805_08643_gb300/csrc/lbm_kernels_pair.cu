@@ -14,7 +14,6 @@
 
 #include <algorithm>
 #include <type_traits>
-#include <type_traits>
 
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
@@ -24,29 +23,6 @@
 
 namespace lbm {
 namespace {
-
-// psi(x + e_a) of both nodes, p[a] (Eq. 15 stencil).
-__device__ __forceinline__ void gather_psi_pair(const float *__restrict__ psi, const Nbhd &nb, const PairX &px,
-                                                V2 p[19]) {
-  // a row with x-moving directions: centre pair, x - 1 and x + 2
-  auto row3 = [&](int row, V2 &c, V2 &plus, V2 &minus) {
-    const float2 m = __ldg((const float2 *)(psi + row + px.x));
-    const float l = __ldg(psi + row + px.xm1), r = __ldg(psi + row + px.xp2);
-    c = V2(m);
-    plus = V2(m.y, r);   // psi(x + 1), psi(x + 2)
-    minus = V2(l, m.x);  // psi(x - 1), psi(x)
-  };
-  auto row1 = [&](int row) { return V2(__ldg((const float2 *)(psi + row + px.x))); };
-  row3(nb.r00, p[0], p[1], p[2]);
-  row3(nb.rp0, p[3], p[7], p[10]);
-  row3(nb.rm0, p[4], p[9], p[8]);
-  row3(nb.r0p, p[5], p[11], p[14]);
-  row3(nb.r0m, p[6], p[13], p[12]);
-  p[15] = row1(nb.rpp);
-  p[16] = row1(nb.rmm);
-  p[17] = row1(nb.rpm);
-  p[18] = row1(nb.rmp);
-}
 
 // R4: a block's 128 pairs as 32 of each of four rows (every block full: rows4).
 template <bool R4 = false>
@@ -65,57 +41,20 @@ __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int 
   return y < P.ny;
 }
 
-// Force and collision of the two nodes of a pair one after the other in scalar
-// FP32: a loop, since the compiler packs the two copies of an unrolled one and
-// contracts their products otherwise than the one-node kernels' code.  A box with an
-// odd Nx and FP32 storage keeps the rounding it always had (that of the one-node
-// kernels) on the loads and stores of the pair kernels.
-template <int OP, bool SIGMA, int Q>
-__device__ __forceinline__ void force_collide_lanes(V2 f[Q], V2 p[Q], const KParams &P) {
-  const Rates<float> r(P);
-#pragma unroll 1
-  for (int k = 0; k < 2; ++k) {
-    float fl[Q], pl[Q], Sx, Sy, Sz;
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      fl[a] = f[a].v.x;
-      pl[a] = p[a].v.x;
-    }
-    if constexpr (Q == 15)
-      q15::psi_gradient<float>(pl, Sx, Sy, Sz);
-    else
-      psi_gradient<float>(pl, Sx, Sy, Sz);
-    const float kk = -P.fG * pl[0];
-    const float Fx = kk * Sx, Fy = kk * Sy, Fz = kk * Sz;
-    const float dS4 = SIGMA ? P.fsigma_coef * (Sx * Sx + Sy * Sy + Sz * Sz) : 0.f;
-    if constexpr (Q == 15)
-      q15::collide<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
-    else if (OP == kNonOrth)
-      collide_nonorth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
-    else
-      collide_orth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {  // the other node comes first, then the order is back
-      f[a].v = make_float2(f[a].v.y, fl[a]);
-      p[a].v.x = p[a].v.y;
-    }
-  }
-}
-
 // Twelve blocks an SM (40 registers): 256^3 FP32 217 -> 201 us against 48 registers
 // (the loads in flight need the warps), FP16 183 -> 180.
-template <typename S, int EOS, bool DF>
-__global__ void __launch_bounds__(128, 12) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
+// ODD: rows padded for an odd Nx, set for FP16 storage only (FP32 sums round alike either way).
+template <typename S, int EOS, bool DF, bool ODD>
+__global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                        const KParams P, unsigned *__restrict__ err) {
   chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
-  V2 f[19];
-  pull_pair<S>(g, (unsigned)P.np, nb, px, f);
+  const V2 drho = pull_drho<S, PairIO<S>, ODD>(g, P, nb, px);
   unsigned e = 0;
-  store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(drho_pair(f), P, px.x), P, e));
+  store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(drho, P, px.x), P, e));
   if (e) atomicOr(err, e);
 }
 
@@ -131,11 +70,11 @@ __global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *_
   if (!pair_of_thread<R4>(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[19];
-  pull_pair<S>(g_in, (unsigned)P.np, nb, px, f);
+  pull_pair<S, PairIO<S>, ODD>(g_in, (unsigned)P.np, nb, px, f);
   V2 p[19];
-  gather_psi_pair(psi, nb, px, p);
-  if constexpr (ODD && std::is_same<S, float>::value)
-    force_collide_lanes<OP, SIGMA, 19>(f, p, P);
+  gather_psi_pair<PairIO<float>>(psi, nb, px, p);
+  if constexpr (ODD)
+    force_collide_lanes<S, OP, SIGMA, 19>(f, p, P);
   else
     force_collide_pair<OP, SIGMA>(f, p, P, Rates<V2>(P), OP);
   store_pair_f<S, ODD>(g_out, P, px.x, (unsigned)nb.self, f);
@@ -144,8 +83,8 @@ __global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *_
 // ------------------------------------------------------------------ D3Q15
 // The same two-node scheme for the D3Q15 variant (lbm_pair15.cuh).
 
-template <typename S, int EOS, bool DF>
-__global__ void __launch_bounds__(128, 12) psi_pair15_kernel(const S *__restrict__ g, float *__restrict__ psi,
+template <typename S, int EOS, bool DF, bool ODD>
+__global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair15_kernel(const S *__restrict__ g, float *__restrict__ psi,
                                                          const KParams P, unsigned *__restrict__ err) {
   chain_wait();
   PairX px;
@@ -153,9 +92,14 @@ __global__ void __launch_bounds__(128, 12) psi_pair15_kernel(const S *__restrict
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[q15::kQ];
-  pull_pair15<S>(g, (unsigned)P.np, nb, px, f);
+  pull_pair15<S, PairIO<S>, ODD>(g, (unsigned)P.np, nb, px, f);
+  V2 drho;
+  if constexpr (ODD)
+    drho = drho_lanes<S, q15::kQ>(f);
+  else
+    drho = q15::drho(f);
   unsigned e = 0;
-  store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(q15::drho(f), P, px.x), P, e));
+  store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(drho, P, px.x), P, e));
   if (e) atomicOr(err, e);
 }
 
@@ -166,12 +110,12 @@ __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
-  if constexpr (ODD && std::is_same<S, float>::value) {
+  if constexpr (ODD) {
     const Nbhd nb(px.x, y, z, P);
     V2 f[q15::kQ], p[q15::kQ];
-    pull_pair15<S>(g_in, (unsigned)P.np, nb, px, f);
+    pull_pair15<S, PairIO<S>, true>(g_in, (unsigned)P.np, nb, px, f);
     gather_psi_pair15(psi, nb, px, p);
-    force_collide_lanes<kNonOrth, SIGMA, q15::kQ>(f, p, P);
+    force_collide_lanes<S, kNonOrth, SIGMA, q15::kQ>(f, p, P);
     store_pair15_f<S, ODD>(g_out, P, px.x, (unsigned)nb.self, f);
   } else {
     fused_pair15_at<S, SIGMA, false, ODD>(g_in, g_out, psi, P, px.x, y, z);
@@ -180,22 +124,23 @@ __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__
 
 dim3 pair_grid(const KParams &P) { return plane_grid(P.px / 2 * P.ny, P.nz); }
 
-template <typename S, bool DF>
+template <typename S, bool DF, bool ODD>
 cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsigned *err, const Launch &L) {
   const dim3 grid = pair_grid(P), block(kThreads);
-  const S *gg = (const S *)g;
-  float *pp = (float *)psi;
+  auto run = [&](auto kernel) {
+    return launch_chained(P.n >= kChainPairs, kernel, grid, block, L.stream, (const S *)g, (float *)psi, P, err);
+  };
   if (P.q == 15) {
     switch (P.eos) {
-      case kEosCS: return launch_chained(P.n >= kChainPairs, psi_pair15_kernel<S, kEosCS, DF>, grid, block, L.stream, gg, pp, P, err);
-      case kEosExp: return launch_chained(P.n >= kChainPairs, psi_pair15_kernel<S, kEosExp, DF>, grid, block, L.stream, gg, pp, P, err);
-      default: return launch_chained(P.n >= kChainPairs, psi_pair15_kernel<S, kEosNone, false>, grid, block, L.stream, gg, pp, P, err);
+      case kEosCS: return run(psi_pair15_kernel<S, kEosCS, DF, ODD>);
+      case kEosExp: return run(psi_pair15_kernel<S, kEosExp, DF, ODD>);
+      default: return run(psi_pair15_kernel<S, kEosNone, false, false>);
     }
   }
   switch (P.eos) {
-    case kEosCS: return launch_chained(P.n >= kChainPairs, psi_pair_kernel<S, kEosCS, DF>, grid, block, L.stream, gg, pp, P, err);
-    case kEosExp: return launch_chained(P.n >= kChainPairs, psi_pair_kernel<S, kEosExp, DF>, grid, block, L.stream, gg, pp, P, err);
-    default: return launch_chained(P.n >= kChainPairs, psi_pair_kernel<S, kEosNone, false>, grid, block, L.stream, gg, pp, P, err);
+    case kEosCS: return run(psi_pair_kernel<S, kEosCS, DF, ODD>);
+    case kEosExp: return run(psi_pair_kernel<S, kEosExp, DF, ODD>);
+    default: return run(psi_pair_kernel<S, kEosNone, false, false>);
   }
 }
 
@@ -254,9 +199,8 @@ __global__ void __launch_bounds__(TXP *TY) batch_psi_kernel(const BatchBox *__re
     float *psi = bb.psi[in ^ 1];
     for (int z = w.z; z < w.w; ++z) {
       const Nbhd nb(x, y, z, P);
-      V2 f[19];
-      pull_pair<S>(g, (unsigned)P.np, nb, px, f);
-      store_pair_psi<true>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, false>(pad_lane<true>(drho_pair(f), P, x), P, e));
+      const V2 drho = pull_drho<S, PairIO<S>, true>(g, P, nb, px);
+      store_pair_psi<true>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, false>(pad_lane<true>(drho, P, x), P, e));
     }
   }
   if (e) atomicOr(err, e);
@@ -367,9 +311,11 @@ cudaError_t launch_batch_pair(int precision, int eos, int tile, const BatchBox *
 
 cudaError_t launch_psi_pair(const KParams &P, int precision, const void *g, void *psi, unsigned *err,
                             const Launch &L, bool df) {
-  if (precision == kF32)
-    return df ? psi_pair_dispatch<float, true>(P, g, psi, err, L) : psi_pair_dispatch<float, false>(P, g, psi, err, L);
-  return df ? psi_pair_dispatch<__half, true>(P, g, psi, err, L) : psi_pair_dispatch<__half, false>(P, g, psi, err, L);
+  auto launch = df ? psi_pair_dispatch<float, true, false> : psi_pair_dispatch<float, false, false>;
+  if (precision == kF16)
+    launch = P.px != P.nx ? (df ? psi_pair_dispatch<__half, true, true> : psi_pair_dispatch<__half, false, true>)
+                          : (df ? psi_pair_dispatch<__half, true, false> : psi_pair_dispatch<__half, false, false>);
+  return launch(P, g, psi, err, L);
 }
 
 cudaError_t launch_fused_pair(const KParams &P, int precision, int op, bool sigma, const void *g_in, void *g_out,

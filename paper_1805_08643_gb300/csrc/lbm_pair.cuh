@@ -6,7 +6,10 @@
 
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "lbm_device.cuh"
+#include "lbm_q15.cuh"
 
 namespace lbm {
 
@@ -69,7 +72,8 @@ struct PairX {
 // Pull the 19 deviations of nodes x and x + 1 (Eq. 5).  Populations with
 // e_x = 0 come from an aligned pair of the source row, those with e_x = +1
 // from (x-1, x) and those with e_x = -1 from (x+1, x+2), read as two scalars.
-template <typename S, typename Ld = PairIO<S>>
+// RAW: stored values as they are (FP16: still divided by w_a).
+template <typename S, typename Ld = PairIO<S>, bool RAW = false>
 __device__ __forceinline__ void pull_pair(const S *g, unsigned n, const Nbhd &nb, const PairX &px,
                                           V2 f[19]) {
 #pragma unroll
@@ -82,8 +86,31 @@ __device__ __forceinline__ void pull_pair(const S *g, unsigned n, const Nbhd &nb
       v = make_float2(Ld::ld1(rowp + px.xm1), Ld::ld1(rowp + px.x));
     else
       v = make_float2(Ld::ld1(rowp + px.x + 1), Ld::ld1(rowp + px.xp2));
-    f[a] = PairIO<S>::decode(v, a);
+    f[a] = RAW ? V2(v) : PairIO<S>::decode(v, a);
   }
+}
+
+// psi(x + e_a) of both nodes, p[a] (Eq. 15 stencil).
+template <typename Ld>
+__device__ __forceinline__ void gather_psi_pair(const float *psi, const Nbhd &nb, const PairX &px, V2 p[19]) {
+  // a row with x-moving directions: centre pair, x - 1 and x + 2
+  auto row3 = [&](int row, V2 &c, V2 &plus, V2 &minus) {
+    const float2 m = Ld::ld2(psi + row + px.x);
+    const float l = Ld::ld1(psi + row + px.xm1), r = Ld::ld1(psi + row + px.xp2);
+    c = V2(m);
+    plus = V2(m.y, r);   // psi(x + 1), psi(x + 2)
+    minus = V2(l, m.x);  // psi(x - 1), psi(x)
+  };
+  auto row1 = [&](int row) { return V2(Ld::ld2(psi + row + px.x)); };
+  row3(nb.r00, p[0], p[1], p[2]);
+  row3(nb.rp0, p[3], p[7], p[10]);
+  row3(nb.rm0, p[4], p[9], p[8]);
+  row3(nb.r0p, p[5], p[11], p[14]);
+  row3(nb.r0m, p[6], p[13], p[12]);
+  p[15] = row1(nb.rpp);
+  p[16] = row1(nb.rmm);
+  p[17] = row1(nb.rpm);
+  p[18] = row1(nb.rmp);
 }
 
 // Stores a pair (two-lane values v of direction a, or psi) at p: both lanes, or
@@ -128,12 +155,14 @@ __device__ __forceinline__ V2 pad_lane(V2 drho, const KParams &P, int x) {
 }
 
 // rho - rho_ref of both nodes: the sum of the pulled deviations (Eq. 6).
-__device__ __forceinline__ V2 drho_pair(const V2 f[19]) {
-  const V2 sax = (f[1] + f[2]) + (f[3] + f[4]) + (f[5] + f[6]);
-  const V2 sdg = ((f[7] + f[8]) + (f[9] + f[10])) + ((f[11] + f[12]) + (f[13] + f[14])) +
+template <typename T>
+__device__ __forceinline__ T drho_sum(const T f[19]) {
+  const T sax = (f[1] + f[2]) + (f[3] + f[4]) + (f[5] + f[6]);
+  const T sdg = ((f[7] + f[8]) + (f[9] + f[10])) + ((f[11] + f[12]) + (f[13] + f[14])) +
                  ((f[15] + f[16]) + (f[17] + f[18]));
   return f[0] + sax + sdg;
 }
+__device__ __forceinline__ V2 drho_pair(const V2 f[19]) { return drho_sum(f); }
 
 // psi of both nodes from rho - rho_ref; DF selects the compensated-FP32 radicand.
 template <int EOS, bool DF, bool ICVT = true>
@@ -182,6 +211,73 @@ __device__ __forceinline__ void force_collide_pair(V2 f[19], const V2 p[19], con
   collide_pair<OP>(f, Fx, Fy, Fz, dS4, P, r, op_rt);
 }
 
+// One-node rounding on the loads and stores of the pair kernels: density, force and
+// collision of the two nodes one after the other in scalar FP32, as the one-node
+// kernels of lbm_kernels.cu compute them, from stored values as they are (RAW: the
+// compiler contracts the FP16 form's weights into the sums).  An odd box keeps with
+// these the rounding it always had: on its own with either storage, in a batch with
+// FP16 storage, where a last place of FP32 shows as one of FP16.  Loops, since the
+// compiler packs the two copies of an unrolled one and contracts their products
+// otherwise than the one-node kernels' code.
+template <typename S, int Q>
+__device__ __forceinline__ float one_node_value(float stored, int a) {
+  if (std::is_same<S, float>::value) return stored;
+  return stored * (float)(Q == 15 ? q15::w(a) : lattice_w(a));
+}
+
+template <typename S, int Q>
+__device__ __forceinline__ V2 drho_lanes(V2 f[Q]) {
+  V2 out;
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    float fl[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      fl[a] = one_node_value<S, Q>(f[a].v.x, a);
+      f[a].v.x = f[a].v.y;
+    }
+    float d;
+    if constexpr (Q == 15)
+      d = q15::drho(fl);
+    else
+      d = drho_sum(fl);
+    out.v = make_float2(out.v.y, d);
+  }
+  return out;
+}
+
+template <typename S, int OP, bool SIGMA, int Q>
+__device__ __forceinline__ void force_collide_lanes(V2 f[Q], V2 p[Q], const KParams &P) {
+  const Rates<float> r(P);
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    float fl[Q], pl[Q], Sx, Sy, Sz;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      fl[a] = one_node_value<S, Q>(f[a].v.x, a);
+      pl[a] = p[a].v.x;
+    }
+    if constexpr (Q == 15)
+      q15::psi_gradient<float>(pl, Sx, Sy, Sz);
+    else
+      psi_gradient<float>(pl, Sx, Sy, Sz);
+    const float kk = -P.fG * pl[0];
+    const float Fx = kk * Sx, Fy = kk * Sy, Fz = kk * Sz;
+    const float dS4 = SIGMA ? P.fsigma_coef * (Sx * Sx + Sy * Sy + Sz * Sz) : 0.f;
+    if constexpr (Q == 15)
+      q15::collide<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
+    else if (OP == kNonOrth)
+      collide_nonorth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
+    else
+      collide_orth<float>(fl, P.frho_ref, Fx, Fy, Fz, dS4, r);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {  // the other node comes first, then the order is back
+      f[a].v = make_float2(f[a].v.y, fl[a]);
+      p[a].v.x = p[a].v.y;
+    }
+  }
+}
+
 // Loads through L2 only, for populations written by other blocks earlier in
 // the same launch (the non-coherent read-only path could hold stale lines).
 template <typename S> struct L2Load;
@@ -193,6 +289,26 @@ template <> struct L2Load<__half> {
   static __device__ __forceinline__ float2 ld2(const __half *p) { return __half22float2(__ldcg((const __half2 *)p)); }
   static __device__ __forceinline__ float ld1(const __half *p) { return __half2float(__ldcg(p)); }
 };
+
+// Whether pairs of padded rows take one-node rounding where a kernel steps even and odd boxes together (batches).
+template <typename S, bool ODD> __device__ __forceinline__ constexpr bool one_node_rounding() {
+  return ODD && std::is_same<S, __half>::value;
+}
+
+// rho - rho_ref of both nodes of a pair from the populations pulled with Ld.
+template <typename S, typename Ld, bool ODD>
+__device__ __forceinline__ V2 pull_drho(const S *g, const KParams &P, const Nbhd &nb, const PairX &px) {
+  V2 f[19];
+  if constexpr (one_node_rounding<S, ODD>()) {
+    pull_pair<S, Ld, true>(g, (unsigned)P.np, nb, px, f);
+    if (P.px != P.nx) return drho_lanes<S, 19>(f);
+#pragma unroll
+    for (int a = 0; a < 19; ++a) f[a] = PairIO<S>::decode(f[a].v, a);
+  } else {
+    pull_pair<S, Ld>(g, (unsigned)P.np, nb, px, f);
+  }
+  return drho_pair(f);
+}
 
 // The pair (x, x+1), x even, of row y in plane z with its periodic x neighbours.
 __device__ __forceinline__ PairX pair_x(const KParams &P, int x) {
@@ -212,29 +328,23 @@ __device__ __forceinline__ void fused_pair_at(const S *g_in, S *__restrict__ g_o
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
   V2 f[19];
+  if constexpr (one_node_rounding<S, ODD>()) {
+    if (P.px != P.nx) {
+      V2 p[19];
+      pull_pair<S, Ld, true>(g_in, (unsigned)P.np, nb, px, f);
+      gather_psi_pair<PsiLd>(psi, nb, px, p);
+      force_collide_lanes<S, OP, SIGMA, 19>(f, p, P);
+      store_pair_f<S, ODD>(g_out, P, x, (unsigned)nb.self, f);
+      return;
+    }
+  }
   // without FORCE_FIRST both sets of loads are issued before either is used
   // (one memory round trip, more registers)
   if (!FORCE_FIRST) pull_pair<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
   V2 Fx, Fy, Fz, dS4;
   {
     V2 p[19];
-    auto row3 = [&](int row, V2 &c, V2 &plus, V2 &minus) {
-      const float2 m = PsiLd::ld2(psi + row + px.x);
-      const float l = PsiLd::ld1(psi + row + px.xm1), rr = PsiLd::ld1(psi + row + px.xp2);
-      c = V2(m);
-      plus = V2(m.y, rr);
-      minus = V2(l, m.x);
-    };
-    auto row1 = [&](int row) { return V2(PsiLd::ld2(psi + row + px.x)); };
-    row3(nb.r00, p[0], p[1], p[2]);
-    row3(nb.rp0, p[3], p[7], p[10]);
-    row3(nb.rm0, p[4], p[9], p[8]);
-    row3(nb.r0p, p[5], p[11], p[14]);
-    row3(nb.r0m, p[6], p[13], p[12]);
-    p[15] = row1(nb.rpp);
-    p[16] = row1(nb.rmm);
-    p[17] = row1(nb.rpm);
-    p[18] = row1(nb.rmp);
+    gather_psi_pair<PsiLd>(psi, nb, px, p);
     force_pair<SIGMA>(p, P, Fx, Fy, Fz, dS4);
   }
   if (FORCE_FIRST) pull_pair<S, Ld>(g_in, (unsigned)P.np, nb, px, f);
@@ -249,20 +359,8 @@ __device__ __forceinline__ void psi_pair_at_l2(const S *__restrict__ g, float *_
                                                int x, int y, int z, unsigned &e) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
-  V2 f[19];
-#pragma unroll
-  for (int a = 0; a < 19; ++a) {
-    const S *rowp = g + (size_t)a * P.np + src_row(nb, a);
-    float2 v;
-    if (ex_of(a) == 0)
-      v = L2Load<S>::ld2(rowp + px.x);
-    else if (ex_of(a) > 0)
-      v = make_float2(L2Load<S>::ld1(rowp + px.xm1), L2Load<S>::ld1(rowp + px.x));
-    else
-      v = make_float2(L2Load<S>::ld1(rowp + px.x + 1), L2Load<S>::ld1(rowp + px.xp2));
-    f[a] = PairIO<S>::decode(v, a);
-  }
-  store_pair_psi<ODD>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, DF, ICVT>(pad_lane<ODD>(drho_pair(f), P, x), P, e));
+  const V2 drho = pull_drho<S, L2Load<S>, ODD>(g, P, nb, px);
+  store_pair_psi<ODD>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, DF, ICVT>(pad_lane<ODD>(drho, P, x), P, e));
 }
 
 // Cross-block signalling inside one launch: a release increment of a

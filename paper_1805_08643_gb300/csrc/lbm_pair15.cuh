@@ -44,8 +44,8 @@ __device__ __forceinline__ int src_row15(const Nbhd &nb, int a) {
 }
 
 // Pull of both nodes' 15 populations; Ld: PairIO<S> (read-only path) or
-// L2Load<S> (populations written earlier in the same launch).
-template <typename S, typename Ld = PairIO<S>>
+// L2Load<S> (populations written earlier in the same launch); RAW as in pull_pair.
+template <typename S, typename Ld = PairIO<S>, bool RAW = false>
 __device__ __forceinline__ void pull_pair15(const S *g, unsigned n, const Nbhd &nb, const PairX &px,
                                             V2 f[q15::kQ]) {
 #pragma unroll
@@ -58,7 +58,7 @@ __device__ __forceinline__ void pull_pair15(const S *g, unsigned n, const Nbhd &
       v = make_float2(Ld::ld1(rowp + px.xm1), Ld::ld1(rowp + px.x));
     else
       v = make_float2(Ld::ld1(rowp + px.x + 1), Ld::ld1(rowp + px.xp2));
-    f[a] = PairIO15<S>::decode(v, a);
+    f[a] = RAW ? V2(v) : PairIO15<S>::decode(v, a);
   }
 }
 

@@ -69,6 +69,8 @@ namespace {
 // difference one instruction, see operator-; 526 / 431 us as it is).  Batches stay at 6
 // (848 against 842 us for 64 boxes at 7, with 180 bytes spilled).
 constexpr int kBatchBlocks = 6;
+// FP16 batches with odd boxes collide those node by node (force_collide_lanes): 372 bytes spilled at 6 blocks.
+constexpr int kOddHalfBatchBlocks = 5;
 __host__ __device__ constexpr int min_blocks(int q) { return q == 15 ? 8 : 7; }
 // The psi jobs convert to and from FP64 with the conversion instructions, not
 // the integer path of the psi pass kernel (the same results): this kernel is
@@ -245,7 +247,7 @@ __device__ __forceinline__ void prefetch_boxes(BatchBox *dst, const BatchBox *__
 
 // ODD: some box has an odd Nx (rows padded to an even length, KParams::px).
 template <typename S, int EOS, bool ODD>
-__global__ void __launch_bounds__(NTH, kBatchBlocks)
+__global__ void __launch_bounds__(NTH, one_node_rounding<S, ODD>() ? kOddHalfBatchBlocks : kBatchBlocks)
     batch_queue_kernel(const BatchBox *__restrict__ boxes, const int4 *__restrict__ items, int nitems, int parity,
                        int *__restrict__ done, int ndone, unsigned *__restrict__ err) {
   __shared__ BatchBox bb[2][2];  // [item parity][fused job's box, psi job's box]
@@ -542,11 +544,11 @@ bool batch_queue_items(const std::vector<const KParams *> &boxes, int grid, std:
   return true;
 }
 
-cudaError_t batch_queue_grid(int precision, int eos, int *grid) {
+cudaError_t batch_queue_grid(int precision, int eos, bool odd, int *grid) {
   int per_sm = 0, dev = 0, sms = 0;
-  cudaError_t e = precision == kF32
-                      ? batch_by_eos<float, true>(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm)
-                      : batch_by_eos<__half, true>(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm);
+  auto query = precision == kF32 ? (odd ? batch_by_eos<float, true> : batch_by_eos<float, false>)
+                                 : (odd ? batch_by_eos<__half, true> : batch_by_eos<__half, false>);
+  cudaError_t e = query(eos, nullptr, nullptr, 0, 0, 0, nullptr, 0, nullptr, 0, &per_sm);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;

@@ -1,0 +1,70 @@
+"""A periodic box filled with copies of a small one evolves as the small one does, whatever kernels the sizes choose.
+So small boxes are the reference for what only large ones reach: here odd-Nx boxes too large for padded rows, which
+the one-node kernels step, and whose rounding every odd box has."""
+
+import numpy as np
+import pytest
+
+from gpu_helpers import coexistence, lattice, physics
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1805_08643_gb300 import _build
+
+    _build.build()
+
+
+def _tile(grid, seed=7):
+    """A density field between the phases without symmetry."""
+    rl, rv = coexistence(0.8)
+    rng = np.random.default_rng(seed)
+    return rv + (rl - rv) * (0.3 + 0.02 * rng.random(grid[::-1])), rv
+
+
+def _fields(grid, op, prec, tile, copies, steps, mode=False):
+    """rho and u on the device after `steps` steps of copies (x, y, z) of the tile."""
+    import torch
+
+    rho0, rv = tile
+    big = tuple(g * c for g, c in zip(grid, copies))
+    lat = lattice(big, op, prec, physics(sigma=0.105))
+    lat.set_tuning(mode)
+    lat.init_field(torch.from_numpy(rho0).cuda().repeat(copies[::-1]).reshape(-1), rv)
+    lat.step(steps)
+    rho = torch.empty(lat.n, dtype=torch.float64, device="cuda")
+    u = torch.empty(3 * lat.n, dtype=torch.float64, device="cuda")
+    lat.moments_device(rho, u)
+    assert lat.check() == 0
+    lat.close()
+    return torch.cat([rho, u]).reshape(4, big[2], big[1], big[0])
+
+
+def _assert_tiled(big, small):
+    _, nz, ny, nx = small.shape
+    d, z, y, x = big.shape
+    for k in range(d):
+        parts = big[k].view(z // nz, nz, y // ny, ny, x // nx, nx)
+        assert bool((parts == small[k].view(1, nz, 1, ny, 1, nx)).all()), k
+
+
+# 6 x 6144 x 6300 padded nodes times 19 directions pass 2^32, 5 x 6144 x 6300 times 19 do not
+ODD, ODD_COPIES = (5, 6, 7), (1, 1024, 900)
+
+
+@pytest.mark.parametrize("prec", ["f32", "f16"])
+@pytest.mark.parametrize("op", ["nonorth", "orth", "nonorth_d3q15"])
+def test_odd_rows_round_as_the_one_node_kernels(op, prec):
+    import torch
+
+    tile = _tile(ODD)
+    small = _fields(ODD, op, prec, tile, (1, 1, 1), 12)
+    big = _fields(ODD, op, prec, tile, ODD_COPIES, 12)
+    _assert_tiled(big, small)
+    del big
+    torch.cuda.empty_cache()
