@@ -21,7 +21,10 @@ namespace lbm {
 // launch's blocks in (they come only once every block of this grid has started)
 // and waits until the grid before this one has completed and its writes are
 // visible.  Every such kernel waits, so a grid completes only after all before
-// it: what it overwrites has been read.
+// it: what it overwrites has been read.  A block may be on its SM while the grid
+// before still writes, so what that grid writes is not read-only for this kernel's
+// lifetime: such a kernel reads populations and psi with plain loads, never through
+// the read-only path (__ldg, const __restrict__ pointers).
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -38,6 +38,9 @@ template <> struct Lat<19> {
   static __device__ __forceinline__ int src(const Nbhd &nb, int a) { return nb.src(a); }
   static __device__ __forceinline__ int dst(const Nbhd &nb, int a) { return nb.dst(a); }
   static __device__ __forceinline__ double w(int a) { return lattice_w(a); }
+  template <typename S> static __device__ __forceinline__ typename Storage<S>::Compute decode(S v, int a) {
+    return Storage<S>::decode(v, a);
+  }
   template <typename S> static __device__ __forceinline__ typename Storage<S>::Compute load(const S *p, int a) {
     return Storage<S>::load(p, a);
   }
@@ -52,6 +55,9 @@ template <> struct Lat<15> {
   static __device__ __forceinline__ int src(const Nbhd &nb, int a) { return q15::src(nb, a); }
   static __device__ __forceinline__ int dst(const Nbhd &nb, int a) { return q15::dst(nb, a); }
   static __device__ __forceinline__ double w(int a) { return q15::w(a); }
+  template <typename S> static __device__ __forceinline__ typename Storage<S>::Compute decode(S v, int a) {
+    return q15::Storage<S>::decode(v, a);
+  }
   template <typename S> static __device__ __forceinline__ typename Storage<S>::Compute load(const S *p, int a) {
     return q15::Storage<S>::load(p, a);
   }
@@ -63,10 +69,14 @@ template <> struct Lat<15> {
   }
 };
 
-template <int Q, typename S, typename T>
-__device__ __forceinline__ void pull_q(const S *__restrict__ g, int n, const Nbhd &nb, T f[Q]) {
+// RO: through the read-only path (not in chained kernels: chain_wait).
+template <int Q, bool RO, typename S, typename T>
+__device__ __forceinline__ void pull_q(const S *g, int n, const Nbhd &nb, T f[Q]) {
 #pragma unroll
-  for (int a = 0; a < Q; ++a) f[a] = (T)Lat<Q>::load(g + (size_t)a * n + Lat<Q>::src(nb, a), a);
+  for (int a = 0; a < Q; ++a) {
+    const S *p = g + (size_t)a * n + Lat<Q>::src(nb, a);
+    f[a] = RO ? (T)Lat<Q>::load(p, a) : (T)Lat<Q>::template decode<S>(*p, a);
+  }
 }
 
 // Stores one node's population of direction a, and its copy at the end of a padded row.
@@ -87,7 +97,7 @@ __device__ __forceinline__ bool node_of_thread(const KParams &P, int &x, int &y,
 
 // ------------------------------------------------------------------ psi pass
 template <int PREC, int EOS, bool DF, int Q>
-__global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S *__restrict__ g,
+__global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S *g,
                                                   typename Types<PREC>::Psi *__restrict__ psi,
                                                   const KParams P, unsigned *__restrict__ err) {
   chain_wait();
@@ -97,7 +107,7 @@ __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S 
   if (!node_of_thread(P, x, y, z)) return;
   const Nbhd nb(x, y, z, P);
   T f[Q];
-  pull_q<Q, S, T>(g, P.np, nb, f);
+  pull_q<Q, false, S, T>(g, P.np, nb, f);
   T drho;
   if constexpr (PREC == kF64) {
     drho = sum64(f);
@@ -125,9 +135,9 @@ __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S 
 
 // ------------------------------------------------------------------ fused pass
 template <int PREC, int OP, bool SIGMA, int Q>
-__global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::S *__restrict__ g_in,
+__global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::S *g_in,
                                                     typename Types<PREC>::S *__restrict__ g_out,
-                                                    const typename Types<PREC>::Psi *__restrict__ psi,
+                                                    const typename Types<PREC>::Psi *psi,
                                                     const KParams P, const Coeffs64 C) {
   chain_wait();
   using S = typename Types<PREC>::S;
@@ -136,12 +146,12 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
   if (!node_of_thread(P, x, y, z)) return;
   const Nbhd nb(x, y, z, P);
   T f[Q];
-  pull_q<Q, S, T>(g_in, P.np, nb, f);
+  pull_q<Q, false, S, T>(g_in, P.np, nb, f);
   // interaction force, Eq. 15
   T p[Q];
 #pragma unroll
-  for (int a = 1; a < Q; ++a) p[a] = (T)__ldg(psi + Lat<Q>::dst(nb, a));
-  p[0] = (T)__ldg(psi + nb.self);
+  for (int a = 1; a < Q; ++a) p[a] = (T)psi[Lat<Q>::dst(nb, a)];
+  p[0] = (T)psi[nb.self];
   T Sx, Sy, Sz;
   auto out = [&](int a, T v) { Lat<Q>::store(g_out + (size_t)a * P.np + nb.self, a, v); };
   if constexpr (PREC == kF64) {
@@ -271,7 +281,7 @@ __device__ __forceinline__ void node_moments(const typename Types<PREC>::S *__re
   // the sums of Eq. 15 with the diagonal (corner) weight taken out: axis entries weigh 2 (8) times as much
   constexpr float axw = Q == 19 ? 2.0f : 8.0f;
   T f[Q], p[Q];
-  pull_q<Q, S, T>(g, P.np, nb, f);
+  pull_q<Q, true, S, T>(g, P.np, nb, f);
 #pragma unroll
   for (int a = 1; a < Q; ++a) p[a] = psi[Lat<Q>::dst(nb, a)];
   p[0] = psi[nb.self];

@@ -45,14 +45,14 @@ __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int 
 // (the loads in flight need the warps), FP16 183 -> 180.
 // ODD: rows padded for an odd Nx, set for FP16 storage only (FP32 sums round alike either way).
 template <typename S, int EOS, bool DF, bool ODD>
-__global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *__restrict__ g, float *__restrict__ psi,
+__global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *g, float *__restrict__ psi,
                                                        const KParams P, unsigned *__restrict__ err) {
   chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
-  const V2 drho = pull_drho<S, PairIO<S>, ODD>(g, P, nb, px);
+  const V2 drho = pull_drho<S, PlainLoad, ODD>(g, P, nb, px);
   unsigned e = 0;
   store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(drho, P, px.x), P, e));
   if (e) atomicOr(err, e);
@@ -62,17 +62,17 @@ __global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *__
 // us, FP32 192^3 orthogonal 164 -> 161; odd FP32 boxes
 // would spill, five there.
 template <typename S, int OP, bool SIGMA, bool ODD, bool R4 = false>
-__global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
-                                                         const float *__restrict__ psi, const KParams P) {
+__global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *g_in, S *__restrict__ g_out,
+                                                         const float *psi, const KParams P) {
   chain_wait();
   PairX px;
   int y, z;
   if (!pair_of_thread<R4>(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[19];
-  pull_pair<S, PairIO<S>, ODD>(g_in, (unsigned)P.np, nb, px, f);
+  pull_pair<S, PlainLoad, ODD>(g_in, (unsigned)P.np, nb, px, f);
   V2 p[19];
-  gather_psi_pair<PairIO<float>>(psi, nb, px, p);
+  gather_psi_pair<PlainLoad>(psi, nb, px, p);
   if constexpr (ODD)
     force_collide_lanes<S, OP, SIGMA, 19>(f, p, P);
   else
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *_
 // The same two-node scheme for the D3Q15 variant (lbm_pair15.cuh).
 
 template <typename S, int EOS, bool DF, bool ODD>
-__global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair15_kernel(const S *__restrict__ g, float *__restrict__ psi,
+__global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair15_kernel(const S *g, float *__restrict__ psi,
                                                          const KParams P, unsigned *__restrict__ err) {
   chain_wait();
   PairX px;
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair15_kernel(const S *
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
   V2 f[q15::kQ];
-  pull_pair15<S, PairIO<S>, ODD>(g, (unsigned)P.np, nb, px, f);
+  pull_pair15<S, PlainLoad, ODD>(g, (unsigned)P.np, nb, px, f);
   V2 drho;
   if constexpr (ODD)
     drho = drho_lanes<S, q15::kQ>(f);
@@ -104,8 +104,8 @@ __global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair15_kernel(const S *
 }
 
 template <typename S, bool SIGMA, bool ODD>
-__global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__ g_in, S *__restrict__ g_out,
-                                                           const float *__restrict__ psi, const KParams P) {
+__global__ void __launch_bounds__(128) fused_pair15_kernel(const S *g_in, S *__restrict__ g_out,
+                                                           const float *psi, const KParams P) {
   chain_wait();
   PairX px;
   int y, z;
@@ -113,12 +113,12 @@ __global__ void __launch_bounds__(128) fused_pair15_kernel(const S *__restrict__
   if constexpr (ODD) {
     const Nbhd nb(px.x, y, z, P);
     V2 f[q15::kQ], p[q15::kQ];
-    pull_pair15<S, PairIO<S>, true>(g_in, (unsigned)P.np, nb, px, f);
-    gather_psi_pair15(psi, nb, px, p);
+    pull_pair15<S, PlainLoad, true>(g_in, (unsigned)P.np, nb, px, f);
+    gather_psi_pair15<PlainLoad>(psi, nb, px, p);
     force_collide_lanes<S, kNonOrth, SIGMA, q15::kQ>(f, p, P);
     store_pair15_f<S, ODD>(g_out, P, px.x, (unsigned)nb.self, f);
   } else {
-    fused_pair15_at<S, SIGMA, false, ODD>(g_in, g_out, psi, P, px.x, y, z);
+    fused_pair15_at<S, SIGMA, false, ODD, PlainLoad, PlainLoad>(g_in, g_out, psi, P, px.x, y, z);
   }
 }
 

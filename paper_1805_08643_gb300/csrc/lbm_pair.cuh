@@ -34,10 +34,12 @@ template <> struct PairIO<__half> {
   }
 };
 
-// Plain loads, for arrays that other blocks write in the same launch: coherent
-// after an acquire, where the read-only path of PairIO could return what was
-// there before.
+// Plain loads, for arrays that other blocks write in the same launch or the grid
+// before a chained one writes (chain_wait): coherent after an acquire, where the
+// read-only path of PairIO could return what was there before.
 struct PlainLoad {
+  static __device__ __forceinline__ float2 ld2(const __half *p) { return __half22float2(*(const __half2 *)p); }
+  static __device__ __forceinline__ float ld1(const __half *p) { return __half2float(*p); }
   static __device__ __forceinline__ float2 ld2(const float *p) { return *(const float2 *)p; }
   static __device__ __forceinline__ float ld1(const float *p) { return *p; }
 };

@@ -76,12 +76,16 @@ __device__ __forceinline__ int dst(const Nbhd &nb, int a) {
 
 // Stored populations: the deviation f_a - w_a rho_ref (FP16: divided by w_a).
 template <typename S> struct Storage {
+  static __device__ __forceinline__ typename lbm::Storage<S>::Compute decode(S v, int a) {
+    return lbm::Storage<S>::decode(v, a);
+  }
   static __device__ __forceinline__ typename lbm::Storage<S>::Compute load(const S *p, int a) {
     return lbm::Storage<S>::load(p, a);
   }
   template <typename T> static __device__ __forceinline__ void store(S *p, int a, T v) { lbm::Storage<S>::store(p, a, v); }
 };
 template <> struct Storage<__half> {
+  static __device__ __forceinline__ float decode(__half v, int a) { return __half2float(v) * (float)w(a); }
   static __device__ __forceinline__ float load(const __half *p, int a) { return __half2float(__ldg(p)) * (float)w(a); }
   template <typename T> static __device__ __forceinline__ void store(__half *p, int a, T v) {
     *p = __float2half_rn((float)v * inv_w(a));

@@ -1,6 +1,6 @@
 """A periodic box filled with copies of a small one evolves as the small one does, whatever kernels the sizes choose.
-So small boxes are the reference for what only large ones reach: here odd-Nx boxes too large for padded rows, which
-the one-node kernels step, and whose rounding every odd box has."""
+So small boxes are the reference for what only large ones reach: odd-Nx boxes too large for padded rows, which the
+one-node kernels step, and whose rounding every odd box has; and two-pass steps whose launches overlap."""
 
 import numpy as np
 import pytest
@@ -68,3 +68,60 @@ def test_odd_rows_round_as_the_one_node_kernels(op, prec):
     _assert_tiled(big, small)
     del big
     torch.cuda.empty_cache()
+
+
+def _chained_pair(tile_grid, copies, op, prec):
+    """A box above the sizes from which launches overlap, and its tile below them, on the two-pass step."""
+    rho0, rv = _tile(tile_grid)
+    small = lattice(tile_grid, op, prec, physics(sigma=0.105))
+    big = lattice(tuple(g * c for g, c in zip(tile_grid, copies)), op, prec, physics(sigma=0.105))
+    assert small.n < 1 << 15 and big.n >= (1 << 18 if prec == "f64" else 1 << 15)
+    for lat, rho in ((small, rho0), (big, np.tile(rho0, copies[::-1]))):
+        lat.set_tuning(False)
+        lat.init_field(rho, rv)
+    return small, big
+
+
+def _assert_same_populations(small, big):
+    import torch
+
+    fs, fb = torch.from_numpy(small.populations()), torch.from_numpy(big.populations())
+    assert small.check() == 0 and big.check() == 0
+    _assert_tiled(fb, fs)
+
+
+CHAINED = [((12, 10, 9), (6, 6, 8)), ((13, 10, 9), (5, 6, 8)), ((32, 8, 5), (4, 10, 14))]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16"])
+@pytest.mark.parametrize("op", ["nonorth", "orth", "nonorth_d3q15"])
+@pytest.mark.parametrize("tile_grid, copies", CHAINED)
+def test_overlapping_launches_step_as_separate_ones(tile_grid, copies, op, prec):
+    small, big = _chained_pair(tile_grid, copies, op, prec)
+    small.step(40)
+    for n in (1, 1, 3, 35):
+        big.step(n)
+    _assert_same_populations(small, big)
+    small.close()
+    big.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16"])
+def test_overlapping_launches_replayed_from_a_graph(prec):
+    import torch
+
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        small, big = _chained_pair(*CHAINED[0], "nonorth", prec)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        g.capture_begin()
+        big.step(2)  # two steps: the state is back in the buffer the capture read
+        g.capture_end()
+        for _ in range(20):
+            g.replay()
+        small.step(40)
+        s.synchronize()
+        _assert_same_populations(small, big)
+        small.close()
+        big.close()
