@@ -47,7 +47,9 @@ constexpr int kOpRuntime = 2;
 
 // One x-y tile of one box marched through planes [z0, z1): the whole single
 // pass for those nodes.  OP is kOrth, kNonOrth or kOpRuntime (then op_rt picks).
-template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY>
+// PAD: rows padded for an odd Nx (KParams::px), an instantiation of its own: in code
+// that even boxes shared, the pad's stores took 256^3 FP16 steps from 754 to 1418 us.
+template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY, bool PAD>
 __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *__restrict__ g_in,
                                              typename OneTypes<PREC>::S *__restrict__ g_out,
                                              const float *__restrict__ psi_in, float *__restrict__ psi_out,
@@ -64,11 +66,13 @@ __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *_
   const bool active = tid < NE;
   const int lx = tid % EX, ly = tid / EX;
   const int nx = P.nx, ny = P.ny, nz = P.nz;
-  const int px = P.px;  // row length of the stored arrays
-  const unsigned n = (unsigned)P.np, nxy = (unsigned)(px * ny);
+  const int px = PAD ? P.px : nx;  // row length of the stored arrays
+  const unsigned n = (unsigned)(PAD ? P.np : P.n), nxy = (unsigned)(px * ny);
   const int gx = wrap(x0 + lx - 1, nx), gy = wrap(y0 + ly - 1, ny);
   const bool interior = active && lx >= 1 && lx <= BX && ly >= 1 && ly <= BY && x0 + lx - 1 < nx &&
                         y0 + ly - 1 < ny;
+  // PAD: the halo thread at x = nx has node 0's f* as well and stores it in the pad
+  const bool pad = PAD && active && x0 + lx - 1 == nx && ly >= 1 && ly <= BY && y0 + ly - 1 < ny;
   const Rates<float> r(P);
   const float rho_ref = P.frho_ref, mG = -P.fG;
 
@@ -166,14 +170,10 @@ __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *_
         collide_nonorth<float>(f, rho_ref, k * Sx, k * Sy, k * Sz, dS4, r);
       else
         collide_orth<float>(f, rho_ref, k * Sx, k * Sy, k * Sz, dS4, r);
-      if (interior && zz >= z0 && zz < z1) {
-        const unsigned self = (unsigned)zz * nxy + o_00;
+      if ((interior || pad) && zz >= z0 && zz < z1) {
+        const unsigned self = (unsigned)zz * nxy + o_00 + (pad ? nx : 0);
 #pragma unroll
         for (int a = 0; a < 19; ++a) Storage<S>::store(g_out + (unsigned)a * n + self, a, f[a]);
-        if (px != nx && gx == 0) {  // the copy of node 0 at the end of a padded row
-#pragma unroll
-          for (int a = 0; a < 19; ++a) Storage<S>::store(g_out + (unsigned)a * n + self + nx, a, f[a]);
-        }
       }
 #pragma unroll
       for (int a = 1; a < 19; ++a) buf[(a - 1) * NE + tid] = f[a];
@@ -207,7 +207,7 @@ __device__ __forceinline__ void onepass_tile(const typename OneTypes<PREC>::S *_
   }
 }
 
-template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY>
+template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY, bool PAD>
 __global__ void __launch_bounds__(((BX + 2) * (BY + 2) + 31) / 32 * 32, (one_min_blocks<BX, BY>()))
     onepass_kernel(const typename OneTypes<PREC>::S *__restrict__ g_in, typename OneTypes<PREC>::S *__restrict__ g_out,
                    const float *__restrict__ psi_in, float *__restrict__ psi_out, const KParams P, int zc,
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(((BX + 2) * (BY + 2) + 31) / 32 * 32, (one_min
   extern __shared__ float smem[];
   unsigned e = 0;
   const int z0 = blockIdx.z * zc;
-  onepass_tile<PREC, OP, SIGMA, EOS, BX, BY>(g_in, g_out, psi_in, psi_out, P, blockIdx.x * BX, blockIdx.y * BY, z0,
+  onepass_tile<PREC, OP, SIGMA, EOS, BX, BY, PAD>(g_in, g_out, psi_in, psi_out, P, blockIdx.x * BX, blockIdx.y * BY, z0,
                                              min(z0 + zc, P.nz), OP, e, smem);
   if (e) atomicOr(err, e);
 }
@@ -240,31 +240,38 @@ __global__ void __launch_bounds__(((BX + 2) * (BY + 2) + 31) / 32 * 32, (one_min
     }
     __syncthreads();
     const int in = bb.cur ^ parity;
-    onepass_tile<PREC, kOpRuntime, true, EOS, BX, BY>(
+    onepass_tile<PREC, kOpRuntime, true, EOS, BX, BY, false>(
         (const S *)bb.g[in], (S *)bb.g[in ^ 1], bb.psi[in], bb.psi[in ^ 1], bb.P, (w.y & 0xffff) * BX,
         (w.y >> 16) * BY, w.z, w.w, bb.op, e, smem);
   }
   if (e) atomicOr(err, e);
 }
 
-template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY>
-cudaError_t launch_tile(const KParams &P, const void *g_in, void *g_out, const void *psi_in, void *psi_out, int zc,
+template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY, bool PAD>
+cudaError_t launch_padded(const KParams &P, const void *g_in, void *g_out, const void *psi_in, void *psi_out, int zc,
                         unsigned *err, cudaStream_t s) {
   using S = typename OneTypes<PREC>::S;
   constexpr int NT = ((BX + 2) * (BY + 2) + 31) / 32 * 32;
   constexpr size_t smem = OneSmem<BX, BY>::bytes;
   static bool attr_set = false;  // per process; the attribute is per function, not per device
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(onepass_kernel<PREC, OP, SIGMA, EOS, BX, BY>,
+    cudaError_t e = cudaFuncSetAttribute(onepass_kernel<PREC, OP, SIGMA, EOS, BX, BY, PAD>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   const dim3 grid((P.nx + BX - 1) / BX, (P.ny + BY - 1) / BY, (P.nz + zc - 1) / zc);
-  onepass_kernel<PREC, OP, SIGMA, EOS, BX, BY><<<grid, NT, smem, s>>>((const S *)g_in, (S *)g_out,
-                                                                      (const float *)psi_in, (float *)psi_out, P, zc,
-                                                                      err);
+  onepass_kernel<PREC, OP, SIGMA, EOS, BX, BY, PAD><<<grid, NT, smem, s>>>(
+      (const S *)g_in, (S *)g_out, (const float *)psi_in, (float *)psi_out, P, zc, err);
   return cudaGetLastError();
+}
+
+template <int PREC, int OP, bool SIGMA, int EOS, int BX, int BY>
+cudaError_t launch_tile(const KParams &P, const void *g_in, void *g_out, const void *psi_in, void *psi_out, int zc,
+                        unsigned *err, cudaStream_t s) {
+  auto launch = P.px != P.nx ? launch_padded<PREC, OP, SIGMA, EOS, BX, BY, true>
+                             : launch_padded<PREC, OP, SIGMA, EOS, BX, BY, false>;
+  return launch(P, g_in, g_out, psi_in, psi_out, zc, err, s);
 }
 
 template <int PREC, int OP, bool SIGMA, int EOS>
