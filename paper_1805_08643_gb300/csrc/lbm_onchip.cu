@@ -132,13 +132,13 @@ __global__ void __launch_bounds__(NTH, 3)
       }
       float *ps = psi_slot(m);
       V2 f[19];
-      pull_pair<S>(g_in, (unsigned)P.n, Nbhd(gxp, gyp, zw, P), pxp, f);
+      pull_pair<S>(g_in, (unsigned)P.n, Nbhd(gxp, gyp, zw, P, P.nx), pxp, f);
       float2 *st = stage_buf(m) + p;
 #pragma unroll
       for (int a = 0; a < 19; ++a) st[a * NI] = f[a].v;
       *(float2 *)(ps + cs) = psi_pair<EOS, DF>(drho_pair(f), P, e);
       if (has_ring) {
-        pull_pair<S>(g_in, (unsigned)P.n, Nbhd(rgx, rgy, zw, P), pxr, f);
+        pull_pair<S>(g_in, (unsigned)P.n, Nbhd(rgx, rgy, zw, P, P.nx), pxr, f);
         *(float2 *)(ps + cr) = psi_pair<EOS, DF>(drho_pair(f), P, e);
       }
       mbar_arrive(&full[m & 3]);
