@@ -248,7 +248,7 @@ lbm_status rebuild(lbm_batch *b) {
     // resident blocks per SM: the pair kernels' own occupancy (the psi kernel needs half the fused kernel's
     // registers), the single-pass kernel's launch bounds
     int pair_per_sm[2] = {1, 1};
-    if (b->pair) BCK(lbm::batch_pair_occupancy(b->precision, b->eos, tile, pair_per_sm), "pair kernel occupancy");
+    if (b->pair) BCK(lbm::batch_pair_occupancy(b->precision, b->eos, tile, padded, pair_per_sm), "pair kernel occupancy");
     const int per_sm = tile == lbm::kTile32x4 ? 4 : 2;
     const int n_odd = b->nitems - n_even;
     const int grid_odd = std::min(b->grid_blocks * per_sm, std::max(n_odd, 1));
@@ -260,7 +260,7 @@ lbm_status rebuild(lbm_batch *b) {
           e = lbm::launch_batch_queue(b->precision, b->eos, padded, b->d_boxes, b->d_items, n_even, parity, b->wl_grid,
                                       b->d_done, (int)b->ndone, b->d_err, b->stream);
       } else if (n_even) {
-        e = lbm::launch_batch_pair(b->precision, b->eos, tile, b->d_boxes, b->d_items, n_even, b->d_fmap,
+        e = lbm::launch_batch_pair(b->precision, b->eos, tile, padded, b->d_boxes, b->d_items, n_even, b->d_fmap,
                                    b->fused_blocks, parity, b->grid_blocks, pair_per_sm, b->d_err, b->stream);
       }
       if (e == cudaSuccess && n_odd)

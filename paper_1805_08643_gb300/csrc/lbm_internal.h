@@ -321,9 +321,10 @@ struct alignas(16) BatchBox {  // 16-byte aligned: copied to shared memory in 16
 // plane by plane, tiles x-fastest.  The psi pass is a persistent grid of
 // sms x per_sm[1] blocks over the items (at most one per item), per_sm as
 // batch_pair_occupancy gives it (resident blocks per SM; [0] is unused).
-cudaError_t batch_pair_occupancy(int precision, int eos, int tile, int per_sm[2]);
-cudaError_t launch_batch_pair(int precision, int eos, int tile, const BatchBox *boxes, const int4 *items, int nitems,
-                              const int *block_box, const int fused_blocks[2], int parity, int sms,
+// odd: some box has rows padded for an odd Nx.
+cudaError_t batch_pair_occupancy(int precision, int eos, int tile, bool odd, int per_sm[2]);
+cudaError_t launch_batch_pair(int precision, int eos, int tile, bool odd, const BatchBox *boxes, const int4 *items,
+                              int nitems, const int *block_box, const int fused_blocks[2], int parity, int sms,
                               const int per_sm[2], unsigned *err, cudaStream_t s);
 cudaError_t launch_batch_onepass(int precision, int eos, int tile, const BatchBox *boxes, const int4 *items,
                                  int nitems, int parity, int grid, unsigned *err, cudaStream_t s);

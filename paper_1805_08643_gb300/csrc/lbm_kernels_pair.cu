@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *g,
   int y, z;
   if (!pair_of_thread(P, px, y, z)) return;
   const Nbhd nb(px.x, y, z, P);
-  const V2 drho = pull_drho<S, PlainLoad, ODD>(g, P, nb, px);
+  const V2 drho = pull_drho<S, PlainLoad, ODD>(g, (unsigned)P.np, P, nb, px);
   unsigned e = 0;
   store_pair_psi<true>(psi, P, px.x, (unsigned)nb.self, psi_pair<EOS, DF>(pad_lane<true>(drho, P, px.x), P, e));
   if (e) atomicOr(err, e);
@@ -174,7 +174,9 @@ cudaError_t fused_pair_dispatch(const KParams &P, int op, bool sigma, const void
 // level in ^ 1; this pass then evaluates psi of level in ^ 1, so after a step
 // psi of the current level is always valid.  (A flat grid of one plane per
 // block, as for the fused pass, measured 2 % slower here.)
-template <typename S, int EOS, int TXP, int TY>
+// ODD: some box has padded rows (in code of their own: 32 even boxes, FP32, stepped in
+// 482 us with the pads' stores compiled in, 400 without).
+template <typename S, int EOS, int TXP, int TY, bool ODD>
 __global__ void __launch_bounds__(TXP *TY) batch_psi_kernel(const BatchBox *__restrict__ boxes,
                                                             const int4 *__restrict__ items, int nitems, int parity,
                                                             unsigned *__restrict__ err) {
@@ -198,9 +200,9 @@ __global__ void __launch_bounds__(TXP *TY) batch_psi_kernel(const BatchBox *__re
     const S *g = (const S *)bb.g[in ^ 1];
     float *psi = bb.psi[in ^ 1];
     for (int z = w.z; z < w.w; ++z) {
-      const Nbhd nb(x, y, z, P);
-      const V2 drho = pull_drho<S, PairIO<S>, true>(g, P, nb, px);
-      store_pair_psi<true>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, false>(pad_lane<true>(drho, P, x), P, e));
+      const Nbhd nb(x, y, z, P, ODD ? P.px : P.nx);
+      const V2 drho = pull_drho<S, PairIO<S>, ODD>(g, (unsigned)(ODD ? P.np : P.n), P, nb, px);
+      store_pair_psi<ODD>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, false>(pad_lane<ODD>(drho, P, x), P, e));
     }
   }
   if (e) atomicOr(err, e);
@@ -217,7 +219,7 @@ constexpr int kFlatFusedThreadsPerSM = 640;
 // loop, as in fused_pair_kernel: a persistent kernel looping over the planes of
 // an item held 128 registers (16 warps per SM) and reached 0.86 of the copy
 // bandwidth, this one holds 96 (5 blocks of 128 threads) and 0.94.
-template <typename S, int OP, int TXP, int TY>
+template <typename S, int OP, int TXP, int TY, bool ODD>
 __global__ void __launch_bounds__(TXP *TY, kFlatFusedThreadsPerSM / (TXP * TY)) batch_flat_fused_kernel(const BatchBox *__restrict__ boxes,
                                                                    const int *__restrict__ block_box, int offset,
                                                                    int parity) {
@@ -230,21 +232,21 @@ __global__ void __launch_bounds__(TXP *TY, kFlatFusedThreadsPerSM / (TXP * TY)) 
   const int x = (t % ntx) * (2 * TXP) + 2 * threadIdx.x, y = (t / ntx) * TY + threadIdx.y;
   if (x >= P.nx || y >= P.ny || z >= P.nz) return;
   const int in = bb.cur ^ parity;
-  fused_pair_at<S, OP, true, false, true>((const S *)bb.g[in], (S *)bb.g[in ^ 1], bb.psi[in], P, x, y, z, Rates<V2>(P));
+  fused_pair_at<S, OP, true, false, ODD>((const S *)bb.g[in], (S *)bb.g[in ^ 1], bb.psi[in], P, x, y, z, Rates<V2>(P));
 }
 
 // The fused and psi kernels of one step for a storage type and tile shape;
 // with query set, per_sm receives their resident blocks per SM instead.
-template <typename S, int TXP, int TY>
+template <typename S, int TXP, int TY, bool ODD>
 cudaError_t batch_pair_shape(int eos, const BatchBox *boxes, const int4 *items, int nitems, const int *block_box,
                              const int fused_blocks[2], int parity, int sms, int per_sm[2], bool query, unsigned *err,
                              cudaStream_t s) {
   using K = void (*)(const BatchBox *, const int4 *, int, int, unsigned *);
   K kpsi;
   switch (eos) {
-    case kEosCS: kpsi = batch_psi_kernel<S, kEosCS, TXP, TY>; break;
-    case kEosExp: kpsi = batch_psi_kernel<S, kEosExp, TXP, TY>; break;
-    default: kpsi = batch_psi_kernel<S, kEosNone, TXP, TY>; break;
+    case kEosCS: kpsi = batch_psi_kernel<S, kEosCS, TXP, TY, ODD>; break;
+    case kEosExp: kpsi = batch_psi_kernel<S, kEosExp, TXP, TY, ODD>; break;
+    default: kpsi = batch_psi_kernel<S, kEosNone, TXP, TY, ODD>; break;
   }
   if (query) {
     per_sm[0] = 0;
@@ -252,9 +254,9 @@ cudaError_t batch_pair_shape(int eos, const BatchBox *boxes, const int4 *items, 
   }
   // fused pass: the flat launches (non-orthogonal boxes' blocks first in block_box, then the orthogonal ones)
   if (fused_blocks[0] > 0)
-    batch_flat_fused_kernel<S, kNonOrth, TXP, TY><<<fused_blocks[0], dim3(TXP, TY), 0, s>>>(boxes, block_box, 0, parity);
+    batch_flat_fused_kernel<S, kNonOrth, TXP, TY, ODD><<<fused_blocks[0], dim3(TXP, TY), 0, s>>>(boxes, block_box, 0, parity);
   if (fused_blocks[1] > 0)
-    batch_flat_fused_kernel<S, kOrth, TXP, TY><<<fused_blocks[1], dim3(TXP, TY), 0, s>>>(boxes, block_box, fused_blocks[0],
+    batch_flat_fused_kernel<S, kOrth, TXP, TY, ODD><<<fused_blocks[1], dim3(TXP, TY), 0, s>>>(boxes, block_box, fused_blocks[0],
                                                                                        parity);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -263,49 +265,47 @@ cudaError_t batch_pair_shape(int eos, const BatchBox *boxes, const int4 *items, 
   return cudaGetLastError();
 }
 
-template <typename S>
+template <typename S, bool ODD>
 cudaError_t batch_pair_tile(int tile, int eos, const BatchBox *boxes, const int4 *items, int nitems,
                             const int *block_box, const int fused_blocks[2], int parity, int sms, int per_sm[2],
                             bool query, unsigned *err, cudaStream_t s) {
   switch (tile) {
     case kTile32x4:
-      return batch_pair_shape<S, 16, 4>(eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
+      return batch_pair_shape<S, 16, 4, ODD>(eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
                                         err, s);
     case kTile64x4:
-      return batch_pair_shape<S, 32, 4>(eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
+      return batch_pair_shape<S, 32, 4, ODD>(eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
                                         err, s);
     default:
-      return batch_pair_shape<S, 16, 8>(eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
+      return batch_pair_shape<S, 16, 8, ODD>(eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
                                         err, s);
   }
 }
 
-cudaError_t batch_pair_dispatch(int precision, int tile, int eos, const BatchBox *boxes, const int4 *items, int nitems,
-                                const int *block_box, const int fused_blocks[2], int parity, int sms, int per_sm[2],
-                                bool query, unsigned *err, cudaStream_t s) {
-  if (precision == kF32)
-    return batch_pair_tile<float>(tile, eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query,
-                                  err, s);
-  if (precision == kF16)
-    return batch_pair_tile<__half>(tile, eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm,
-                                   query, err, s);
-  return cudaErrorInvalidValue;
+cudaError_t batch_pair_dispatch(int precision, int tile, int eos, bool odd, const BatchBox *boxes, const int4 *items,
+                                int nitems, const int *block_box, const int fused_blocks[2], int parity, int sms,
+                                int per_sm[2], bool query, unsigned *err, cudaStream_t s) {
+  if (precision != kF32 && precision != kF16) return cudaErrorInvalidValue;
+  auto launch = precision == kF32 ? (odd ? batch_pair_tile<float, true> : batch_pair_tile<float, false>)
+                                  : (odd ? batch_pair_tile<__half, true> : batch_pair_tile<__half, false>);
+  return launch(tile, eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, per_sm, query, err, s);
 }
 
 }  // namespace
 
 bool pair_supported(const KParams &P, int precision) { return precision != kF64 && P.px % 2 == 0; }
 
-cudaError_t batch_pair_occupancy(int precision, int eos, int tile, int per_sm[2]) {
+cudaError_t batch_pair_occupancy(int precision, int eos, int tile, bool odd, int per_sm[2]) {
   const int none[2] = {0, 0};
-  return batch_pair_dispatch(precision, tile, eos, nullptr, nullptr, 0, nullptr, none, 0, 0, per_sm, true, nullptr, 0);
+  return batch_pair_dispatch(precision, tile, eos, odd, nullptr, nullptr, 0, nullptr, none, 0, 0, per_sm, true, nullptr,
+                             0);
 }
 
-cudaError_t launch_batch_pair(int precision, int eos, int tile, const BatchBox *boxes, const int4 *items, int nitems,
-                              const int *block_box, const int fused_blocks[2], int parity, int sms,
+cudaError_t launch_batch_pair(int precision, int eos, int tile, bool odd, const BatchBox *boxes, const int4 *items,
+                              int nitems, const int *block_box, const int fused_blocks[2], int parity, int sms,
                               const int per_sm[2], unsigned *err, cudaStream_t s) {
   int ps[2] = {per_sm[0], per_sm[1]};
-  return batch_pair_dispatch(precision, tile, eos, boxes, items, nitems, block_box, fused_blocks, parity, sms, ps,
+  return batch_pair_dispatch(precision, tile, eos, odd, boxes, items, nitems, block_box, fused_blocks, parity, sms, ps,
                              false, err, s);
 }
 

@@ -297,17 +297,17 @@ template <typename S, bool ODD> __device__ __forceinline__ constexpr bool one_no
   return ODD && std::is_same<S, __half>::value;
 }
 
-// rho - rho_ref of both nodes of a pair from the populations pulled with Ld.
+// rho - rho_ref of both nodes of a pair from the populations pulled with Ld (n: stored nodes of a direction).
 template <typename S, typename Ld, bool ODD>
-__device__ __forceinline__ V2 pull_drho(const S *g, const KParams &P, const Nbhd &nb, const PairX &px) {
+__device__ __forceinline__ V2 pull_drho(const S *g, unsigned n, const KParams &P, const Nbhd &nb, const PairX &px) {
   V2 f[19];
   if constexpr (one_node_rounding<S, ODD>()) {
-    pull_pair<S, Ld, true>(g, (unsigned)P.np, nb, px, f);
+    pull_pair<S, Ld, true>(g, n, nb, px, f);
     if (P.px != P.nx) return drho_lanes<S, 19>(f);
 #pragma unroll
     for (int a = 0; a < 19; ++a) f[a] = PairIO<S>::decode(f[a].v, a);
   } else {
-    pull_pair<S, Ld>(g, (unsigned)P.np, nb, px, f);
+    pull_pair<S, Ld>(g, n, nb, px, f);
   }
   return drho_pair(f);
 }
@@ -361,7 +361,7 @@ __device__ __forceinline__ void psi_pair_at_l2(const S *__restrict__ g, float *_
                                                int x, int y, int z, unsigned &e) {
   const PairX px = pair_x(P, x);
   const Nbhd nb(x, y, z, P);
-  const V2 drho = pull_drho<S, L2Load<S>, ODD>(g, P, nb, px);
+  const V2 drho = pull_drho<S, L2Load<S>, ODD>(g, (unsigned)P.np, P, nb, px);
   store_pair_psi<ODD>(psi, P, x, (unsigned)nb.self, psi_pair<EOS, DF, ICVT>(pad_lane<ODD>(drho, P, x), P, e));
 }
 
