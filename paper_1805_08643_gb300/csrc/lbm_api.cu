@@ -183,7 +183,7 @@ lbm_status ensure_queue(lbm_ctx *c) {
     CK(cudaMemsetAsync(m, 0, bytes, c->L.stream), "clear work list counters");
     return LBM_OK;
   }
-  CK(lbm::queue_grid(c->precision, c->P.q, &grid), "work list occupancy");
+  CK(lbm::queue_grid(c->P, c->precision, &grid), "work list occupancy");
   std::vector<int4> items;
   if (!lbm::queue_items(c->P, grid, items)) return fail(c, LBM_ERR_ARG, "no valid work list for this box");
   const size_t ib = (items.size() * sizeof(int4) + 255) / 256 * 256;

@@ -373,7 +373,7 @@ struct QueueState {
   int *done;
 };
 bool queue_supported(const KParams &P, int precision);
-cudaError_t queue_grid(int precision, int q, int *grid);
+cudaError_t queue_grid(const KParams &P, int precision, int *grid);
 size_t queue_counters(const KParams &P);
 bool queue_items(const KParams &P, int grid, std::vector<int4> &out);
 // stamp: 1 + the number of earlier launches on these counters.
