@@ -195,9 +195,10 @@ cudaError_t by_op(const KParams &P, int op, bool lin, bool df, const void *g_in,
                : by_eos<S, kOrth, false>(P, df, g_in, g_out, psi_in, psi_out, q, stamp, err, s);
 }
 
-// Resident blocks per SM of the kernels a context launches: the smallest over
-// the instantiations of the storage type and lattice, so that a cooperative
-// launch of that many blocks per SM fits whichever one runs.
+// Resident blocks per SM of the kernels a context launches: what the launch
+// bounds promise for every instantiation of the storage type and lattice, so that
+// a cooperative launch of that many fits whichever one runs; fewer where the
+// device gives one of those looked at fewer (shared memory set aside by a tool).
 template <typename S>
 cudaError_t occupancy_of(int q, int *per_sm) {
   using K = void (*)(const S *, S *, const float *, float *, const KParams, const TileMap, const int4 *, int, int *, int,
@@ -213,7 +214,7 @@ cudaError_t occupancy_of(int q, int *per_sm) {
     if (e != cudaSuccess) return e;
     m = std::min(m, v);
   }
-  *per_sm = m;
+  *per_sm = std::min(m, min_blocks(q));
   return cudaSuccess;
 }
 
