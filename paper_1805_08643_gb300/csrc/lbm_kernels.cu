@@ -240,7 +240,9 @@ __device__ __forceinline__ SplitScale split_scale(unsigned max_abs_bits) {
   return s;
 }
 
-// moment_sums of FP32 values through that split, assembled in FP64.
+// moment_sums of FP32 values through that split, assembled in FP64.  s is the scale of
+// v[1..]: v[0] enters r alone and is added there, so that a large one leaves x, y
+// and z their last places.
 template <int Q, bool R>
 __device__ __forceinline__ void moment_sums_split(float v[Q], float axw, const SplitScale &s, double &r, double &x,
                                                   double &y, double &z) {
@@ -249,25 +251,27 @@ __device__ __forceinline__ void moment_sums_split(float v[Q], float axw, const S
   for (int k = 0; k < 3; ++k) {
     float w[Q];
     const float m = k == 0 ? s.m1 : s.m2;
+    w[0] = 0.f;
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
+    for (int a = 1; a < Q; ++a) {
       w[a] = k == 2 ? v[a] : __fsub_rn(__fadd_rn(v[a], m), m);
       v[a] = __fsub_rn(v[a], w[a]);
     }
     moment_sums<Q, R, float>(w, axw, h[k][0], h[k][1], h[k][2], h[k][3]);
   }
   auto join = [&](int q) { return widen_f32(h[0][q]) + (widen_f32(h[1][q]) + widen_f32(h[2][q])); };
-  if (R) r = join(0);
+  if (R) r = widen_f32(v[0]) + join(0);
   x = join(1);
   y = join(2);
   z = join(3);
 }
 
+// Of v[1..].
 template <int Q>
 __device__ __forceinline__ unsigned max_abs_bits(const float v[Q]) {
   unsigned m = 0;
 #pragma unroll
-  for (int a = 0; a < Q; ++a) m = max(m, __float_as_uint(v[a]) & 0x7fffffffu);
+  for (int a = 1; a < Q; ++a) m = max(m, __float_as_uint(v[a]) & 0x7fffffffu);
   return m;
 }
 
