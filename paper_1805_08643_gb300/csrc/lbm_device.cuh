@@ -206,35 +206,37 @@ __device__ __forceinline__ double recip(double x) {
 }
 
 // psi0 exp(-rho0 / rho) rounded to FP32.  With CUDA's FP64 division and exp()
-// it took about 85 FP64 instructions a node (70 us per 80^3 work-list step, 45
-// with this one); this one takes 11, and everything that FP32 can carry without
-// showing in the result runs there:
-//   y = -rho0 log2(e) / rho: an FP32 reciprocal and one Newton step in FP64
-//     (relative error 2^-45, so 2^-38 at most in y where |y| < 100);
+// it took about 85 FP64 instructions a node (70 us per 80^3 work-list step); this
+// one takes 15, and what FP32 can carry without showing in an FP64 result runs
+// there:
+//   y = -rho0 log2(e) / rho: an FP32 reciprocal and one cubic Newton step in FP64;
 //   exp(-rho0 / rho) = 2^k 2^f, k = round(y), |f| <= 1/2: the Taylor series of
-//     2^f (coefficients ln(2)^j / j!), terms 0 to 4 in FP64, terms 5 to 10,
-//     together below 2^-14, in FP32.
-// The FP64 value before the rounding is good to 2^-37: against the extended-
-// precision function the rounded result's largest and rms errors over
-// rho in [0.05, 6] equal those of the FP64 exp() to eight digits.  Exponents of
-// 100 and above (results near or beyond FP32's range), and everything
-// that is not finite, take the FP64 functions.
-__device__ __forceinline__ float exp_psi(double rho, float rho_f, const KParams &P) {
+//     2^f (coefficients ln(2)^j / j!), terms 0 to 7 in FP64, terms 8 to 12,
+//     together below 2^-27, in FP32; the next is below 2^-52.
+// The FP64 value before the rounding is good to 2^-48.3 over rho in [0.05, 6], 2^-46.4
+// in [0.015, 0.05], whatever rho_ref (rho0 = 1; the FP64 exp() of the FP64 quotient:
+// 2^-48.9, 2^-47.0; both by the rounding of the exponent, which exp multiplies by its
+// size), and none of 2 10^6 results rounded to FP32 differs.  Exponents of 100 and above
+// (results near or beyond FP32's range), and everything that is not finite, take the
+// FP64 functions.
+__device__ __forceinline__ float exp_psi(double rho, const KParams &P) {
   float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(rho_f));
-  const double r0 = widen_f32(r), y0 = P.exp_k * r0;
-  const double y = fma(y0, fma(-rho, r0, 1.0), y0);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(narrow_f64(rho)));
+  const double r0 = widen_f32(r), e = fma(-rho, r0, 1.0), y0 = P.exp_k * r0;
+  const double y = fma(y0, fma(e, e, e), y0);
   const float yf = narrow_f64(y);
   if (!(fabsf(yf) < 100.0f)) return (float)(P.psi0 * exp(-P.rho0 / rho));
   const float k = rintf(yf);
   const double f = y - widen_f32(k);
   const float g = narrow_f64(f);
-  float t = fmaf(7.054911620801121e-09f, g, 1.0178086009239696e-07f);
+  float t = fmaf(2.5678435993488196e-11f, g, 4.445538271870811e-10f);
+  t = fmaf(t, g, 7.054911620801121e-09f);
+  t = fmaf(t, g, 1.0178086009239696e-07f);
   t = fmaf(t, g, 1.3215486790144305e-06f);
-  t = fmaf(t, g, 1.5252733804059838e-05f);
-  t = fmaf(t, g, 1.5403530393381606e-04f);
-  t = fmaf(t, g, 1.3333558146428441e-03f);
-  double p = fma(widen_f32(t), f, 0.009618129107628477);
+  double p = fma(widen_f32(t), f, 1.5252733804059838e-05);
+  p = fma(p, f, 1.5403530393381606e-04);
+  p = fma(p, f, 1.3333558146428441e-03);
+  p = fma(p, f, 0.009618129107628477);
   p = fma(p, f, 0.055504108664821576);
   p = fma(p, f, 0.2402265069591007);
   p = fma(p, f, 0.6931471805599453);
@@ -254,7 +256,7 @@ __device__ __forceinline__ float eos_psi_d(float d, const KParams &P, unsigned &
   const float rho_f = P.frho_ref + d;
   if (!isfinite(rho_f)) { err |= kErrNonFinite; return nan; }
   if (!(rho_f > 0.0f)) { err |= kErrEosDomain; return nan; }
-  if (EOS == kEosExp) return exp_psi(P.rho_ref + widen_f32(d), rho_f, P);
+  if (EOS == kEosExp) return exp_psi(P.rho_ref + widen_f32(d), P);
   if (!(rho_f < P.f_rho_max)) { err |= kErrEosDomain; return nan; }
   const double x = ICVT ? widen_f32(d) : (double)d;
   const double X = fma(fma(fma(fma(fma(P.c[5], x, P.c[4]), x, P.c[3]), x, P.c[2]), x, P.c[1]), x, P.c[0]);
@@ -302,7 +304,7 @@ __device__ __forceinline__ float eos_psi_f2(float drho, const KParams &P, unsign
   const float rho_f = P.frho_ref + drho;
   if (!isfinite(rho_f)) { err |= kErrNonFinite; return nan; }
   if (!(rho_f > 0.0f)) { err |= kErrEosDomain; return nan; }
-  if (EOS == kEosExp) return exp_psi(P.rho_ref + widen_f32(drho), rho_f, P);
+  if (EOS == kEosExp) return exp_psi(P.rho_ref + widen_f32(drho), P);
   if (!(rho_f < P.f_rho_max)) { err |= kErrEosDomain; return nan; }
   F2 rho = two_sum(P.rr_h, drho);
   rho = fast_two_sum(rho.h, __fadd_rn(rho.l, P.rr_l));
