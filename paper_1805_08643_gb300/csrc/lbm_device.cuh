@@ -193,8 +193,8 @@ __device__ __forceinline__ float narrow_f64(double v) {
   return __uint_as_float(r);
 }
 
-// 1 / x in FP64: an FP32 reciprocal (error 2^-23) and one cubic Newton step,
-// r (1 + e + e^2) with e = 1 - x r, three FP64 instructions, wrong by 2^-69
+// 1 / x in FP64: an FP32 reciprocal (of x rounded to FP32: |e| < 2^-22, e = 1 - x r) and
+// one cubic Newton step, r (1 + e + e^2), three FP64 instructions, wrong by 2^-66
 // before its last rounding; exponents FP32 cannot hold take the division.
 __device__ __forceinline__ double recip(double x) {
   const unsigned e11 = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
@@ -203,6 +203,17 @@ __device__ __forceinline__ double recip(double x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(narrow_f64(x)));
   const double r0 = widen_f32(r), e = fma(-x, r0, 1.0);
   return fma(r0, fma(e, e, e), r0);
+}
+// a / x from inv = recip(x): the product and its remainder, one rounding like the
+// division's (a product alone has two); what is not finite takes the division.
+__device__ __forceinline__ double quotient(double a, double x, double inv) {
+  const double q = a * inv;
+  double c = fma(fma(-q, x, a), inv, q);
+  if ((__double2hiint(c) & 0x7ff00000) == 0x7ff00000) {
+    asm volatile("" : "+d"(x));  // a branch, not a division computed for every node and selected
+    c = a / x;
+  }
+  return c;
 }
 
 // psi0 exp(-rho0 / rho) rounded to FP32.  With CUDA's FP64 division and exp()

@@ -183,11 +183,12 @@ __global__ void __launch_bounds__(256) fused_kernel(const typename Types<PREC>::
 // bound by the FP64 unit unless almost all of the work runs elsewhere: with
 // every conversion, sum and division in FP64 (149 instructions per node) the
 // fields of a 256^3 FP32 box took 5.11 ms, against 0.28 ms for their bytes;
-// they take 0.88 ms now (FP16 storage: 5.89 -> 1.7, FP64 at 128^3: 0.50 -> 0.29).
+// they take 0.99 ms now (FP16 storage: 5.89 -> 0.98, FP64 at 128^3: 0.50 -> 0.31).
 // Both forms below share the pair differences among the sums and take one
-// reciprocal for the three velocities.  The FP32-arithmetic forms also take
-// their sums on the FP32 units, exactly (split_scale), which leaves 29 FP64
-// instructions per node.
+// reciprocal for the three velocities (0.82 ms without their remainders, which
+// round each like a division).  The FP32-arithmetic forms also take their sums
+// on the FP32 units, exactly (split_scale), which leaves 36 FP64 instructions
+// per node.
 
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
@@ -330,20 +331,20 @@ __global__ void moments_kernel(const typename Types<PREC>::S *__restrict__ g,
   if (rho_out) rho_out[i] = rho;
   if (u_out) {
     const double inv = recip(rho);
-    u_out[i] = rux * inv;
-    u_out[(size_t)P.n + i] = ruy * inv;
-    u_out[2 * (size_t)P.n + i] = ruz * inv;
+    u_out[i] = quotient(rux, rho, inv);
+    u_out[(size_t)P.n + i] = quotient(ruy, rho, inv);
+    u_out[2 * (size_t)P.n + i] = quotient(ruz, rho, inv);
   }
 }
 
-// Block-partial FP64 sums of (rho, rho u) and max |u|^2, grid-stride over
-// nodes, then one block folds the partials in a fixed order (deterministic)
-// and takes the root.
+// Block-partial FP64 sums of (rho, rho u) and max |u|, grid-stride over nodes,
+// then one block folds the partials in a fixed order (deterministic).
 template <int PREC, int Q>
 __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<PREC>::S *__restrict__ g,
                                                            const typename Types<PREC>::Psi *__restrict__ psi,
                                                            const KParams P, double *__restrict__ partials) {
   double acc[5] = {0, 0, 0, 0, 0};
+  double most = 0.0, most_j2 = 0.0, most_rho = 1.0;  // the fastest node: |u|^2 (to compare), |rho u|^2 and rho
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
     const int x = i % P.nx, yz = i / P.nx, y = yz % P.ny, z = yz / P.ny;
     const Nbhd nb(x, y, z, P);
@@ -354,10 +355,12 @@ __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<
     acc[2] += ruy;
     acc[3] += ruz;
     const double inv = recip(rho);
-    double u2 = (rux * rux + ruy * ruy + ruz * ruz) * (inv * inv);
+    const double j2 = rux * rux + ruy * ruy + ruz * ruz;
+    double u2 = j2 * inv * inv;
     if (__double2hiint(rho) < 0) u2 = -u2;  // a negative density never holds the maximum
-    acc[4] = (u2 > acc[4] || u2 != u2) ? u2 : acc[4];
+    if (u2 > most || u2 != u2) most = u2, most_j2 = j2, most_rho = rho;
   }
+  acc[4] = sqrt(most_j2) / most_rho;
   __shared__ double red[5][256];
 #pragma unroll
   for (int k = 0; k < 5; ++k) red[k][threadIdx.x] = acc[k];
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(256) max_du_kernel(const typename Types<PREC>:
     double rho, rux, ruy, ruz;
     node_moments<PREC, Q>(g, psi, P, nb, rho, rux, ruy, ruz);
     const double inv = recip(rho);
-    const double u[3] = {rux * inv, ruy * inv, ruz * inv};
+    const double u[3] = {quotient(rux, rho, inv), quotient(ruy, rho, inv), quotient(ruz, rho, inv)};
     double d2 = 0.0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -435,7 +438,7 @@ __global__ void __launch_bounds__(256) diag_final_kernel(const double *__restric
     }
     __syncthreads();
   }
-  if (threadIdx.x < 5) result[threadIdx.x] = threadIdx.x == 4 ? sqrt(red[4][0]) : red[threadIdx.x][0];
+  if (threadIdx.x < 5) result[threadIdx.x] = red[threadIdx.x][0];
 }
 
 // ------------------------------------------------------------------ initial state
