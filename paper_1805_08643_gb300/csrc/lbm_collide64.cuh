@@ -76,6 +76,7 @@ struct InDouble {
   __device__ __forceinline__ double in(double v) const { return v; }
   __device__ __forceinline__ double out(double v) const { return v; }
   __device__ __forceinline__ double out_half(double v) const { return 0.5 * v; }
+  template <int K> __device__ __forceinline__ double out_over(double v) const { return v * (1.0 / (1 << K)); }
   __device__ __forceinline__ double out_twice(double v) const { return 2.0 * v; }
   static __device__ __forceinline__ double half(double v) { return 0.5 * v; }
 };
@@ -92,6 +93,7 @@ template <int S> struct InFixed {
   }
   __device__ __forceinline__ double out(Fixed x) const { return back(x, E); }
   __device__ __forceinline__ double out_half(Fixed x) const { return back(x, E - 1); }
+  template <int K> __device__ __forceinline__ double out_over(Fixed x) const { return back(x, E - K); }  // over 2^K
   __device__ __forceinline__ double out_twice(Fixed x) const { return back(x, E + 1); }
   static __device__ __forceinline__ Fixed half(Fixed x) { return {x.v >> 1}; }
   static __device__ __forceinline__ double back(Fixed x, int E) {
@@ -179,8 +181,19 @@ struct Node64 {
   }
 };
 
+// The even moments that carry the density, m4 and the fourth-order ones, of the
+// raw-monomial bases (the non-orthogonal operator and D3Q15): m + s d, d = m_eq + (c / s) S
+// - m, with the density's part of m_eq and m subtracted first, so that d is small and
+// the result is rounded once at the size of m.  (As a m + s m_eq + c S, whose terms all
+// round at that size, rest populations were up to a fifth further off than FP64
+// sums'.)  m4:
+__device__ __forceinline__ double relax4(double m, double drho, double usq, double Fu, double S2, const Coeffs64 &C) {
+  const double d = (drho - m) + fma(C.k[kE5], S2, fma(C.k[kE4], Fu, usq));
+  return fma(C.k[kE1], d, m);
+}
+
 // ------------------------------------------------------------------ non-orthogonal operator
-// f* = M^-1 m* (App. A) from drho, e4 = m4* / 6, e5 = m5* / 12, e6 = m6* / 4,
+// f* = M^-1 m* (App. A) from drho - m4*, e4 = m4* / 6, e5 = m5* / 12, e6 = m6* / 4,
 // p_k = m_k* / 4 (16, 17, 18, 7, 8, 9), twice the odd parts of the axes, and the
 // odd parts of the diagonals.
 template <typename Sc, typename Out>
@@ -189,7 +202,7 @@ __device__ __forceinline__ void inverse_nonorth_l(const double (&v)[19], const S
   const L e4 = c.in(v[1]), e5 = c.in(v[2]), e6 = c.in(v[3]);
   const L p16 = c.in(v[4]), p17 = c.in(v[5]), p18 = c.in(v[6]);
   const L a = p16 + p17;
-  out(0, fma(4.0, c.out(a + p18), fma(-6.0, v[1], v[0])));  // drho in the sums would set their cut
+  out(0, fma(4.0, c.out(a + p18), v[0]));  // v[0] in the sums would set their cut
   auto axis = [&](int k, const L &even2, double odd2) {  // both twice their value
     const L o = c.in(odd2);
     out(k, c.out_half(even2 + o));
@@ -242,14 +255,19 @@ __device__ __forceinline__ void collide_nonorth_l(const double (&f_)[19], const 
   const Node64 N(rho_ref + drho, jx, jy, jz, Fx, Fy, Fz, S2);
   const double usq = N.qxx + N.qyy + N.qzz, Fu = N.Fux + N.Fuy + N.Fuz;
   double v[19];
-  v[0] = drho;
   // relaxed moments (Eq. 4 with Eqs. 11, 13, 14, 16), scaled as the inverse takes them
-  v[1] = C.k[kE1] * c.out(sax + times<2>(sdg)) + C.k[kE2] * (drho + usq) + C.k[kE4] * Fu + C.k[kE5] * S2;
-  // Eq. 13's phi + (rho - rho_ref)/9 and third-axis parts: m16 takes the sum over the axes less the z part, ...
-  const double c4 = C.k[kP2] * drho + C.k[kP3] * usq + C.k[kP4] * Fu;
-  v[4] = C.k[kP1] * c.out(l16) + (c4 - (C.k[kP5] * N.qzz + C.k[kP4] * N.Fuz));
-  v[5] = C.k[kP1] * c.out(l17) + (c4 - (C.k[kP5] * N.qyy + C.k[kP4] * N.Fuy));
-  v[6] = C.k[kP1] * c.out(l18) + (c4 - (C.k[kP5] * N.qxx + C.k[kP4] * N.Fux));
+  const double m4 = relax4(c.out(sax + times<2>(sdg)), drho, usq, Fu, S2, C);
+  v[0] = drho - m4;
+  v[1] = (1.0 / 6.0) * m4;
+  // Eq. 13's phi + (rho - rho_ref)/9 and third-axis parts, over 4: m16 takes the sum over the axes less the z part, ...
+  const double c4 = fma(C.k[kP4], Fu, (1.0 / 24.0) * usq);
+  auto relax_p = [&](double m, double q, double Fq) {
+    const double d = fma(1.0 / 36.0, drho, -m) + fma(-C.k[kP4], Fq, fma(-1.0 / 12.0, q, c4));
+    return fma(C.k[kP1], d, m);
+  };
+  v[4] = relax_p(c.template out_over<2>(l16), N.qzz, N.Fuz);
+  v[5] = relax_p(c.template out_over<2>(l17), N.qyy, N.Fuy);
+  v[6] = relax_p(c.template out_over<2>(l18), N.qxx, N.Fux);
   const Shear64 n = shear64<19>(P, C, N.rho);
   const double Bx = n.b1 * N.rux + n.b2 * Fx, By = n.b1 * N.ruy + n.b2 * Fy, Bz = n.b1 * N.ruz + n.b2 * Fz;
   const double Gx = N.ux * Bx, Gy = N.uy * By, Gz = N.uz * Bz;
@@ -378,14 +396,14 @@ __device__ __forceinline__ void collide_orth_l(const double (&f_)[19], const Sc 
 
 // ------------------------------------------------------------------ D3Q15
 // The basis and readings of lbm_q15.cuh; the four odd corner moments relax with one
-// rate, so the corner differences relax themselves.  v: drho, m4* / 6, -m5* / 12,
+// rate, so the corner differences relax themselves.  v: drho - m4*, m4* / 6, -m5* / 12,
 // m6* / 4, m_k* / 8 (14, 7, 8, 9), twice the odd parts of the axes, the odd parts of
 // the corner pairs.
 template <typename Sc, typename Out>
 __device__ __forceinline__ void inverse_q15_l(const double (&v)[15], const Sc &c, Out &&out) {
   using L = typename Sc::Value;
   const L e4 = c.in(v[1]), e5 = c.in(v[2]), e6 = c.in(v[3]), p14 = c.in(v[4]);
-  out(0, fma(16.0, v[4], fma(-6.0, v[1], v[0])));
+  out(0, fma(16.0, v[4], v[0]));
   auto axis = [&](int k, const L &even, double odd2) {
     const L e = times<2>(even), o = c.in(odd2);
     out(k, c.out_half(e + o));
@@ -434,9 +452,11 @@ __device__ __forceinline__ void collide_q15_l(const double (&f_)[15], const Sc &
   const Node64 N(rho_ref + drho, jx, jy, jz, Fx, Fy, Fz, S2);
   const double usq = N.qxx + N.qyy + N.qzz, Fu = N.Fux + N.Fuy + N.Fuz;
   double v[15];
-  v[0] = drho;
-  v[1] = C.k[kE1] * c.out(sax + times<3>(l14)) + C.k[kE2] * (drho + usq) + C.k[kE4] * Fu + C.k[kE5] * S2;
-  v[4] = C.k[kP1] * c.out(l14) + C.k[kP2] * drho + C.k[kP3] * usq + C.k[kP4] * Fu;
+  const double m4 = relax4(c.out(sax + times<3>(l14)), drho, usq, Fu, S2, C);
+  v[0] = drho - m4;
+  v[1] = (1.0 / 6.0) * m4;
+  const double p14 = c.template out_over<3>(l14);
+  v[4] = fma(C.k[kP1], fma(1.0 / 72.0, drho, -p14) + fma(C.k[kP4], Fu, (1.0 / 144.0) * usq), p14);
   const Shear64 n = shear64<15>(P, C, N.rho);
   const double Bx = n.b1 * N.rux + n.b2 * Fx, By = n.b1 * N.ruy + n.b2 * Fy, Bz = n.b1 * N.ruz + n.b2 * Fz;
   const double Gx = N.ux * Bx, Gy = N.uy * By, Gz = N.uz * Bz;

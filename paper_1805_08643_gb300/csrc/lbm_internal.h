@@ -195,7 +195,7 @@ enum Coeff {
   kQ2,        // a_q                    (non-orthogonal and D3Q15)
   kQa,        // a_q / 2; orthogonal: a_q / 40
   kQb1, kQb2, // s_q / 12, c_q / 12; orthogonal over 60, D3Q15 over 24
-  // energy; non-orthogonal: moment 4 over 6; orthogonal: e over 2394
+  // energy; non-orthogonal and D3Q15: of moment 4 (relax4); orthogonal: of e over 2394
   kE1, kE2, kE3, kE4, kE5,
   // fourth-order moments over 4 (D3Q15: over 8); orthogonal: pi_xx over 72
   kP1, kP2, kP3, kP4, kP5,
@@ -251,26 +251,20 @@ inline Coeffs64 coeffs64(const KParams &P, int op) {
     k[kQa] = (1 - sq) / 2;
     k[kQb1] = sq / 12;
     k[kQb2] = cq / 12;
-    k[kE1] = (1 - se) / 6;
-    k[kE2] = se / 6;
-    k[kE4] = 2 * ce / 6;
-    k[kE5] = ce * sig / 6;
+    k[kE1] = se;
+    k[kE4] = 2 * ce / se;
+    k[kE5] = ce * sig / se;
     if (op == kNonOrth) {
-      k[kP1] = (1 - sp) / 4;
-      k[kP2] = sp / 36;  // drho
-      k[kP3] = sp / 24;  // usq
-      k[kP4] = cp / 6;   // F . u
-      k[kP5] = sp / 12;  // rho u_i^2
+      k[kP1] = sp;
+      k[kP4] = cp / (6 * sp);  // F . u
     } else {             // D3Q15: corner moments over 8
       k[kON] = (1 - sn) / 8;
       k[kNb1] = sn / 16;
       k[kNb2] = cn / 8;
       k[kQb1] = sq / 24;
       k[kQb2] = cq / 24;
-      k[kP1] = (1 - sp) / 8;
-      k[kP2] = sp / 72;
-      k[kP3] = sp / 144;
-      k[kP4] = cp / 18;
+      k[kP1] = sp;
+      k[kP4] = cp / (18 * sp);
     }
   }
   return c64;
