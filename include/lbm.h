@@ -334,8 +334,9 @@ lbm_status lbm_batch_init_flat(lbm_batch *b, int id, int axis, double lo, double
  * block-to-box table of 4 bytes per block), then the psi pass over work items
  * of a tile through z planes.  Boxes with an odd Nx step like
  * the others (their stored rows hold one element more), but for boxes so large
- * that the longer rows would leave the index range (19 N near 2^32): those run
- * the one-node single pass in the same step, tile shape as chosen (32x8 under 3).  For box id >= 0,
+ * that the longer rows would leave the index range (19 N near 2^32) or a plane the
+ * work list's tile numbers (about 16.7 10^6 nodes): those run the one-node single
+ * pass in the same step, tile shape as chosen (32x8 under 3).  For box id >= 0,
  * z_planes sets its planes per work item of the psi pass and the single pass
  * (0 = automatic).  Results do not depend on the choice (the work list and the
  * two-pass kernels are equal bit for bit). */

@@ -6,6 +6,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
 namespace lbm {
@@ -76,10 +77,14 @@ inline unsigned row_multiplier(long long d, long long count) {
 }
 
 // KParams::px of a box: rows of an odd nx get one element more where the
-// two-node kernels run, unless that leaves the index range (19 np < 2^32).
+// two-node kernels run, unless that leaves the index range (19 np < 2^32) or a
+// plane has more tiles, of 128 pairs or 64 x 4 nodes, than the 16 bits a batch's
+// work list has for one (65535: 16.7 10^6 nodes): the one-node kernels step those.
 inline int stored_row(int precision, const int grid[3]) {
-  const long long padded = (long long)(grid[0] + 1) * grid[1] * grid[2];
-  return precision != kF64 && grid[0] % 2 != 0 && 19 * padded < (1LL << 32) ? grid[0] + 1 : grid[0];
+  const long long plane = (long long)(grid[0] + 1) * grid[1];
+  const long long tiles = std::max((plane / 2 + 127) / 128, (grid[0] + 63LL) / 64 * ((grid[1] + 3LL) / 4));
+  return precision != kF64 && grid[0] % 2 != 0 && 19 * plane * grid[2] < (1LL << 32) && tiles <= 0xffff ? grid[0] + 1
+                                                                                                         : grid[0];
 }
 
 constexpr int kDefaultSpinLimit = 1 << 22;
