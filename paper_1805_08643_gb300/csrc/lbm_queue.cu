@@ -61,17 +61,19 @@ namespace lbm {
 namespace {
 
 // Resident blocks per SM the register budgets are set for.  The fused jobs wait
-// for memory most of the time, so a block more is worth more than the spills it
-// costs, up to a point; taking the force from psi before the populations are
-// pulled (FORCE_FIRST) is what lets a thread live on 72 registers.  256^3 FP32
-// steps, non-orthogonal / D3Q15, at 6, 7 and 8 blocks: 527 / 457, 515 / 444 and
-// 551 / 430 us (192^3: 250 / 229, 220 / 235 and 233 / 190; with every V2
-// difference one instruction, see operator-; 526 / 431 us as it is).  Batches stay at 6
-// (848 against 842 us for 64 boxes at 7, with 180 bytes spilled).
+// for memory most of the time, so a block more is worth some spilled registers,
+// up to a point; taking the force from psi before the populations are pulled
+// (FORCE_FIRST) is what lets a thread live on 80 or fewer.  Steps at 6, 7 and 8
+// blocks: 256^3 FP32 non-orthogonal 508, 523 and 583 us, orthogonal 526, 538 and 603,
+// D3Q15 436 (6 and 7) and 429; 192^3 218, 223 and 249, 224, 228 and 258, 187 and 185;
+// FP16 storage at 6 and 7 256^3 485 and 455, 192^3 208 and 195.  Batches take 6 (848
+// against 842 us for 64 boxes at 7, with 180 bytes spilled).
 constexpr int kBatchBlocks = 6;
 // FP16 batches with odd boxes collide those node by node (force_collide_lanes): 372 bytes spilled at 6 blocks.
 constexpr int kOddHalfBatchBlocks = 5;
-__host__ __device__ constexpr int min_blocks(int q) { return q == 15 ? 8 : 7; }
+template <typename S> __host__ __device__ constexpr int min_blocks(int q) {
+  return q == 15 ? 8 : std::is_same<S, __half>::value ? 7 : 6;
+}
 // The psi jobs convert to and from FP64 with the conversion instructions, not
 // the integer path of the psi pass kernel (the same results): this kernel is
 // not bound by the FP64 unit, and the integer work cost 1 % (FP32 storage) and
@@ -94,7 +96,7 @@ __device__ __forceinline__ int next_item(unsigned c, int nitems, unsigned &e) {
 // Q: 19 (both operators) or 15 (the D3Q15 non-orthogonal variant).  LIN: TileMap::lin.
 // The Eq. 16 term is compiled in (a zero coefficient switches it off).
 template <typename S, int OP, bool LIN, int EOS, bool DF, int Q>
-__global__ void __launch_bounds__(NTH, min_blocks(Q))
+__global__ void __launch_bounds__(NTH, min_blocks<S>(Q))
     queue_kernel(const S *__restrict__ g_in, S *__restrict__ g_out, const float *__restrict__ psi_in,
                  float *__restrict__ psi_out, const KParams P, const TileMap G, const int4 *__restrict__ items,
                  int nitems, int *__restrict__ done, int stamp, unsigned *__restrict__ err) {
@@ -214,7 +216,7 @@ cudaError_t occupancy_of(int q, int *per_sm) {
     if (e != cudaSuccess) return e;
     m = std::min(m, v);
   }
-  *per_sm = std::min(m, min_blocks(q));
+  *per_sm = std::min(m, min_blocks<S>(q));
   return cudaSuccess;
 }
 
@@ -347,12 +349,15 @@ std::vector<long long> by_ready(const std::vector<long long> &ready) {
 
 // Items between a psi job and the last fused job it reads: 3/8 of a wave of the
 // grid where a plane is large (the populations leave L2 sooner), 5/8 where it
-// is small (more of the list hangs on each plane).  At 1/4, 3/8, 1/2, 5/8 and
-// 3/4: 128^3 89.0, 84.2, 78.4, 74.3 and 73.7 us per step, 160^3 164, 148, 136,
-// 134 and 135, 256^3 558, 514, 518, 526 and 534, 512^3 4.66, 4.32, 4.34, 4.38 and
-// 4.42 ms; 192^3 (144 tiles a plane) 267, 236, 220, 220 and 222.
+// is small (more of the list hangs on each plane).  FP32 non-orthogonal steps at 1/4,
+// 3/8, 1/2, 5/8 and 3/4: 128^3 (64 tiles a plane) 89.8, 84.4, 77.4, 72.8 and 71.7 us,
+// 160^3 (100) 167, 152, 136, 133 and 133, 192^3 (144) 267, 225, 218.5, 218 and 219,
+// 224^3 (196) 428, 364, 353, 355 and 359, 240^3 (225) 525, 432, 423, 425 and 430,
+// 256^3 537, 508, 511, 518 and 527, 320^3 (400) 1120, 1001, 1002, 1012 and 1024, 512^3
+// 4.51, 4.38, 4.40, 4.43 and 4.46 ms; orthogonal and D3Q15 boxes alike (D3Q15 240^3
+// 489, 377, 360, 360 and 361).
 long long psi_lag(int grid, int tiles_per_plane) {
-  return std::max(1LL, (long long)grid * (tiles_per_plane < 192 ? 5 : 3) / 8);
+  return std::max(1LL, (long long)grid * (tiles_per_plane < 240 ? 5 : 3) / 8);
 }
 
 // Psi jobs go to the first free item at least `lag` items after the last of
@@ -378,9 +383,10 @@ bool place_psi_jobs(std::vector<int4> &out, const std::vector<long long> &ready,
 // wherever the row does, whatever Nx is; 64 x 4 tiles leave lanes idle where Nx
 // is no multiple of 64 or Ny of 4 (80 x 80: 38 %, 200 x 180: 22 %), and tiles
 // narrowed to 16 nodes start off a 32-byte sector in most rows.  They are also
-// the faster ones where 64 x 4 fits: per step, 64 x 4 / consecutive, 80^3 36.9 /
-// 25.5 us, 160^3 184 / 136, 192^3 259 / 220, 200 x 180 x 256 (orthogonal) 379 /
-// 304, 256^3 530 / 518; a batch of six boxes of edges 62 to 140 314 / 257 (16-
+// the faster ones where 64 x 4 fits: per step, 64 x 4 (with the better lag) /
+// consecutive, 80^3 34.3 / 26.3 us, 128^3 73.9 / 72.8, 160^3 148 / 133, 192^3 225 /
+// 218, 200 x 180 x 256 (orthogonal) 354 / 295, 256^3 535 / 508, 320^3 1028 / 1001,
+// 512^3 4.49 / 4.38 ms; a batch of six boxes of edges 62 to 140 314 / 257 us (16-
 // and 32-node tiles: 301).  A psi job then waits for whole rows around its
 // tile; past 512 nodes a row that is more tiles than a warp has lanes to poll
 // with, and the 64 x 4 tiles take over.
