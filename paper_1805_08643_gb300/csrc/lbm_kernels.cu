@@ -343,8 +343,8 @@ template <int PREC, int Q>
 __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<PREC>::S *__restrict__ g,
                                                            const typename Types<PREC>::Psi *__restrict__ psi,
                                                            const KParams P, double *__restrict__ partials) {
-  double acc[5] = {0, 0, 0, 0, 0};
-  double most = 0.0, most_j2 = 0.0, most_rho = 1.0;  // the fastest node: |u|^2 (to compare), |rho u|^2 and rho
+  // sums of rho and rho u; of the fastest node |u|^2 (to compare by), |rho u|^2 and rho
+  double acc[7] = {0, 0, 0, 0, 0, 0, 1};
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
     const int x = i % P.nx, yz = i / P.nx, y = yz % P.ny, z = yz / P.ny;
     const Nbhd nb(x, y, z, P);
@@ -358,25 +358,25 @@ __global__ void __launch_bounds__(256) diag_partial_kernel(const typename Types<
     const double j2 = rux * rux + ruy * ruy + ruz * ruz;
     double u2 = j2 * inv * inv;
     if (__double2hiint(rho) < 0) u2 = -u2;  // a negative density never holds the maximum
-    if (u2 > most || u2 != u2) most = u2, most_j2 = j2, most_rho = rho;
+    if (u2 > acc[4] || u2 != u2) acc[4] = u2, acc[5] = j2, acc[6] = rho;
   }
-  acc[4] = sqrt(most_j2) / most_rho;
-  __shared__ double red[5][256];
+  __shared__ double red[7][256];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) red[k][threadIdx.x] = acc[k];
+  for (int k = 0; k < 7; ++k) red[k][threadIdx.x] = acc[k];
   __syncthreads();
   for (int s = blockDim.x / 2; s > 0; s >>= 1) {
     if (threadIdx.x < s) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + s];
       const double a = red[4][threadIdx.x], b = red[4][threadIdx.x + s];
-      red[4][threadIdx.x] = (b > a || b != b) ? b : a;
+      if (b > a || b != b)
+#pragma unroll
+        for (int k = 4; k < 7; ++k) red[k][threadIdx.x] = red[k][threadIdx.x + s];
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) partials[blockIdx.x * 5 + k] = red[k][0];
+  if (threadIdx.x < 4) partials[blockIdx.x * 5 + threadIdx.x] = red[threadIdx.x][0];
+  if (threadIdx.x == 0) partials[blockIdx.x * 5 + 4] = sqrt(red[5][0]) / red[6][0];
 }
 
 // max over nodes of |u(x) - u_prev(x)| (Eq. 6 velocity, FP64), folded into

@@ -36,11 +36,13 @@ namespace {
 
 constexpr int kBlocks = 7;  // resident blocks per SM the registers are set for
 // Tiles per block up to which a box is stepped here: per step, this kernel /
-// the list, 32^3 4.9 / 10.3 us, 48^3 7.0 / 10.3, 64^3 10.0 / 16.4, 80^3 17.9 / 25.3,
-// 96^3 34.6 / 40.6, 104^3 (4.1 tiles per block) 46.5 / 50.9, 112^3 (5.2) 59.5 /
-// 59.9, 128^3 77.3 / 77.7; D3Q15 96^3 28.9 / 36.4, 112^3 50.3 / 50.8.  (With 6
-// blocks per SM 64^3 takes 12.8, with 8 10.9.)
-constexpr int kMaxTiles = 5;
+// the list, 32^3 4.9 / 9.3 us, 48^3 7.2 / 12.1, 64^3 10.2 / 18.9, 80^3 18.1 / 26.6,
+// 96^3 34.4 / 38.7, 104^3 (4.1 tiles per block) 47.0 / 45.9, 112^3 (5.2) 59.3 / 53.1;
+// D3Q15 64^3 9.1 / 16.4, 96^3 29.1 / 35.0, 104^3 38.8 / 41.1, 112^3 50.4 / 47.5.  (At 6, 7
+// and 8 blocks per SM 64^3 takes 13.0, 10.2 and 11.3 us, 80^3 20.5, 18.1 and 19.5, 96^3
+// 33.6, 34.5 and 34.6.  At 7, 72 registers, the D3Q19 kernels spill 84 to 136 bytes,
+// the D3Q15 ones 48 to 60.)
+constexpr int max_tiles(int q) { return q == 15 ? 5 : 4; }
 
 struct StepBuffers {
   float *g[2], *psi[2];  // [0]: the state the launch starts from
@@ -130,7 +132,7 @@ cudaError_t steps_grid(const KParams &P, int precision, int *grid) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   if (e != cudaSuccess) return e;
   const long long nf = (long long)P.nz * G.T, most = (long long)kBlocks * sms;
-  if (!coop || !G.lin || nf > most * kMaxTiles) return cudaSuccess;
+  if (!coop || !G.lin || nf > most * max_tiles(P.q)) return cudaSuccess;
   const long long share = (nf + most - 1) / most;
   *grid = (int)((nf + share - 1) / share);
   return cudaSuccess;
