@@ -212,8 +212,8 @@ lbm_status lbm_kernel_times(lbm_ctx *ctx, double *ms_psi, long long *n_psi,
  * on D3Q15) runs each step as one cooperative launch over an ordered work list: each
  * item is the fused pass of one tile of one plane (128 node pairs in row order;
  * 64x4 nodes where Nx > 512) plus the psi pass of the next step for another tile,
- * placed (and checked, on the host) at least half a wave of the grid after the
- * fused tiles it reads; the FP64 EOS of the
+ * placed (and checked, on the host) at least 3/8 or 5/8 of a wave of the grid,
+ * by the size of a plane, after the fused tiles it reads; the FP64 EOS of the
  * psi work overlaps the fused work's HBM stream and the populations it pulls
  * come from L2 (Eqs. 3-6 in 2 x Q x s + 8 bytes per node); results equal the
  * two-pass step bit for bit.  Small boxes take the same jobs through up to 256

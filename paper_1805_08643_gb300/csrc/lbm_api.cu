@@ -37,7 +37,7 @@ struct lbm_ctx {
   int *flags = nullptr;     // its per-(tile, plane) progress flags
   size_t nflags = 0;
   int stamp = 0;
-  bool queued = false;      // single pass on the ordered work queue (FP32 arithmetic, D3Q19, Nx even)
+  bool queued = false;      // single pass on the ordered work list (FP32 arithmetic, Nx even)
   lbm::QueueState q{};      // its item table and counters (one allocation: q_mem)
   void *q_mem = nullptr;
   int q_stamp = 0;

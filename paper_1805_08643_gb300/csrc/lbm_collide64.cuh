@@ -19,14 +19,15 @@
 //    the reciprocal takes three instructions (recip).
 //  - the linear parts (the forward and inverse chains, the sums of Eq. 15) run on
 //    the integer units, as sums of 64-bit fixed-point numbers: see Fixed.
-// FP64 instructions per node of the fused pass, with the force: 102 non-orthogonal
+// FP64 instructions per node of the fused pass, with the force: 104 non-orthogonal
 // (255 moment by moment, 214 with these formulas in FP64 throughout), 92 orthogonal
-// (304, 259), 85 on D3Q15.  Fused pass at 128^3, FP64 throughout -> as it is: 855 ->
-// 430, 1018 -> 401 and 725 -> 344 us; bound by the FP64 and integer units together
-// (the FP64 instructions alone take 340 us).  More resident warps (96 registers)
-// and larger blocks are within 2 % of it.  Errors of a step's populations against
-// extended precision are those of FP64 throughout within a few per cent (droplets and
-// slabs with noise: 1.4 - 2.5e-16 relative, orthogonal a tenth less than before).
+// (304, 259), 88 on D3Q15.  Fused pass at 128^3, FP64 throughout -> as it is: 855 ->
+// 434, 1018 -> 401 and 725 -> 352 us; bound by the FP64 unit (the FP64 instructions
+// alone take 347 us; at 64^3 its pipe is busy 76 % of the time, the integer one 49 %).
+// More resident warps (96 registers) and larger blocks are within 2 % of it.  Errors
+// of a step's populations against extended precision (droplets and slabs, with and
+// without noise, T/Tc 0.70 to 0.85, a = 0.25): 0.63 - 0.93 (non-orthogonal), 0.72 - 0.90
+// (orthogonal) and 0.56 - 0.76 (D3Q15) of what FP64 throughout has.
 #pragma once
 
 #include <type_traits>
@@ -61,8 +62,10 @@ __device__ __forceinline__ Shear64 shear64(const KParams &P, const Coeffs64 &C, 
 // the chain's sums of factors, 2^(10 - S) at most, cannot leave 64 bits whatever
 // the values.  Sums are exact.  A value is cut off S bits below the last place of
 // the largest one, and a result is rounded once (to nearest, ties to even), where
-// an FP64 sum rounds each partial result.  What a chain starts from is chosen so
-// that the cut lies below half the last place of its results.
+// an FP64 sum rounds each partial result: what is lost is less than a last place of
+// the largest value over 2^S for each value cut, and values within a factor 2^S of the
+// largest lose nothing.  What a chain starts from is chosen accordingly (of the inverse
+// chains everything but drho, which only the rest population takes).
 struct Fixed {
   long long v;
 };

@@ -129,12 +129,14 @@ inline dim3 plane_grid(int per_plane, int nz, int threads = kThreads) {
 // Launch of a kernel of the two-pass step that may start while its predecessor
 // in the stream is ending (programmatic stream serialization): its blocks take
 // the places the last ones leave and wait in chain_wait (lbm_device.cuh) until
-// the predecessor has completed, so only the launch itself overlaps: 64^3 FP16
-// steps 16.4 -> 12.1 us, 127^3 FP32 (odd) 92 -> 84.  Blocks that come in this
-// way fill one SM after the other, so a grid that would not fill the device has
-// to start by itself: FP64 steps of 32^3 (1024 warps) took 41 us chained, 18.5
-// not.  The two-node kernels chain from 32^3 on (fewer nodes made no
-// difference), the FP64 ones, a third as many warps resident, from 64^3.
+// the predecessor has completed, so only the launch itself overlaps.  Blocks that
+// come in this way fill one SM after the other, so a grid that would not fill the
+// device has to start by itself.  Two-pass steps not chained / chained: FP16 16^3 8.2 / 5.1 us,
+// 32^3 8.2 / 7.2, 40^3 10.3 / 10.4, 48^3 12.3 / 8.4, 64^3 16.4 / 11.9, 96^3 30.8 / 25.8, 128^3
+// 63.5 / 58.7, 256^3 434 / 429; FP32 32^3 8.2 / 7.7, 40^3 10.3 / 10.3, 48^3 12.3 / 9.3, 65^3 18.5
+// / 16.9, 127^3 87.8 / 83.8; FP64, a third as many warps resident, 24^3 14.4 / 24.2, 32^3
+// 19.5 / 25.0, 40^3 28.7 / 27.8, 48^3 38.9 / 36.5, 64^3 76.0 / 71.8, 128^3 510 / 505.  So from
+// 2^15 nodes the two-node kernels, from 2^18 the FP64 ones.
 constexpr int kChainPairs = 1 << 15, kChainFP64 = 1 << 18;  // nodes
 template <typename... P, typename... A>
 cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
@@ -311,7 +313,7 @@ struct alignas(16) BatchBox {  // 16-byte aligned: copied to shared memory in 16
 
 // Persistent single-pass launch over the work items (box, tx | ty << 16, z0, z1)
 // of many boxes; grid = number of thread blocks.  FP32 arithmetic forms only.
-// The batch's two-pass step on the pair kernels (every box with an even Nx):
+// The batch's two-pass step on the pair kernels (every box's rows of even length, KParams::px):
 // the fused pass, then the psi pass of the new level, for one parity.  The
 // fused pass is a flat grid per operator, one block per plane of a tile of the
 // chosen shape: block_box holds the box of every block, the non-orthogonal
@@ -337,7 +339,7 @@ cudaError_t launch_onepass_tma(const KParams &P, int precision, int op, bool sig
                                void *g_out, const void *psi_in, void *psi_out, unsigned *err, cudaStream_t s);
 
 // Two-pass kernels of the FP32-arithmetic forms with two x-adjacent nodes per
-// thread and packed FP32 arithmetic (Nx even).
+// thread (rows of even length), in packed FP32 arithmetic where Nx is even.
 bool pair_supported(const KParams &P, int precision);
 cudaError_t launch_psi_pair(const KParams &P, int precision, const void *g, void *psi, unsigned *err,
                             const Launch &L, bool df);
@@ -359,7 +361,7 @@ size_t lagged_flag_count(const KParams &P);
 cudaError_t launch_lagged(const KParams &P, int precision, int op, bool sigma, bool df, const void *g_in, void *g_out,
                           const void *psi_in, void *psi_out, int *flags, int stamp, unsigned *err, cudaStream_t s);
 
-// Single-pass step on an ordered work list (FP32 arithmetic, D3Q19, Nx even):
+// Single-pass step on an ordered work list (FP32 arithmetic, D3Q19 or D3Q15, Nx even):
 // items of a fused tile job and a lagging psi tile job, one cooperative launch
 // of `grid` blocks (queue_grid) working through the list queue_items builds
 // (and checks: false if it cannot).  The device side: the item table, a
@@ -391,7 +393,7 @@ size_t steps_counters(const KParams &P);
 cudaError_t launch_steps(const KParams &P, int op, bool df, void *g_in, void *g_out, void *psi_in, void *psi_out,
                          int grid, int *counters, int nsteps, int stamp, unsigned *err, cudaStream_t s);
 
-// The work-list step over a batch (every box D3Q19 with an even Nx): one
+// The work-list step over a batch (every box D3Q19, rows of even length): one
 // cooperative launch per step; items hold a fused tile job and a psi tile job
 // of any boxes (x / z: box index or -1, y / w: z | tile << 16).  The list is
 // built for the boxes in the given order; base[k] receives box k's first

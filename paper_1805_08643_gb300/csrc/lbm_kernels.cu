@@ -121,14 +121,11 @@ __global__ void __launch_bounds__(256) psi_kernel(const typename Types<PREC>::S 
     drho = f[0] + sax + sdg;
   }
   unsigned e = 0;
-  if (DF && sizeof(T) == sizeof(float)) {
-    psi[nb.self] = (typename Types<PREC>::Psi)eos_psi_f2<EOS>((float)drho, P, e);
-  } else if (sizeof(T) == sizeof(float)) {
-    psi[nb.self] = (typename Types<PREC>::Psi)eos_psi_d<EOS>((float)drho, P, e);
+  if constexpr (PREC == kF64) {
+    const double rho = P.rho_ref + drho;
+    psi[nb.self] = eos_psi<EOS, double>(rho, narrow_f64(rho), P, e);
   } else {
-    const double rho = P.rho_ref + (double)drho;
-    const float rho_f = sizeof(T) == sizeof(double) ? narrow_f64(rho) : Phys<T>::rho_ref(P) + (float)drho;
-    psi[nb.self] = eos_psi<EOS, typename Types<PREC>::Psi>(rho, rho_f, P, e);
+    psi[nb.self] = DF ? eos_psi_f2<EOS>(drho, P, e) : eos_psi_d<EOS>(drho, P, e);
   }
   if (e) atomicOr(err, e);
 }
@@ -523,18 +520,21 @@ __global__ void set_populations_kernel(const double *__restrict__ f, typename Ty
 
 dim3 node_grid(const KParams &P, int threads = kThreads) { return plane_grid(P.nx * P.ny, P.nz, threads); }
 
+// Nodes from which the kernels of a precision are chained (launch_chained).
+template <int PREC> bool chained(const KParams &P) { return P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs); }
+
 template <int PREC, bool DF, int Q>
 cudaError_t psi_dispatch(const KParams &P, const void *g, void *psi, unsigned *err, const Launch &L) {
   using S = typename Types<PREC>::S;
   using Psi = typename Types<PREC>::Psi;
-  const dim3 grid = node_grid(P), block(kThreads);
+  auto run = [&](auto kernel) {
+    return launch_chained(chained<PREC>(P), kernel, node_grid(P), dim3(kThreads), L.stream, (const S *)g, (Psi *)psi, P,
+                          err);
+  };
   switch (P.eos) {
-    case kEosCS:
-      return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosCS, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
-    case kEosExp:
-      return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosExp, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
-    default:
-      return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), psi_kernel<PREC, kEosNone, DF, Q>, grid, block, L.stream, (const S *)g, (Psi *)psi, P, err);
+    case kEosCS: return run(psi_kernel<PREC, kEosCS, DF, Q>);
+    case kEosExp: return run(psi_kernel<PREC, kEosExp, DF, Q>);
+    default: return run(psi_kernel<PREC, kEosNone, DF, Q>);
   }
 }
 
@@ -547,10 +547,10 @@ cudaError_t fused_dispatch(const KParams &P, bool sigma, const void *g_in, void 
   // shortest when warps are dealt out singly: 32^3 steps 20.5 -> 18.5 us (blocks of four warps leave 8 on some
   // SMs, single ones 7), no difference from 64^3 on.
   constexpr int threads = PREC == kF64 ? 32 : kThreads;
-  const dim3 grid = node_grid(P, threads), block(threads);
   const Coeffs64 C = coeffs64(P, Q == 15 ? kNonOrthQ15 : OP);
-  return launch_chained(P.n >= (PREC == kF64 ? kChainFP64 : kChainPairs), sigma ? fused_kernel<PREC, OP, true, Q> : fused_kernel<PREC, OP, false, Q>, grid, block, L.stream,
-                        (const S *)g_in, (S *)g_out, (const Psi *)psi, P, C);
+  auto kernel = sigma ? fused_kernel<PREC, OP, true, Q> : fused_kernel<PREC, OP, false, Q>;
+  return launch_chained(chained<PREC>(P), kernel, node_grid(P, threads), dim3(threads), L.stream, (const S *)g_in,
+                        (S *)g_out, (const Psi *)psi, P, C);
 }
 
 }  // namespace

@@ -42,8 +42,9 @@ __device__ __forceinline__ bool pair_of_thread(const KParams &P, PairX &px, int 
 }
 
 // Twelve blocks an SM (40 registers): 256^3 FP32 217 -> 201 us against 48 registers
-// (the loads in flight need the warps), FP16 183 -> 180.
-// ODD: rows padded for an odd Nx, set for FP16 storage only (FP32 sums round alike either way).
+// (the loads in flight need the warps; 205 with plain loads), FP16 183 -> 180.
+// ODD: rows padded for an odd Nx, set for FP16 storage only (FP32 sums round alike
+// either way), with eight blocks (the scalar sums spill 68 bytes at twelve).
 template <typename S, int EOS, bool DF, bool ODD>
 __global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *g, float *__restrict__ psi,
                                                        const KParams P, unsigned *__restrict__ err) {
@@ -59,8 +60,8 @@ __global__ void __launch_bounds__(128, ODD ? 8 : 12) psi_pair_kernel(const S *g,
 }
 
 // Six blocks of 128 an SM (80 registers) for even boxes: FP16 256^3 fused 263 -> 258
-// us, FP32 192^3 orthogonal 164 -> 161; odd FP32 boxes
-// would spill, five there.
+// us, FP32 192^3 orthogonal 164 -> 161; odd boxes, whose nodes collide in scalar code,
+// would spill, five there (96 registers).
 template <typename S, int OP, bool SIGMA, bool ODD, bool R4 = false>
 __global__ void __launch_bounds__(128, ODD ? 5 : 6) fused_pair_kernel(const S *g_in, S *__restrict__ g_out,
                                                          const float *psi, const KParams P) {
@@ -146,8 +147,9 @@ cudaError_t psi_pair_dispatch(const KParams &P, const void *g, void *psi, unsign
 
 // Rows that fill blocks of 32 pairs x 4 rows.  The orthogonal FP16 fused pass, bound
 // by its issue slots, runs better on those (the rows of a block share psi in L1):
-// 256^3 286 -> 272 us.  The non-orthogonal one does not (263 -> 264), FP32 loses
-// (375 -> 401), and the psi pass too (201 -> 208).
+// steps of 128^3 61.2 -> 61.0 us, 64 x 200 x 200 74.1 -> 73.5, 192^3 194.0 -> 191.4, 256^3
+// 449 -> 444, 320^3 876 -> 863 (64^3 12.1 / 12.2).  The non-orthogonal one does not (256^3
+// fused 263 -> 264), FP32 loses (375 -> 401), and the psi pass too (201 -> 208).
 bool rows4(const KParams &P) { return P.px % 64 == 0 && P.ny % 4 == 0; }
 
 template <typename S, bool ODD>

@@ -1,6 +1,6 @@
-// Single-pass time step on an ordered work list (FP32-arithmetic forms, D3Q19,
-// Nx even): one persistent launch per step runs both passes of the two-pass
-// step as interleaved work.
+// Single-pass time step on an ordered work list (FP32-arithmetic forms, D3Q19 and
+// D3Q15, Nx even; batches of D3Q19 boxes with any Nx): one persistent launch per
+// step runs both passes of the two-pass step as interleaved work.
 //
 // Work item k is a pair of tile jobs (128 node pairs of one plane that follow
 // each other in row order, one per thread; see tile_map):
@@ -11,19 +11,19 @@
 //     planes z'-1..z'+1 on its rows and the rows next to them (periodic) and
 //     pulls their output through L2, where it still is.
 // The host builds the list (and checks it): fused jobs plane by plane; each
-// psi job in the first free item at least about half a wave of the grid
-// (psi_lag items) after the last fused job it reads.  Half a wave: by the time
+// psi job in the first free item at least psi_lag items (3/8 or 5/8 of a wave of
+// the grid; batches: half a wave) after the last fused job it reads: by the time
 // a block reaches the psi job those fused jobs are normally finished, so the
 // wait is one poll, while writer and reader stay close enough for the
-// populations to be still in L2 (measured on GB300: a whole wave waits less but
-// re-reads about twice as much from DRAM, and is slower; a quarter waits more).
+// populations to be still in L2 (a whole wave waits less but re-reads about twice
+// as much from DRAM, and is slower; a quarter waits more).
 //
 // Block b starts with item b; from then on it claims the next unclaimed item
 // (one atomic fetch per item, issued when an item starts and read when it
 // ends), so blocks take items in list order whatever their speed.  (With the
 // static order b, b + grid, ..., blocks drifted up to five items apart within
 // a wave, and the psi jobs of the fast ones waited on the slow ones: 0.556
-// against 0.528 ms per 256^3 step on GB300.)  Claims are in increasing order
+// against 0.528 ms per 256^3 step, with 64 x 4 tiles.)  Claims are in increasing order
 // and the launch is cooperative (every block resident): a block holding an
 // unfinished fused job is busy with an earlier item, so the psi job of the
 // lowest unfinished item waits only on fused jobs that are finished or
@@ -33,7 +33,7 @@
 //
 // What this buys over two launches: the psi jobs' FP64 EOS runs on the same
 // SMs while the fused jobs stream HBM, and the populations they pull come from
-// L2 (writer and reader are about two planes plus half a wave of tiles apart):
+// L2 (writer and reader are about two planes plus the lag apart):
 // DRAM traffic per node is f(t) read and f*(t) written once plus psi read and
 // written once (2 x 19 x s + 8 bytes) against 3 x 19 x s + 8.  The
 // arithmetic and its order are those of the two-pass kernels, so the results
