@@ -75,10 +75,10 @@ HEADLINE = ("nonorth", "f32")
 FUSED_DRAM_BYTES = {("nonorth", "f32"): 152.6, ("nonorth", "f16"): 77.3}
 # DRAM bytes per node of one launch of the work-list single pass at 256^3 (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch over the nodes), from a capture of the current kernel only
-QUEUE_DRAM_BYTES = {("nonorth", "f32"): 175.4}
+QUEUE_DRAM_BYTES = {("nonorth", "f32"): 162.3}
 # FP64 instructions per node of the fused pass (ncu instruction counts at 64^3 over the nodes) and the FP64
 # issue peak of one GB300: 2 per SM per clock x 152 SMs x 2070 MHz.
-FUSED_FP64_INSTR = {"nonorth": 102.0, "orth": 92.0, "nonorth_d3q15": 85.0}
+FUSED_FP64_INSTR = {"nonorth": 104.0, "orth": 92.0, "nonorth_d3q15": 88.0}
 FP64_PEAK_GINSTR = 2 * 152 * 2070e6 / 1e9
 PREC_TEXT = {"f64": "FP64 compute and storage", "f32": "FP32 compute and storage",
              "f16": "FP32 compute, FP16 storage"}
