@@ -84,7 +84,7 @@ template <int Q, typename S, typename T>
 __device__ __forceinline__ void store_node(S *__restrict__ g, int a, const KParams &P, const Nbhd &nb, T v) {
   S *at = g + (size_t)a * P.np + nb.self;
   Lat<Q>::store(at, a, v);
-  if (P.px != P.nx && nb.x == 0) Lat<Q>::store(at + P.nx, a, v);
+  if (sizeof(S) < sizeof(double) && P.px != P.nx && nb.x == 0) Lat<Q>::store(at + P.nx, a, v);
 }
 
 __device__ __forceinline__ bool node_of_thread(const KParams &P, int &x, int &y, int &z) {
@@ -478,7 +478,7 @@ __global__ void state_from_rho_kernel(const double *__restrict__ rho, typename T
   using S = typename Types<PREC>::S;
   int x, y, z;
   if (!node_of_thread(P, x, y, z)) return;
-  const Nbhd nb(x, y, z, P), pub(x, y, z, P, P.nx);
+  const Nbhd nb(x, y, z, P), pub(x, y, z, P, PREC == kF64 ? P.px : P.nx);
 #pragma unroll
   for (int a = 0; a < Q; ++a) {
     const double v = Lat<Q>::w(a) * (rho[Lat<Q>::dst(pub, a)] - P.rho_ref);
@@ -494,7 +494,7 @@ __global__ void get_populations_kernel(const typename Types<PREC>::S *__restrict
   int x, y, z;
   if (!node_of_thread(P, x, y, z)) return;
   const Nbhd nb(x, y, z, P);
-  const int i = x + P.nx * (y + P.ny * z);
+  const int i = PREC == kF64 ? nb.self : x + P.nx * (y + P.ny * z);
 #pragma unroll
   for (int a = 0; a < Q; ++a)
     if (a >= a_lo && a < a_hi)
@@ -509,7 +509,7 @@ __global__ void set_populations_kernel(const double *__restrict__ f, typename Ty
   using S = typename Types<PREC>::S;
   int x, y, z;
   if (!node_of_thread(P, x, y, z)) return;
-  const Nbhd nb(x, y, z, P), pub(x, y, z, P, P.nx);
+  const Nbhd nb(x, y, z, P), pub(x, y, z, P, PREC == kF64 ? P.px : P.nx);
 #pragma unroll
   for (int a = 0; a < Q; ++a)
     if (a >= a_lo && a < a_hi) {
